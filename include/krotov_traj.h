@@ -130,7 +130,7 @@ typedef struct {
                                (Eq. cross_traj_update), co-states xi_k(T) = |tgt> and
                                Delta eps_c = S_c / (M^2 lambda_c) sum_{k,k'}
                                Im[<xi_k|h_c|psi_k'><psi_k'|xi_k>] (all pairs of trajectories) */
-  int jump_scheme;          /* 0: jump times located by bisection of the norm, several jumps per
+  int jump_scheme;          /* 0: jump times located as the root of the norm, several jumps per
                                interval possible (Sec. 2.1); 1: the first-order scheme of Sec. 2.1,
                                at most one jump per interval, applied at its end (s* = dt) */
   int ckpt_prefix;          /* with ckpt_interval = K > 0: the co-states of t_0 .. t_ckpt_prefix
@@ -152,9 +152,13 @@ typedef struct {
                                lets the copy land, the block leaves) and the sweep returns
                                KT_ERR_TIMEOUT; the device stays usable.  Each wait is bounded
                                (about 2 s) whatever this flag. */
-  int items_per_thread;     /* thread mapping of the interval kernels.  0 = automatic: for the node
+  int items_per_thread;     /* thread mapping of the interval kernels.  0 = automatic: small problems whose
+                               couplings are real or imaginary (at most three nodes, d <= 256; two nodes, d up to
+                               the block size) one element per thread with its generator row in registers, when the
+                               tile width is automatic too; else for the node
                                dimensions 6 and 9 one thread per last-node fiber (the cavity-structure
-                               kernels when the generator has that structure) -- unless a trajectory has
+                               kernels when the generator has that structure, a block of fibers for four nodes
+                               in FP32-mixed) -- unless a trajectory has
                                fewer than 16 fibers and the tile width is automatic too, then the strided
                                mapping with one item per thread -- else the strided mapping with the
                                fewest items per thread that fit; with tile_traj = -1 the autotuner also
@@ -162,11 +166,11 @@ typedef struct {
                                1, 2, 4, 8 or 16: the strided mapping (item q of thread t is element
                                t + q * threads of the tile) with that many items per thread -- more
                                threads per trajectory for problems too small to fill the GPU otherwise */
-  int per_interval_launches; /* 0 = automatic: when the problem runs on the strided mapping, every tile
+  int per_interval_launches; /* 0 = automatic: when the problem runs on the strided mapping or one element per thread, every tile
                                is resident on the GPU at once and every co-state is kept (small
                                problems), each sweep is one
                                launch -- the backward sweep a plain one, the forward sweep a cooperative
-                               one whose CTAs meet at a grid barrier after each interval to form the
+                               one whose CTAs exchange their partial sums after each interval to form the
                                update (Sec. 2.2: the update of interval j+1 needs every trajectory's
                                state at t_j); bit-identical to the per-interval launches.  Not used for
                                shards, the cross-trajectory rule, the sweeps that keep states for the
@@ -330,8 +334,9 @@ typedef struct {
                                co-states of t_0 .. t_{ckpt_kept_prefix} kept, then every K-th */
   int ckpt_kept_prefix;
   int costate_slots;        /* co-state slots held in device memory */
-  int items_per_thread;     /* thread mapping of the interval kernels: 0 = one thread per last-node
-                               fiber, else the strided mapping with this many items per thread */
+  int items_per_thread;     /* thread mapping of the interval kernels: 0 = fibers or blocks of them, or one element
+                               per thread of an automatic mapping of 16 fibers and more, else the strided mapping
+                               with this many items per thread */
   int whole_sweep;          /* 1: sweeps run as one launch each (see kt_config.per_interval_launches) */
 } kt_info;
 KT_API kt_status krotov_get_info(kt_problem *p, kt_info *info);

@@ -4,22 +4,22 @@
 
 namespace kt {
 // a whole sweep (strided mapping only, the mapping of the small problems) runs one tile per CTA
-template <typename R, int EPT, int NL, int ACS>
+template <typename R, int EPT, int NL, int ACS, int MAXT>
 static cudaError_t launch_bwd_t(const KtGeom &g, const KtGenImage &im, const KtOps &ops, const BwdArgs &a, size_t smem,
                                 cudaStream_t st) {
   if (a.sweep) {
-    if constexpr (NL == 0 && ACS == 0) {
-      const cudaError_t attr = kt_allow_large_smem((const void *)bwd_kernel<R, EPT, 0, 0, true>);
+    if constexpr (NL == 0) {
+      const cudaError_t attr = kt_allow_large_smem((const void *)bwd_kernel<R, EPT, 0, ACS, true, MAXT>);
       if (attr != cudaSuccess) return attr;
-      bwd_kernel<R, EPT, 0, 0, true><<<g.n_tiles, g.nthreads, smem, st>>>(g, im, ops, a);
+      bwd_kernel<R, EPT, 0, ACS, true, MAXT><<<g.n_tiles, g.nthreads, smem, st>>>(g, im, ops, a);
       return cudaGetLastError();
     } else {
       return cudaErrorInvalidValue;
     }
   }
-  const cudaError_t attr = kt_allow_large_smem((const void *)bwd_kernel<R, EPT, NL, ACS, false>);
+  const cudaError_t attr = kt_allow_large_smem((const void *)bwd_kernel<R, EPT, NL, ACS, false, MAXT>);
   if (attr != cudaSuccess) return attr;
-  bwd_kernel<R, EPT, NL, ACS, false><<<g.bwd_grid > 0 ? g.bwd_grid : g.n_tiles, g.nthreads, smem, st>>>(g, im, ops, a);
+  bwd_kernel<R, EPT, NL, ACS, false, MAXT><<<g.bwd_grid > 0 ? g.bwd_grid : g.n_tiles, g.nthreads, smem, st>>>(g, im, ops, a);
   return cudaGetLastError();
 }
 }  // namespace kt
@@ -27,19 +27,31 @@ static cudaError_t launch_bwd_t(const KtGeom &g, const KtGenImage &im, const KtO
 cudaError_t kt_launch_bwd_f64(int ept, const KtGeom &g, const KtGenImage &im, const KtOps &ops, const BwdArgs &a,
                              size_t smem, cudaStream_t st) {
   switch (ept) {
-    case 1: return kt::launch_bwd_t<double, 1, 0, 0>(g, im, ops, a, smem, st);   // strided, small problems
-    case 2: return kt::launch_bwd_t<double, 2, 0, 0>(g, im, ops, a, smem, st);
-    case 4: return kt::launch_bwd_t<double, 4, 0, 0>(g, im, ops, a, smem, st);
-    case 8: return kt::launch_bwd_t<double, 8, 0, 0>(g, im, ops, a, smem, st);
-    case 16: return kt::launch_bwd_t<double, 16, 0, 0>(g, im, ops, a, smem, st);
-    case -6: return kt::launch_bwd_t<double, 6, 6, 0>(g, im, ops, a, smem, st);   // fiber mapping, n_loc = 6
-    case -9: return kt::launch_bwd_t<double, 9, 9, 0>(g, im, ops, a, smem, st);   // fiber mapping, n_loc = 9
-    case -106: return kt::launch_bwd_t<double, 6, 6, 1>(g, im, ops, a, smem, st);  // cavity structure, cutoff 1
-    case -109: return kt::launch_bwd_t<double, 9, 9, 1>(g, im, ops, a, smem, st);  // cavity structure, cutoff 2
-    case -209: return kt::launch_bwd_t<double, 9, 9, 2>(g, im, ops, a, smem, st);  // cavity structure, cutoff 2, T = 1
-    case -306: return kt::launch_bwd_t<double, 6, 6, 3>(g, im, ops, a, smem, st);  // real / imaginary couplings, cutoff 1
-    case -309: return kt::launch_bwd_t<double, 9, 9, 3>(g, im, ops, a, smem, st);  // real / imaginary couplings, cutoff 2
-    case -409: return kt::launch_bwd_t<double, 9, 9, 4>(g, im, ops, a, smem, st);  // the same with T = 1
+    case 1: return kt::launch_bwd_t<double, 1, 0, 0, 512>(g, im, ops, a, smem, st);   // strided, small problems
+    case 2: return kt::launch_bwd_t<double, 2, 0, 0, 512>(g, im, ops, a, smem, st);
+    case 4: return kt::launch_bwd_t<double, 4, 0, 0, 512>(g, im, ops, a, smem, st);
+    case 8: return kt::launch_bwd_t<double, 8, 0, 0, 512>(g, im, ops, a, smem, st);
+    case 16: return kt::launch_bwd_t<double, 16, 0, 0, 512>(g, im, ops, a, smem, st);
+    case 21:   // row mapping, up to two nodes and one pair
+      return g.nthreads <= 256 ? kt::launch_bwd_t<double, 1, 0, 6, 256>(g, im, ops, a, smem, st)
+                               : kt::launch_bwd_t<double, 1, 0, 6, 1024>(g, im, ops, a, smem, st);
+    case 33:   // row mapping, up to three nodes and three pairs
+      return g.nthreads <= 256 ? kt::launch_bwd_t<double, 1, 0, 7, 256>(g, im, ops, a, smem, st)
+                               : kt::launch_bwd_t<double, 1, 0, 7, 768>(g, im, ops, a, smem, st);
+    case -6: return kt::launch_bwd_t<double, 6, 6, 0, 736>(g, im, ops, a, smem, st);   // fiber mapping, n_loc = 6
+    case -9: return kt::launch_bwd_t<double, 9, 9, 0, 736>(g, im, ops, a, smem, st);   // fiber mapping, n_loc = 9
+    case -106: return kt::launch_bwd_t<double, 6, 6, 1, 736>(g, im, ops, a, smem, st);  // cavity structure, cutoff 1
+    case -109: return kt::launch_bwd_t<double, 9, 9, 1, 736>(g, im, ops, a, smem, st);  // cavity structure, cutoff 2
+    case -209: return kt::launch_bwd_t<double, 9, 9, 2, 736>(g, im, ops, a, smem, st);  // cavity structure, cutoff 2, T = 1
+    case -306:  // real / imaginary couplings, cutoff 1
+      return g.nthreads <= 256 ? kt::launch_bwd_t<double, 6, 6, 3, 256>(g, im, ops, a, smem, st)
+                               : kt::launch_bwd_t<double, 6, 6, 3, 736>(g, im, ops, a, smem, st);
+    case -309:  // real / imaginary couplings, cutoff 2
+      return g.nthreads <= 256 ? kt::launch_bwd_t<double, 9, 9, 3, 256>(g, im, ops, a, smem, st)
+                               : kt::launch_bwd_t<double, 9, 9, 3, 736>(g, im, ops, a, smem, st);
+    case -409:  // the same with T = 1
+      return g.nthreads <= 256 ? kt::launch_bwd_t<double, 9, 9, 4, 256>(g, im, ops, a, smem, st)
+                               : kt::launch_bwd_t<double, 9, 9, 4, 736>(g, im, ops, a, smem, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -59,6 +59,7 @@ KT_HD int kt_bessel_miller(double alpha, int n, double *out) {
   for (int k = 0; k < n; ++k) out[k] = 0.0;
   double jp1 = 0.0, jk = 1e-200, norm = 0.0;
   const double inv = 2.0 / alpha;
+  const bool small = alpha < 1.0 || start > 140;   // else J_start / J_0 > 1e-290 and nothing overflows
   for (int k = start; k >= 1; --k) {
     double jm1 = (double)k * inv * jk - jp1;
     jp1 = jk;
@@ -66,7 +67,7 @@ KT_HD int kt_bessel_miller(double alpha, int n, double *out) {
     int km1 = k - 1;
     if (km1 < n) out[km1] = jk;
     if (km1 > 0 && (km1 & 1) == 0) norm += 2.0 * jk;
-    if (jk > 1e150 || jk < -1e150) {
+    if (small && (jk > 1e150 || jk < -1e150)) {
       jk *= 1e-150; jp1 *= 1e-150; norm *= 1e-150;
       for (int q = km1; q < n; ++q) out[q] *= 1e-150;
     }
@@ -90,7 +91,7 @@ struct KtGeom {
   int prefetch_chi;                  // forward kernel keeps a third tile buffer for chi(t_j)
   int bwd_grid;                      // > 0: backward kernel CTAs looping over tiles, next input prefetched
   int fwd_grid;                      // > 0: the same for the forward kernel (psi and chi of the next tile prefetched)
-  int first_order;                   // jump scheme: 0 jump times by bisection, 1 at most one jump per interval, at its end
+  int first_order;                   // jump scheme: 0 jump times located in the interval, 1 at most one jump per interval, at its end
   int stride[KT_MAX_NODES];          // element stride of node i (n_loc^(N-1-i))
   int ctrl_node[KT_MAX_CTRL];        // node of control c (its ket node for a density matrix)
   int n_cterms;                      // control terms: control cterm_ctrl[t] acting on node cterm_node[t]
@@ -104,29 +105,52 @@ struct KtGeom {
   double c_fwd, c_bwd, r;            // generator centre (per direction) and half width
 };
 
-// Precomputed (pulse independent) generator tables of one direction, FP64, in global memory.
+// Precomputed (pulse independent) tables of one direction, FP64, in global memory: the generator G as
+// B = -2i (G - c) / r, so that the series of exp(-i G s) is a real sum of y_k = (-i)^k T_k((G - c) / r) v with
+// y_{k+1} = y_{k-1} + B y_k (see kt_device.cuh).
 struct KtGenImage {
   const int *loc_dl;          // [N][n_loc][S] local column delta y - x (0 = no entry)
-  const KtCplx *loc_base;     // [N][n_loc][S] scaled (1/r) drift part
-  const KtCplx *ctrl_slot;    // [n_cterms][n_loc][S] scaled per-unit-eps part of term t on node cterm_node[t]
-  const KtCplx *diag_base;    // [N][n_loc] scaled diagonal (node 0 also holds -c/r)
-  const KtCplx *ctrl_diag;    // [n_cterms][n_loc] scaled per-unit-eps diagonal part
+  const KtCplx *loc_base;     // [N][n_loc][S] drift part of B
+  const KtCplx *ctrl_slot;    // [n_cterms][n_loc][S] per-unit-eps part of term t on node cterm_node[t]
+  const KtCplx *diag_base;    // [N][n_loc] diagonal of B (node 0 also holds the shift by c)
+  const KtCplx *ctrl_diag;    // [n_cterms][n_loc] per-unit-eps diagonal part
   const int *pair_off;        // [P][n_loc*n_loc] element offset (in elements, before *T); 0 = none
-  const KtCplx *pair_val;     // [P][n_loc*n_loc] scaled
-  const KtCplx *cheb_full;    // [K] full-step coefficients, phase exp(-i c dt) folded in
-  const KtCplx *pair_coef;    // [P] scaled coefficient of pair term p (value = coef * a^dag a entries)
+  const KtCplx *pair_val;     // [P][n_loc*n_loc]
+  const double *cheb_full;    // [sets][K] full-step coefficients lambda_s (2 - delta_k0) J_k(r dt)
+  const KtCplx *phase_full;   // [sets] exp(-i c dt) / lambda_s
+  int sets;                   // interval j takes set j % sets (a power of two)
+  const KtCplx *pair_coef;    // [P] coefficient of pair term p (value = coef * a^dag a entries)
   int pair_dst[KT_MAX_PAIRS]; // node raised by pair term p of this direction
   int pair_src[KT_MAX_PAIRS]; // node lowered by pair term p of this direction
   // Cavity-structure kernels with real / imaginary coupling classes: the pulse-independent
   // coefficients that every Chebyshev term reads, as kernel-parameter constants in both precisions
   // (the kernels then take them as constant-bank operands instead of shared-memory loads).
-  float kd32[2 * KT_MAX_NL];  // last node's diagonal, (re, im) per local index
-  double kd64[2 * KT_MAX_NL];
-  float kc32[2 * 2];          // last node's cavity couplings: [n-1] row (r, n-1) <- (g, n), [NC + n-1] the reverse
+  float kd32[3 * KT_MAX_NL];  // last node's diagonal per local index: real part, imaginary part in two floats (kt_split)
+  double kd64[2 * KT_MAX_NL]; // the same, (re, im)
+  float kc32[2 * 2];          // last node's cavity couplings (imaginary): [n-1] row (r, n-1) <- (g, n), [NC + n-1] the reverse
   double kc64[2 * 2];
-  float kp32[KT_MAX_PAIRS];   // imaginary part of pair coefficient p
+  float kp32[KT_MAX_PAIRS];   // pair coefficient p (real)
   double kp64[KT_MAX_PAIRS];
+  // Block mapping: the pair coefficients by the kinds of their nodes.  Of the outer node i: kh[0][i] and kh[1][i]
+  // of the hop that raises the middle / last node and lowers i, kh[2][i] and kh[3][i] of the reverse ones; of
+  // the middle and the last node: kh[4][0] raising the last, kh[4][1] raising the middle one.
+  float kh[5][2];
 };
+
+// FP32 coefficient sets.  A state that barely changes from one interval to the next meets the same roundings
+// of the same coefficients each time, and they add up (4e-8 per interval in the norm at d = 81); scaling the
+// coefficients by a different lambda_s from interval to interval, undone in the two-float phase, makes
+// them random: 1e-5 -> 2e-6 over 100 intervals at d = 81.
+#define KT_COEF_SETS 32
+
+// A diagonal value as a float on a 2^-21 grid and the float of what is left.  The dominant part of the
+// diagonal's phase otherwise turns by its own rounding, 6e-8 r dt per interval and always the same way;
+// the parts of different nodes add without rounding on the grid.
+KT_HD void kt_split(double v, float *hi, float *lo) {
+  const double h = (double)(long long)(v * 2097152.0 + (v < 0.0 ? -0.5 : 0.5)) * (1.0 / 2097152.0);
+  *hi = (float)h;
+  *lo = (float)(v - (double)*hi);
+}
 
 // Pulse-independent operators shared by both directions.
 struct KtOps {

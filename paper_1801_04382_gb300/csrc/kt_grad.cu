@@ -10,9 +10,10 @@
 // state at the start of piece q and W_q the co-state at its end.  dP(tau)/deps_i is evaluated
 // exactly with the Chebyshev series of the block-triangular generator [[G, H_i], [0, G]] applied
 // to [0; Z]: T_k of that block matrix carries dT_k(Ghat)/deps in its upper-right block, so the
-// recurrences z_{k+1} = 2 Ghat z_k - z_{k-1} and y_{k+1} = 2 (Ghat y_k + Hhat_i z_k) - y_{k-1}
-// (y_0 = 0, y_1 = Hhat_i z_0) give dP/deps_i Z = sum_k a_k y_k with the propagator's own
-// coefficients a_k (the same constants c, r: only Ghat depends on eps).
+// recurrences z_{k+1} = z_{k-1} + B z_k and y_{k+1} = y_{k-1} + B y_k + B_i z_k (B = -2i (G - c) / r as in
+// kt_device.cuh, B_i = -2i H_i / r its derivative; z_1 = B z_0 / 2, y_0 = 0, y_1 = B_i z_0 / 2) give
+// dP/deps_i Z = exp(-i c tau) sum_k m_k y_k with the propagator's own coefficients (the same constants c, r:
+// only B depends on eps).
 //
 // One CTA per trajectory, gathered from the problem's interleaved tile layout.
 #include "kt_device.cuh"
@@ -37,7 +38,7 @@ __device__ __forceinline__ void gather_traj(const IT &it, const typename C2<R>::
     if (it.ok(q)) dst[it.item(q)] = src[(size_t)it.item(q) * T_layout];
 }
 
-// (H_c / r) v at one item (control factor c, scaled like the generator)
+// B_c v = -2i H_c / r v at one item
 template <typename R>
 __device__ __forceinline__ typename C2<R>::T hc_item(const KtGeom &g, const Smem &sm, int c,
                                                      const typename C2<R>::T *v, int item, uint32_t dig, R invr) {
@@ -50,63 +51,62 @@ __device__ __forceinline__ typename C2<R>::T hc_item(const KtGeom &g, const Smem
     const C w = hv[base + e];
     if (w.x != (R)0 || w.y != (R)0) h = cfma(w, v[item + sm.hc_off[base + e]], h);
   }
-  return mkc(h.x * invr, h.y * invr);
+  return mkc((R)2 * h.y * invr, (R)-2 * h.x * invr);
 }
 
-// acc = sum_k a_k y_k, the derivative along control c of sum_k a_k T_k(Ghat) z0 (z0 in A, synced).
+// acc = exp(-i c s) sum_k m_k y_k, the derivative along control c of the propagator's series on z0 (z0 in A, synced).
 // Uses A, B (z recurrence) and C, D (y recurrence).  Ends synchronised.
 template <typename R, int EPT, class IT>
 __device__ void aug_run(const KtGeom &g, const KtGenImage &im, const Smem &sm, const IT &it, int K, int c,
                         typename C2<R>::T *Dbuf, typename C2<R>::T (&acc)[EPT]) {
   typedef typename C2<R>::T C;
   C *A = (C *)sm.bufA, *B = (C *)sm.bufB, *Cb = (C *)sm.bufC, *D = Dbuf;
-  const C *cf = (const C *)sm.coef;
+  const R *cf = (const R *)sm.coef;
   const R invr = (R)(1.0 / g.r);
-  C dv[EPT];
+  const C zero = mkc((R)0, (R)0);
+  Diag<R> dv[EPT];
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
-    dv[q] = it.ok(q) ? diag_of<R>(g, sm, it.dig(q)) : mkc((R)0, (R)0);
-    acc[q] = mkc((R)0, (R)0);
-    if (it.ok(q)) Cb[it.item(q)] = mkc((R)0, (R)0);   // y_0 = 0
+    acc[q] = zero;
+    if (!it.ok(q)) continue;
+    dv[q] = diag_of<R>(g, sm, it.dig(q));
+    Cb[it.item(q)] = zero;   // y_0 = 0
   }
   if (K < 2) { __syncthreads(); return; }
-  const C c1 = cf[1];
+  const R c1 = cf[1];
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
     if (!it.ok(q)) continue;
     const int i = it.item(q);
-    B[i] = apply_item<R>(g, im, sm, A, i, it.dig(q), dv[q]);       // z_1 = Ghat z_0
-    const C y1 = hc_item<R>(g, sm, c, A, i, it.dig(q), invr);       // y_1 = Hhat z_0
-    D[i] = y1;
-    acc[q] = cfma(c1, y1, acc[q]);
+    const C z1 = apply_item<R>(g, im, sm, A, i, it.dig(q), dv[q], zero);
+    const C y1 = hc_item<R>(g, sm, c, A, i, it.dig(q), invr);
+    B[i] = mkc((R)0.5 * z1.x, (R)0.5 * z1.y);
+    D[i] = mkc((R)0.5 * y1.x, (R)0.5 * y1.y);
+    acc[q] = rfma(c1, D[i], acc[q]);
   }
   __syncthreads();
   C *Pz = A, *Qz = B, *Py = Cb, *Qy = D;
   for (int k = 2; k < K; ++k) {
-    const C ak = cf[k];
+    const R ak = cf[k];
 #pragma unroll
     for (int q = 0; q < EPT; ++q) {
       if (!it.ok(q)) continue;
       const int i = it.item(q);
-      const C tz = apply_item<R>(g, im, sm, Qz, i, it.dig(q), dv[q]);
-      C ty = apply_item<R>(g, im, sm, Qy, i, it.dig(q), dv[q]);
       const C hz = hc_item<R>(g, sm, c, Qz, i, it.dig(q), invr);
-      ty.x += hz.x;
-      ty.y += hz.y;
-      const C oz = Pz[i], oy = Py[i];
-      const C nz = mkc(tz.x + tz.x - oz.x, tz.y + tz.y - oz.y);
-      const C ny = mkc(ty.x + ty.x - oy.x, ty.y + ty.y - oy.y);
-      Pz[i] = nz;
+      const C oy = Py[i];
+      const C ny = apply_item<R>(g, im, sm, Qy, i, it.dig(q), dv[q], mkc(oy.x + hz.x, oy.y + hz.y));
+      Pz[i] = apply_item<R>(g, im, sm, Qz, i, it.dig(q), dv[q], Pz[i]);
       Py[i] = ny;
-      acc[q] = cfma(ak, ny, acc[q]);
+      acc[q] = rfma(ak, ny, acc[q]);
     }
     __syncthreads();
     C *t1 = Pz; Pz = Qz; Qz = t1;
     C *t2 = Py; Py = Qy; Qy = t2;
   }
+  apply_phase<R, EPT>(g, sm, 0, acc, [&](int q) { return it.ok(q) ? dv[q].lo : (R)0; });
 }
 
-// Fiber form of (H_c / r) v for the thread's fiber (tile width 1): a control on the last node
+// Fiber form of B_c v for the thread's fiber (tile width 1): a control on the last node
 // takes row q of its factor for element q, a control on another node one row for the whole fiber.
 // Same entries and order as hc_item.
 template <typename R, int NL>
@@ -138,7 +138,7 @@ __device__ __forceinline__ void hc_fiber(const KtGeom &g, const Smem &sm, int c,
     }
   }
 #pragma unroll
-  for (int q = 0; q < NL; ++q) h[q] = mkc(h[q].x * invr, h[q].y * invr);
+  for (int q = 0; q < NL; ++q) h[q] = mkc((R)2 * h[q].y * invr, (R)-2 * h[q].x * invr);
 }
 
 // aug_run in the fiber mapping with tile width 1, for the cavity structure with real / imaginary
@@ -149,19 +149,14 @@ __device__ void aug_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &s
   typedef typename C2<R>::T C;
   constexpr int NL = 3 * (NC + 1);
   C *A = (C *)sm.bufA, *B = (C *)sm.bufB, *Cb = (C *)sm.bufC, *D = Dbuf;
-  const C *cf = (const C *)sm.coef;
-  const C *dg = (const C *)sm.diag;
+  const R *cf = (const R *)sm.coef;
   const R invr = (R)(1.0 / g.r);
   const bool ok = it.ok(0);
   const int base = it.item(0);
   const uint32_t fdig = it.dig(0);
   const int last = g.n_nodes - 1;
-  C Df = mkc((R)0, (R)0);
-  for (int i = 0; i < last; ++i) {
-    const C v = dg[i * NL + ((fdig >> (4 * i)) & 15)];
-    Df.x += v.x;
-    Df.y += v.y;
-  }
+  Diag<R> Df{(R)0, (R)0, (R)0};
+  for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
 #pragma unroll
   for (int q = 0; q < NL; ++q) {
     acc[q] = mkc((R)0, (R)0);
@@ -174,45 +169,43 @@ __device__ void aug_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &s
   if (ok) {
 #pragma unroll
     for (int q = 0; q < NL; ++q) v[q] = A[base + q];
-    apply_acs<R, NC, 1, true, true>(g, im, sm, A, base, fdig, Df, v, t, rc);      // z_1 = Ghat z_0
-    hc_fiber<R, NL>(g, sm, c, A, base, fdig, invr, h);                // y_1 = Hhat z_0
-    const C c1 = cf[1];
+    apply_acs<R, NC, 1, true, true, false>(g, im, sm, A, A, base, fdig, Df, v, t, rc);
+    hc_fiber<R, NL>(g, sm, c, A, base, fdig, invr, h);
+    const R c1 = cf[1];
 #pragma unroll
     for (int q = 0; q < NL; ++q) {
-      B[base + q] = t[q];
-      D[base + q] = h[q];
-      acc[q] = cfma(c1, h[q], acc[q]);
+      B[base + q] = mkc((R)0.5 * t[q].x, (R)0.5 * t[q].y);
+      D[base + q] = mkc((R)0.5 * h[q].x, (R)0.5 * h[q].y);
+      acc[q] = rfma(c1, mkc((R)0.5 * h[q].x, (R)0.5 * h[q].y), acc[q]);
     }
   }
   __syncthreads();
   C *Pz = A, *Qz = B, *Py = Cb, *Qy = D;
   for (int k = 2; k < K; ++k) {
     if (ok) {
-      const C ak = cf[k];
+      const R ak = cf[k];
 #pragma unroll
       for (int q = 0; q < NL; ++q) v[q] = Qz[base + q];
-      apply_acs<R, NC, 1, true, true>(g, im, sm, Qz, base, fdig, Df, v, t, rc);
+      apply_acs<R, NC, 1, true, true, true>(g, im, sm, Qz, Pz, base, fdig, Df, v, t, rc);
       hc_fiber<R, NL>(g, sm, c, Qz, base, fdig, invr, h);
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
-        const C oz = Pz[base + q];
-        Pz[base + q] = mkc(t[q].x + t[q].x - oz.x, t[q].y + t[q].y - oz.y);
+        Pz[base + q] = t[q];
         v[q] = Qy[base + q];
       }
-      apply_acs<R, NC, 1, true, true>(g, im, sm, Qy, base, fdig, Df, v, t, rc);
+      apply_acs<R, NC, 1, true, true, true>(g, im, sm, Qy, Py, base, fdig, Df, v, t, rc);
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
-        const C ty = mkc(t[q].x + h[q].x, t[q].y + h[q].y);
-        const C oy = Py[base + q];
-        const C ny = mkc(ty.x + ty.x - oy.x, ty.y + ty.y - oy.y);
+        const C ny = mkc(t[q].x + h[q].x, t[q].y + h[q].y);
         Py[base + q] = ny;
-        acc[q] = cfma(ak, ny, acc[q]);
+        acc[q] = rfma(ak, ny, acc[q]);
       }
     }
     __syncthreads();
     C *t1 = Pz; Pz = Qz; Qz = t1;
     C *t2 = Py; Py = Qy; Qy = t2;
   }
+  apply_phase<R, NL>(g, sm, 0, acc, [&](int q) { return Df.lo + acs_kd<R>(im, q).lo; });
 }
 
 // NL = 0: strided items (EPT per thread); NL = 9 with ACS = 4: fiber mapping, tile width 1,
@@ -295,7 +288,9 @@ __global__ void __launch_bounds__(NL > 0 ? 96 : (EPT == 4 ? 256 : 1024), NL > 0 
     // ---- derivative of piece q along every control: <W_q| dP(tau_q)/deps_c |Z_q>
     if (threadIdx.x == 0) {
       if (m == 0) {
-        for (int e = 0; e < g.K; ++e) ((C *)sm.coef)[e] = from_kc<C>(imf.cheb_full[e]);
+        const int set = j & (imf.sets - 1);
+        for (int e = 0; e < g.K; ++e) ((R *)sm.coef)[e] = (R)imf.cheb_full[(size_t)set * g.K + e];
+        store_phase<R>(g, sm, 0, imf.phase_full[set].re, imf.phase_full[set].im, g.dt);
       } else {
         tau_coefs<R>(g, sm, 0, g.c_fwd, sb(q + 1) - sb(q));
       }

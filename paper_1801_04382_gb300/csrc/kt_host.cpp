@@ -269,7 +269,8 @@ kt_status kt_fail(kt_status s, const char *msg) { return fail(s, "%s", msg); }
 // ---------------------------------------------------------------------------- problem object
 struct kt_problem {
   KtGeom g{};
-  int fp64 = 1, ept = 4, cross = 0, density = 0;
+  int fp64 = 1, ept = 4, cross = 0, density = 0, items_reported = 0;
+  bool cavity_ri = false;
   size_t esz = 16;
   // trajectory sharding: this problem holds trajectories [traj_offset, traj_offset + M) of M_total,
   // tiles [tile_off, tile_off + n_tiles) of n_tiles_total; the per-interval update sums the tile
@@ -305,9 +306,9 @@ struct kt_problem {
   int *cursor = nullptr;
   double *partials = nullptr;
   unsigned *counter = nullptr;
-  // whole-sweep launches (kt_config.per_interval_launches): sync = the grid barrier's two words
+  // whole-sweep launches (kt_config.per_interval_launches): wpart = the tile partials of every interval
   int whole_sweep = 0;
-  unsigned *sync = nullptr;
+  double *wpart = nullptr;
   KtCplx *tau = nullptr;
   double *norm2 = nullptr;
   int *status = nullptr;
@@ -451,7 +452,6 @@ kt_status read_status(kt_problem *p, cudaStream_t st) {
   KT_CUDA(cudaMemsetAsync(p->status, 0, sizeof(int), st));
   // a CTA that left early (a wait that ran out) took no last-CTA ticket: start the next sweep at zero
   KT_CUDA(cudaMemsetAsync(p->counter, 0, sizeof(unsigned), st));
-  if (p->sync) KT_CUDA(cudaMemsetAsync(p->sync, 0, 2 * sizeof(unsigned), st));
   KT_CUDA(cudaStreamSynchronize(st));
   switch (s) {
     case KT_DEV_NONFINITE: return fail(KT_ERR_NONFINITE, "non-finite norm, overlap or pulse value on the device");
@@ -642,8 +642,10 @@ kt_status enqueue_forward(kt_problem *p, int update, cudaStream_t st, bool save_
     a.psi_ring[1] = p->psi[1];
     a.chi_slots = p->chi;
     a.slot_bytes = p->state_bytes;
-    a.sync = p->sync;
-    KT_CUDA(cudaMemsetAsync(p->sync, 0, 2 * sizeof(unsigned), st));
+    if (a.overlap) {
+      a.partials = p->wpart;
+      KT_CUDA(cudaMemsetAsync(p->wpart, 0xff, (size_t)p->nt * p->g.n_tiles * p->g.n_ctrl * sizeof(double), st));
+    }
     kt_status s = prof_begin(p, KT_PROF_FWD, st);
     if (s != KT_OK) return s;
     KT_CUDA(kt_launch_fwd(p->fp64, p->ept, p->g, p->im_fwd, p->ops, a, st));
@@ -701,7 +703,7 @@ kt_status grad_setup(kt_problem *p, cudaStream_t st) {
   // compiled block size): one thread per last-node fiber; otherwise 4 items per thread up to 256
   // threads, else 8 up to 1024
   int ept;
-  if ((p->ept == -309 || p->ept == -409) && g1.d / 9 <= 96) {
+  if (p->cavity_ri && g1.n_loc == 9 && g1.d / 9 <= 96) {
     ept = -409;
     g1.nthreads = std::max(32, (g1.d / 9 + 31) / 32 * 32);
   } else {
@@ -993,15 +995,21 @@ namespace {
 // Everything krotov_init computes on the host, before any device call.
 struct HostImage {
   std::vector<int> dl, poff;
-  std::vector<KtCplx> base, cslot, dg, cdg, pval, cf, pc;
+  std::vector<KtCplx> base, cslot, dg, cdg, pval, pc;
+  std::vector<double> cf;
+  std::vector<KtCplx> phase;
   int pdst[KT_MAX_PAIRS], psrc[KT_MAX_PAIRS];
   double kd[2 * KT_MAX_NL] = {}, kc[4] = {}, kp[KT_MAX_PAIRS] = {};   // constants of the real / imaginary kernels
+  double kh[5][2] = {};                                              // and of the block mapping
 };
 
 struct HostPlan {
   KtGeom g{};
   int fp64 = 1, ept = 4, ckpt = 0, ckpt_dense = 0, cross = 0, density = 0;
   int sharded = 0, tile_off = 0, n_tiles_total = 0, M_total = 0;
+  bool cavity_ri = false;      // cavity structure with real / imaginary coupling classes
+  bool sweeps = false;         // mapping whose sweeps may run as one launch
+  int items_reported = 0;      // kt_info::items_per_thread
   std::vector<double> psi0;    // density: vec(rho_0) [d][2]; empty otherwise (the model's psi0 is used)
   double e_min = 0, e_max = 0, damping = 0;
   HostImage fwd, bwd;
@@ -1072,16 +1080,15 @@ bool acs_constants_ok(const Gen &gf, const Gen &gb, const std::vector<cd> &lo_va
   return true;
 }
 
-// Real / imaginary coupling classes, checked on top of the cavity structure: every off-diagonal
-// entry of every node factor (drift and controls, both directions) is purely real or purely
-// imaginary, a row has at most one entry of each class, the last node's cavity couplings are real
-// and its drive couplings imaginary, every pair coefficient is imaginary and the ladder factor is
+// Real / imaginary coupling classes: every off-diagonal entry of every node factor (drift and controls, both directions) is purely real or purely
+// imaginary, a row has at most one entry of each class, (cavity: checked on top of the cavity structure) the
+// last node's cavity couplings are real and its drive couplings imaginary, every pair coefficient is imaginary and the ladder factor is
 // real (true of the node of Sec. 3.1: g real, drive (i/2)(sigma_re - sigma_er), cascade -2i kappa).
 // Then each row's slots are re-ordered [real entry, imaginary entry] (x itself marks an empty
 // slot), and the kernels apply each coupling with two real FMAs instead of a complex one; the
 // result is bit-identical, the products with the zero part being exact zeros.
 bool ri_classes(const Gen &gf, const Gen &gb, const std::vector<cd> &lo_val, const std::vector<cd> &ra_val,
-                std::vector<std::vector<int>> &cols) {
+                std::vector<std::vector<int>> &cols, bool cavity) {
   const int N = gf.N, nl = gf.nl, NP = nl / 3;
   for (int x = 0; x < nl; ++x)
     if (lo_val[x].imag() != 0.0 || ra_val[x].imag() != 0.0) return false;
@@ -1119,11 +1126,27 @@ bool ri_classes(const Gen &gf, const Gen &gb, const std::vector<cd> &lo_val, con
           yi = y;
         }
       }
-      if (i == N - 1 && yr != x && (x / NP) * (yr / NP) != 0) return false;   // cavity: g <-> r only
-      if (i == N - 1 && yi != x && (x / NP) * (yi / NP) != 2) return false;   // drive: e <-> r only
+      if (cavity && i == N - 1 && yr != x && (x / NP) * (yr / NP) != 0) return false;   // cavity: g <-> r only
+      if (cavity && i == N - 1 && yi != x && (x / NP) * (yi / NP) != 2) return false;   // drive: e <-> r only
       out[(size_t)i * nl + x] = {yr, yi};
     }
   cols.swap(out);
+  return true;
+}
+
+// The block mapping (kt_device.cuh, apply_blk) on top of the real / imaginary classes: the middle node (the one
+// before the last) couples like the last one -- slot 0 (r, n-1) <-> (g, n), slot 1 (r, n) <-> (e, n), the drive at
+// every photon number or at none -- and one or two nodes lie outside.
+bool block_structure(int N, int nl, const std::vector<std::vector<int>> &cols) {
+  if (N < 3 || N > 4) return false;
+  const int NP = nl / 3, NC = NP - 1, m = N - 2;
+  for (int x = 0; x < nl; ++x) {
+    const int a = x / NP, n = x % NP, yr = cols[(size_t)m * nl + x][0], yi = cols[(size_t)m * nl + x][1];
+    const bool cavity = (a == 0 && n >= 1 && yr == x + 2 * NP - 1) || (a == 2 && n < NC && yr == x - 2 * NP + 1);
+    if (yr != x && !cavity) return false;
+    if (yi != x && !((a == 1 && yi == x + NP) || (a == 2 && yi == x - NP))) return false;
+    if ((yi != x) != (cols[(size_t)m * nl + x - n][1] != x - n)) return false;
+  }
   return true;
 }
 
@@ -1407,17 +1430,25 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
   if (cfg->items_per_thread != 0 && cfg->items_per_thread != 1 && cfg->items_per_thread != 2 &&
       cfg->items_per_thread != 4 && cfg->items_per_thread != 8 && cfg->items_per_thread != 16)
     return fail(KT_ERR_ARG, "items_per_thread must be 0 (automatic), 1, 2, 4, 8 or 16");
-  // automatic mapping: one thread per last-node fiber, unless a trajectory has fewer than 16 fibers
-  // (d <= 81) and the tile width is automatic too (or fixed at 1 by a density matrix's single state):
-  // then a CTA would hold a few warps at most, and the strided mapping with one item per thread runs
-  // n_loc times as many threads per trajectory (measured faster at d = 36 and 81, about 5x in FP64,
-  // where the fiber kernels' register arrays spill)
-  const bool small = (nl == 6 || nl == 9) && d / nl < 16 && (cfg->tile_traj <= 0 || density);
-  const int ipt = cfg->items_per_thread > 0 ? cfg->items_per_thread : (small ? 1 : 0);
+  // automatic mapping.  Real / imaginary coupling classes with at most three nodes, two slots per node row and
+  // three pair terms take the row mapping (one element per thread, its row in registers) while a trajectory
+  // fits a CTA; other problems of fewer than 16 fibers the strided mapping with one item per thread (the fiber
+  // mapping would leave a CTA a few warps at most); then one thread per last-node fiber, or block of them.
+  // The line at d = 256 for three nodes: at d = 216 the row mapping takes half the fiber mapping's time, at d = 729 a
+  // third more (figures at cheb_run_row in kt_device.cuh).
+  const bool acs = (nl == 6 || nl == 9) && S <= 2 && cavity_structure(gf, gb, lo_dl, lo_val, ra_dl, ra_val);
+  const bool ri = acs && acs_constants_ok(gf, gb, lo_val, ra_val) && ri_classes(gf, gb, lo_val, ra_val, cols, true);
+  const int npair = (int)gf.pairs.size();
+  const bool few = (nl == 6 || nl == 9) && d / nl < 16;
+  const bool autom = cfg->items_per_thread == 0 && (cfg->tile_traj <= 0 || (density && few));
+  const int row_max = N <= 2 && npair <= 1 ? (cfg->prec == KT_FP64 ? 512 : 1024) : 736;   // its launch bounds
+  const bool row = N <= 3 && npair <= 3 && S <= 2 && (long long)d * std::max(1, cfg->tile_traj) <= row_max && (N <= 2 || d <= 256) &&
+                   (autom || cfg->items_per_thread == 1) &&
+                   (ri || ri_classes(gf, gb, lo_val, ra_val, cols, false));
+  if (ri || row) S = 2;
+  const bool small = few && autom;
+  const int ipt = cfg->items_per_thread > 0 ? cfg->items_per_thread : (small || row ? 1 : 0);
   const bool fiber = (nl == 6 || nl == 9) && ipt == 0;
-  const bool acs = fiber && cavity_structure(gf, gb, lo_dl, lo_val, ra_dl, ra_val);
-  const bool ri = acs && S <= 2 && ri_classes(gf, gb, lo_val, ra_val, cols) && acs_constants_ok(gf, gb, lo_val, ra_val);
-  if (ri) S = 2;
   g.S = std::max(S, 1);
   int SH = 1;
   for (int t = 0; t < nterm; ++t)
@@ -1431,7 +1462,7 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
 
   // ---- tile width, threads per CTA, items per thread
   const int esz = P.fp64 ? 16 : 8;
-  const int maxthr = P.fp64 ? 512 : 1024;
+  const int maxthr = row ? row_max : (P.fp64 ? 512 : 1024);
   if (cfg->tile_traj > 0 && ((cfg->tile_traj & (cfg->tile_traj - 1)) || cfg->tile_traj > 32))
     return fail(KT_ERR_ARG, "tile_traj must be a power of two <= 32");
   // fiber mapping (one thread per run of n_loc elements along the last node) for the compiled
@@ -1457,7 +1488,7 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
     if (kt_smem_bytes(t, esz, false) > 227 * 1024) continue;
     // small problems on the automatic strided mapping: tiles of at most 128 items (a few warps),
     // latency rather than throughput decides there
-    if (small && cfg->items_per_thread == 0 && cfg->tile_traj <= 0 && T > 1 && (long long)d * T > 128) continue;
+    if ((small || row) && cfg->items_per_thread == 0 && cfg->tile_traj <= 0 && T > 1 && (long long)d * T > 128) continue;
     Tsel = T;
     // prefer more tiles when the trajectories would not fill the GPU
     // (a shard plans with the whole problem's trajectory count: every shard needs the same tile width)
@@ -1480,10 +1511,32 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
     P.n_tiles_total = (cfg->M_total + Tsel - 1) / Tsel;
   }
   g.tile_elems = (d * Tsel + 3) / 4 * 4;
+  int regs = 128;   // registers per thread, roughly (the launch bounds cap them): resident CTAs below
+  if (fiber) {
+    // launcher codes -(100 v + nl): v = 0 fiber, 1 cavity structure, 2 the same with T = 1 compiled
+    // in, 3 cavity structure with real / imaginary couplings, 4 the same with T = 1 (n_loc = 9)
+    int v = 0;
+    if (acs) v = ri ? (nl == 9 && Tsel == 1 ? 4 : 3) : (nl == 9 && Tsel == 1 ? 2 : 1);
+    P.ept = -(100 * v + nl);
+    g.nthreads = std::max(32, ((d / nl) * Tsel + 31) / 32 * 32);
+    regs = g.nthreads <= 256 && ri && P.fp64 ? 160 : 80;
+    // 5: block mapping of four-node problems in FP32 (three nodes leave it 27 threads per trajectory)
+    if (ri && !P.fp64 && Tsel == 1 && N == 4 && block_structure(N, nl, cols)) {
+      P.ept = -(500 + nl);
+      g.nthreads = (d / (nl / 3 * nl) + 31) / 32 * 32;
+      regs = 255;
+    }
+  } else {
+    const int items = d * Tsel;
+    int ept = ipt > 0 ? ipt : 4;
+    while ((items + ept - 1) / ept > maxthr) ept *= 2;
+    P.ept = ept;
+    g.nthreads = std::max(32, ((items + ept - 1) / ept + 31) / 32 * 32);
+    if (row) P.ept = N <= 2 && npair <= 1 ? 21 : 33;   // ept is 1
+    if (row) regs = g.nthreads > 256 ? (P.fp64 ? 80 : 40) : (P.fp64 ? 128 : 80);
+  }
   {
-    KtGeom t = g;
-    t.nthreads = fiber ? std::max(32, ((d / nl) * Tsel + 31) / 32 * 32) : maxthr;
-    const size_t smem3 = kt_smem_bytes(t, esz, true);
+    const size_t smem3 = kt_smem_bytes(g, esz, true);
     g.prefetch_chi = smem3 <= 227 * 1024 ? 1 : 0;
     // backward kernel: when the tiles need several waves and a third buffer fits, CTAs loop over
     // tiles (about one CTA per SM slot) and prefetch the next tile's input during the current series
@@ -1492,32 +1545,20 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
     g.fwd_grid = 0;
     if (g.prefetch_chi && cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
-      const int per_sm = std::max(1, std::min((int)((227 * 1024) / smem3), 2048 / std::max(32, t.nthreads)));
+      const int slots = std::max(1, std::min(2048 / g.nthreads, 65536 / (regs * g.nthreads)));
+      const int per_sm = std::max(1, std::min((int)((227 * 1024) / smem3), slots));
       if (g.n_tiles > sms * per_sm) g.bwd_grid = sms * per_sm;
       // forward kernel: the same tile loop when a fourth buffer (the next tile's psi) fits as well
-      const size_t smem4 = kt_smem_bytes(t, esz, true, true);
+      const size_t smem4 = kt_smem_bytes(g, esz, true, true);
       if (smem4 <= 227 * 1024) {
-        const int per_sm4 = std::max(1, std::min((int)((227 * 1024) / smem4), 2048 / std::max(32, t.nthreads)));
+        const int per_sm4 = std::max(1, std::min((int)((227 * 1024) / smem4), slots));
         if (g.n_tiles > sms * per_sm4) g.fwd_grid = sms * per_sm4;
       }
     }
   }
-  if (fiber) {
-    // launcher codes -(100 v + nl): v = 0 fiber, 1 cavity structure, 2 the same with T = 1 compiled
-    // in, 3 cavity structure with real / imaginary couplings, 4 the same with T = 1 (n_loc = 9)
-    int v = 0;
-    if (acs) v = ri ? (nl == 9 && Tsel == 1 ? 4 : 3) : (nl == 9 && Tsel == 1 ? 2 : 1);
-    P.ept = -(100 * v + nl);
-    g.nthreads = std::max(32, ((d / nl) * Tsel + 31) / 32 * 32);
-  } else {
-    const int items = d * Tsel;
-    int ept = ipt > 0 ? ipt : 4;
-    while ((items + ept - 1) / ept > maxthr) ept *= 2;
-    P.ept = ept;
-    g.nthreads = std::max(32, ((items + ept - 1) / ept + 31) / 32 * 32);
-  }
 
-  // ---- generator tables (scaled by 1/r) for both directions
+  // ---- generator tables for both directions: B = -2i (G - c) / r
+  const cd scale = cd(0.0, -2.0) / r;
   auto build_image = [&](const Gen &gen, double cgen, HostImage &im) {
     const int nls = nl * g.S;
     im.dl.assign((size_t)N * nls, 0);
@@ -1532,11 +1573,12 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
           if (cl[q] == x) continue;                  // empty slot
           const size_t e = (size_t)i * nls + x * g.S + q;
           im.dl[e] = cl[q] - x;
-          const cd v = at(gen.loc, i * nl * nl, nl, x, cl[q]) / r;
+          const cd v = at(gen.loc, i * nl * nl, nl, x, cl[q]) * scale;
           im.base[e] = KtCplx{v.real(), v.imag()};
         }
-        cd dv = at(gen.loc, i * nl * nl, nl, x, x) / r;
-        if (i == 0) dv -= cgen / r;
+        cd dv = at(gen.loc, i * nl * nl, nl, x, x);
+        if (i == 0) dv -= cgen;
+        dv *= scale;
         im.dg[(size_t)i * nl + x] = KtCplx{dv.real(), dv.imag()};
       }
     for (int t = 0; t < nterm; ++t) {
@@ -1545,10 +1587,10 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
         const std::vector<int> &cl = cols[(size_t)i * nl + x];
         for (size_t q = 0; q < cl.size(); ++q) {
           if (cl[q] == x) continue;
-          const cd v = at(gen.ctrl, t * nl * nl, nl, x, cl[q]) / r;
+          const cd v = at(gen.ctrl, t * nl * nl, nl, x, cl[q]) * scale;
           im.cslot[(size_t)t * nls + x * g.S + q] = KtCplx{v.real(), v.imag()};
         }
-        const cd dv = at(gen.ctrl, t * nl * nl, nl, x, x) / r;
+        const cd dv = at(gen.ctrl, t * nl * nl, nl, x, x) * scale;
         im.cdg[(size_t)t * nl + x] = KtCplx{dv.real(), dv.imag()};
       }
     }
@@ -1560,7 +1602,8 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
       const Pair &pr = gen.pairs[q];
       im.pdst[q] = pr.dst;
       im.psrc[q] = pr.src;
-      im.pc[q] = KtCplx{(pr.coef / r).real(), (pr.coef / r).imag()};
+      const cd ps = pr.coef * scale;
+      im.pc[q] = KtCplx{ps.real(), ps.imag()};
       const bool rd = pr.kind != 1, rs = pr.kind == 2;     // raise the dst / src node?
       for (int xd = 0; xd < nl; ++xd)
         for (int xs = 0; xs < nl; ++xs) {
@@ -1568,7 +1611,7 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
           if (vd == 0.0 || vs == 0.0) continue;
           const size_t e = (size_t)q * nl2 + xd * nl + xs;
           im.poff[e] = (rd ? ra_dl[xd] : lo_dl[xd]) * g.stride[pr.dst] + (rs ? ra_dl[xs] : lo_dl[xs]) * g.stride[pr.src];
-          const cd v = pr.coef * vd * vs / r;
+          const cd v = pr.coef * vd * vs * scale;
           im.pval[e] = KtCplx{v.real(), v.imag()};
         }
     }
@@ -1579,25 +1622,33 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
         im.kd[2 * x] = im.dg[(size_t)last * nl + x].re;
         im.kd[2 * x + 1] = im.dg[(size_t)last * nl + x].im;
       }
-      auto slot_re = [&](int x, int y) {
+      auto slot_im = [&](int x, int y) {
         for (int q = 0; q < g.S; ++q) {
           const size_t e = (size_t)last * nls + x * g.S + q;
-          if (im.dl[e] == y - x) return im.base[e].re;
+          if (im.dl[e] == y - x) return im.base[e].im;
         }
         return 0.0;
       };
       for (int n = 1; n <= NC; ++n) {
         const int qr = 2 * NP + n - 1, qg = n;
-        im.kc[n - 1] = slot_re(qr, qg);
-        im.kc[NC + n - 1] = slot_re(qg, qr);
+        im.kc[n - 1] = slot_im(qr, qg);
+        im.kc[NC + n - 1] = slot_im(qg, qr);
       }
-      for (int q = 0; q < g.n_pairs; ++q) im.kp[q] = im.pc[q].im;
+      for (int q = 0; q < g.n_pairs; ++q) {
+        im.kp[q] = im.pc[q].re;
+        const int ds = im.pdst[q], sr = im.psrc[q], mid = N - 2;
+        if (ds >= mid && sr < mid) im.kh[ds == mid ? 0 : 1][sr & 1] = im.kp[q];
+        else if (ds < mid && sr >= mid) im.kh[sr == mid ? 2 : 3][ds & 1] = im.kp[q];
+        else if (ds >= mid && sr >= mid) im.kh[4][ds == last ? 0 : 1] = im.kp[q];
+      }
     }
-    im.cf.resize(K);
-    const cd ph = std::exp(cd(0.0, -cgen * dt));
-    for (int k = 0; k < K; ++k) {
-      const cd v = (k == 0 ? 1.0 : 2.0) * J[k] * std::pow(cd(0.0, -1.0), k) * ph;
-      im.cf[k] = KtCplx{v.real(), v.imag()};
+    const int sets = P.fp64 ? 1 : KT_COEF_SETS;
+    im.cf.resize((size_t)sets * K);
+    im.phase.resize(sets);
+    for (int s = 0; s < sets; ++s) {
+      const double golden = 0.6180339887498949 * s, lambda = 1.0 + (golden - std::floor(golden));
+      for (int k = 0; k < K; ++k) im.cf[(size_t)s * K + k] = lambda * (k == 0 ? 1.0 : 2.0) * J[k];
+      im.phase[s] = KtCplx{std::cos(cgen * dt) / lambda, -std::sin(cgen * dt) / lambda};
     }
   };
   build_image(gf, c_fwd, P.fwd);
@@ -1637,6 +1688,9 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
   P.tgt.resize(d);
   for (int x = 0; x < d; ++x) P.tgt[x] = KtCplx{psi_t[x].real(), psi_t[x].imag()};
   P.density = density ? 1 : 0;
+  P.cavity_ri = ri;
+  P.items_reported = fiber || (row && !few && cfg->items_per_thread == 0) ? 0 : ipt > 0 ? ipt : P.ept;
+  P.sweeps = !fiber && (few || g.nthreads <= 256 || cfg->items_per_thread > 0 || !row);
   g.density = P.density;
   if (density) {
     P.psi0.resize((size_t)2 * d);
@@ -1657,7 +1711,7 @@ kt_status upload_image(kt_problem *p, const HostImage &h, KtGenImage &im, cudaSt
   if ((t = upload(p, (KtCplx **)&im.ctrl_diag, h.cdg.data(), h.cdg.size(), st)) != KT_OK) return t;
   if ((t = upload(p, (int **)&im.pair_off, h.poff.data(), h.poff.size(), st)) != KT_OK) return t;
   if ((t = upload(p, (KtCplx **)&im.pair_val, h.pval.data(), h.pval.size(), st)) != KT_OK) return t;
-  if ((t = upload(p, (KtCplx **)&im.cheb_full, h.cf.data(), h.cf.size(), st)) != KT_OK) return t;
+  if ((t = upload(p, (double **)&im.cheb_full, h.cf.data(), h.cf.size(), st)) != KT_OK) return t;
   if ((t = upload(p, (KtCplx **)&im.pair_coef, h.pc.data(), h.pc.size(), st)) != KT_OK) return t;
   for (int q = 0; q < KT_MAX_PAIRS; ++q) {
     im.pair_dst[q] = h.pdst[q];
@@ -1665,10 +1719,14 @@ kt_status upload_image(kt_problem *p, const HostImage &h, KtGenImage &im, cudaSt
     im.kp32[q] = (float)h.kp[q];
     im.kp64[q] = h.kp[q];
   }
-  for (int q = 0; q < 2 * KT_MAX_NL; ++q) {
-    im.kd32[q] = (float)h.kd[q];
-    im.kd64[q] = h.kd[q];
+  if ((t = upload(p, (KtCplx **)&im.phase_full, h.phase.data(), h.phase.size(), st)) != KT_OK) return t;
+  im.sets = (int)h.phase.size();
+  for (int q = 0; q < 2 * KT_MAX_NL; ++q) im.kd64[q] = h.kd[q];
+  for (int q = 0; q < KT_MAX_NL; ++q) {
+    im.kd32[3 * q] = (float)h.kd[2 * q];
+    kt_split(h.kd[2 * q + 1], &im.kd32[3 * q + 1], &im.kd32[3 * q + 2]);
   }
+  for (int q = 0; q < 10; ++q) im.kh[q / 2][q % 2] = (float)h.kh[q / 2][q % 2];
   for (int q = 0; q < 4; ++q) {
     im.kc32[q] = (float)h.kc[q];
     im.kc64[q] = h.kc[q];
@@ -1732,6 +1790,8 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
   p->g = P.g;
   p->fp64 = P.fp64;
   p->ept = P.ept;
+  p->cavity_ri = P.cavity_ri;
+  p->items_reported = P.items_reported;
   p->cross = P.cross;
   p->density = P.density;
   p->sharded = P.sharded;
@@ -1800,8 +1860,7 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
     if (cudaMemsetAsync(p->jcount[b], 0, Mp * sizeof(int), st) != cudaSuccess) { krotov_free(p); return fail(KT_ERR_CUDA, "memset"); }
   }
   TRY(dev_alloc(p, (void **)&p->cursor, Mp * sizeof(int)));
-  // two sets: a whole-sweep launch alternates them by interval parity
-  TRY(dev_alloc(p, (void **)&p->partials, (size_t)2 * g.n_tiles * nc * sizeof(double)));
+  TRY(dev_alloc(p, (void **)&p->partials, (size_t)g.n_tiles * nc * sizeof(double)));
   if (p->sharded) {
     TRY(dev_alloc(p, (void **)&p->spart, (size_t)p->n_tiles_total * nc * sizeof(double)));
     TRY(dev_alloc(p, (void **)&p->tau_all, (size_t)p->M_total * sizeof(KtCplx)));
@@ -1828,15 +1887,15 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
     TRY(dev_alloc(p, &p->chi, p->state_bytes * p->n_chi_slots));
     if (p->ckpt > 0) TRY(dev_alloc(p, &p->seg, p->state_bytes * (p->ckpt + 1)));
     // whole-sweep launches: the strided mapping (the small problems' mapping; the sweep kernels are
-    // compiled for it only), every tile resident at once (the forward sweep's grid barrier), every
+    // compiled for it only), every tile resident at once (the forward sweep's exchange of partials), every
     // co-state kept (each interval's co-state has its slot), no exchange with other shards and no
     // pair sums between intervals
     int dev = 0, sms = 0, per = 0;
-    if (!cfg->per_interval_launches && p->ept > 0 && p->ckpt == 0 && !p->sharded && !p->cross &&
+    if (!cfg->per_interval_launches && P.sweeps && p->ckpt == 0 && !p->sharded && !p->cross &&
         cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         kt_fwd_blocks_per_sm(p->fp64, p->ept, g, &per) == cudaSuccess && (long long)per * sms >= g.n_tiles) {
-      TRY(dev_alloc(p, (void **)&p->sync, 2 * sizeof(unsigned)));
+      TRY(dev_alloc(p, (void **)&p->wpart, (size_t)nt * g.n_tiles * nc * sizeof(double)));
       p->whole_sweep = 1;
     }
     cudaGetLastError();   // an occupancy query that failed leaves per-interval launches
@@ -1997,6 +2056,7 @@ KT_API kt_status kt_generator_dense(const kt_model_desc *md, const kt_config *cf
   const KtGeom &g = P.g;
   const HostImage &im = (direction & 1) ? P.bwd : P.fwd;
   const double cgen = (direction & 1) ? g.c_bwd : g.c_fwd;
+  const cd unscale = cd(0.0, 0.5) * g.r;   // the tables hold B = -2i (G - c) / r
   const int d = g.d, nl = g.n_loc, nls = nl * g.S, nl2 = nl * nl;
   std::fill(out, out + (size_t)d * d * 2, 0.0);
   auto add = [&](int x, int y, cd v) -> bool {
@@ -2021,17 +2081,17 @@ KT_API kt_status kt_generator_dense(const kt_model_desc *md, const kt_config *cf
         for (int t = 0; t < g.n_cterms; ++t)
           if (g.cterm_node[t] == i)
             v += eps[g.cterm_ctrl[t]] * cd(im.cslot[(size_t)t * nls + xi * g.S + q].re, im.cslot[(size_t)t * nls + xi * g.S + q].im);
-        if (!add(x, x + im.dl[e] * g.stride[i], v * g.r)) return fail(KT_ERR_RANGE, "node entry leaves the space at row %d", x);
+        if (!add(x, x + im.dl[e] * g.stride[i], v * unscale)) return fail(KT_ERR_RANGE, "node entry leaves the space at row %d", x);
       }
     }
     for (int q = 0; q < g.n_pairs; ++q) {
       const int xd = (dig >> (4 * im.pdst[q])) & 15, xs = (dig >> (4 * im.psrc[q])) & 15;
       const size_t e = (size_t)q * nl2 + xd * nl + xs;
       if (!im.poff[e]) continue;
-      if (!add(x, x + im.poff[e], cd(im.pval[e].re, im.pval[e].im) * g.r))
+      if (!add(x, x + im.poff[e], cd(im.pval[e].re, im.pval[e].im) * unscale))
         return fail(KT_ERR_RANGE, "pair entry leaves the space at row %d", x);
     }
-    add(x, x, dv * g.r + cgen);
+    add(x, x, dv * unscale + cgen);
   }
   return KT_OK;
 }
@@ -2249,7 +2309,7 @@ KT_API kt_status krotov_get_info(kt_problem *p, kt_info *info) {
   info->ckpt_interval = p->ckpt;
   info->ckpt_kept_prefix = p->ckpt == 0 ? p->nt : p->ckpt_dense;
   info->costate_slots = p->n_chi_slots;
-  info->items_per_thread = p->ept > 0 ? p->ept : 0;
+  info->items_per_thread = p->items_reported;
   info->whole_sweep = p->whole_sweep;
   return KT_OK;
 }

@@ -54,14 +54,12 @@ struct FwdArgs {
   // whole forward sweep in one cooperative launch (one tile per CTA, every CTA resident): intervals
   // j .. nt, the state kept in shared memory between them; psi(t_i) goes to psi_ring[i & 1] (the
   // input of interval 1 is psi_in), chi(t_i) is read from chi_slots + i * slot_bytes.  With the
-  // update the CTAs meet at a grid barrier (sync: two words, zero at the launch) after each
-  // interval's overlap, and every CTA forms Delta eps from all tiles' partials in the finisher's
-  // order (partials double-buffered by interval parity: [2][n_tiles][n_ctrl]).
+  // update every CTA puts its partials of interval i into partials [nt][n_tiles][n_ctrl] (every bit set
+  // at the launch: not there yet), and forms Delta eps from all tiles' partials in the finisher's order.
   int sweep;
   void *psi_ring[2];
   const void *chi_slots;
   size_t slot_bytes;
-  unsigned *sync;
 };
 
 struct BwdArgs {
