@@ -15,6 +15,18 @@
 // dP/deps_i Z = exp(-i c tau) sum_k m_k y_k with the propagator's own coefficients (the same constants c, r:
 // only B depends on eps).
 //
+// That costs 2 n_ctrl generator applications per term.  Where the generator has the cavity structure with real /
+// imaginary classes and the controls are its drives, grad_adj_kernel differentiates the series in reverse instead:
+// with Wt = exp(-i c tau)^* W,
+//   b_k = m_k Wt + b_{k+2} + B^dag b_{k+1}  (b_K = 0; the last step, k = 0, with B^dag b_1 / 2),
+//   Re <W| dP/deps_i |Z> = Re sum_{k >= 1} <b_{k+1}| B_i |z_k> + Re <b_1| B_i |z_0> / 2,   b_0 = P^dag W,
+// two applications per term whatever the number of controls, and b_0 is the co-state at the start of the piece, so the
+// backward interval kernel is not launched.  B_i has the drive's entries only: its bilinear forms take the neighbour
+// values that B^dag loads anyway.  The z_k of a thread's own fiber wait in global memory (K states; written and
+// read back once, coalesced, mostly in L2).  Per interval, gradient, backward and replay launches of before together against
+// this one: d = 729, 1024 trajectories, three controls, FP32 572 -> 175 us; d = 6561, 64 trajectories 2084 -> 159 us; d = 216,
+// 200 trajectories 362 -> 50 us; d = 81, 100 trajectories, FP64 693 -> 380 us.
+//
 // One CTA per trajectory, gathered from the problem's interleaved tile layout.
 #include "kt_device.cuh"
 
@@ -106,112 +118,341 @@ __device__ void aug_run(const KtGeom &g, const KtGenImage &im, const Smem &sm, c
   apply_phase<R, EPT>(g, sm, 0, acc, [&](int q) { return it.ok(q) ? dv[q].lo : (R)0; });
 }
 
-// Fiber form of B_c v for the thread's fiber (tile width 1): a control on the last node
-// takes row q of its factor for element q, a control on another node one row for the whole fiber.
-// Same entries and order as hc_item.
-template <typename R, int NL>
-__device__ __forceinline__ void hc_fiber(const KtGeom &g, const Smem &sm, int c, const typename C2<R>::T *v, int base,
-                                         uint32_t fdig, R invr, typename C2<R>::T (&h)[NL]) {
-  typedef typename C2<R>::T C;
-  const C *hv = (const C *)sm.hc_val;
-  const int node = g.ctrl_node[c];
-#pragma unroll
-  for (int q = 0; q < NL; ++q) h[q] = mkc((R)0, (R)0);
-  if (node == g.n_nodes - 1) {
-#pragma unroll
-    for (int q = 0; q < NL; ++q) {
-      const int b = (c * g.n_loc + q) * g.SH;
-      for (int e = 0; e < g.SH; ++e) {
-        const C w = hv[b + e];
-        if (w.x != (R)0 || w.y != (R)0) h[q] = cfma(w, v[base + q + sm.hc_off[b + e]], h[q]);
-      }
-    }
-  } else {
-    const int b = (c * g.n_loc + ((fdig >> (4 * node)) & 15)) * g.SH;
-    for (int e = 0; e < g.SH; ++e) {
-      const C w = hv[b + e];
-      if (w.x != (R)0 || w.y != (R)0) {
-        const int off = sm.hc_off[b + e];
-#pragma unroll
-        for (int q = 0; q < NL; ++q) h[q] = cfma(w, v[base + off + q], h[q]);
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < NL; ++q) h[q] = mkc((R)2 * h[q].y * invr, (R)-2 * h[q].x * invr);
-}
-
-// aug_run in the fiber mapping with tile width 1, for the cavity structure with real / imaginary
-// coupling classes: the same two recurrences, Ghat applied by apply_acs.
-template <typename R, int NC, class IT>
-__device__ void aug_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &sm, const IT &it, int K, int c,
-                            typename C2<R>::T *Dbuf, typename C2<R>::T (&acc)[3 * (NC + 1)]) {
-  typedef typename C2<R>::T C;
-  constexpr int NL = 3 * (NC + 1);
-  C *A = (C *)sm.bufA, *B = (C *)sm.bufB, *Cb = (C *)sm.bufC, *D = Dbuf;
-  const R *cf = (const R *)sm.coef;
-  const R invr = (R)(1.0 / g.r);
-  const bool ok = it.ok(0);
-  const int base = it.item(0);
-  const uint32_t fdig = it.dig(0);
-  const int last = g.n_nodes - 1;
-  Diag<R> Df{(R)0, (R)0, (R)0};
-  for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
-#pragma unroll
-  for (int q = 0; q < NL; ++q) {
-    acc[q] = mkc((R)0, (R)0);
-    if (ok) Cb[base + q] = mkc((R)0, (R)0);   // y_0 = 0
-  }
-  if (K < 2) { __syncthreads(); return; }
-  C v[NL], t[NL], h[NL];
-  RowCache<R> rc;
-  if (ok) load_rows<R, NL>(g, sm, fdig, rc);
-  if (ok) {
-#pragma unroll
-    for (int q = 0; q < NL; ++q) v[q] = A[base + q];
-    apply_acs<R, NC, 1, true, true, false>(g, im, sm, A, A, base, fdig, Df, v, t, rc);
-    hc_fiber<R, NL>(g, sm, c, A, base, fdig, invr, h);
-    const R c1 = cf[1];
-#pragma unroll
-    for (int q = 0; q < NL; ++q) {
-      B[base + q] = mkc((R)0.5 * t[q].x, (R)0.5 * t[q].y);
-      D[base + q] = mkc((R)0.5 * h[q].x, (R)0.5 * h[q].y);
-      acc[q] = rfma(c1, mkc((R)0.5 * h[q].x, (R)0.5 * h[q].y), acc[q]);
-    }
+// The CTA's sums per control and, in the last CTA, dJ_T/deps of interval j.
+__device__ __forceinline__ void grad_finish(const KtGeom &g, const Smem &sm, const GradArgs &a, double (&part)[KT_MAX_CTRL]) {
+  const int k = blockIdx.x, j = a.j;
+  reduce_tau<KT_MAX_CTRL>(part, g, sm.red, sm.tsc + TS_V0 * g.T);
+  if (threadIdx.x < g.n_ctrl) a.partials[(size_t)k * g.n_ctrl + threadIdx.x] = sm.tsc[TS_V0 * g.T + threadIdx.x];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned ticket = atomicAdd(a.counter, 1u);
+    sm.flag[3] = (ticket == (unsigned)(gridDim.x - 1));
   }
   __syncthreads();
-  C *Pz = A, *Qz = B, *Py = Cb, *Qy = D;
-  for (int k = 2; k < K; ++k) {
-    if (ok) {
-      const R ak = cf[k];
-#pragma unroll
-      for (int q = 0; q < NL; ++q) v[q] = Qz[base + q];
-      apply_acs<R, NC, 1, true, true, true>(g, im, sm, Qz, Pz, base, fdig, Df, v, t, rc);
-      hc_fiber<R, NL>(g, sm, c, Qz, base, fdig, invr, h);
-#pragma unroll
-      for (int q = 0; q < NL; ++q) {
-        Pz[base + q] = t[q];
-        v[q] = Qy[base + q];
-      }
-      apply_acs<R, NC, 1, true, true, true>(g, im, sm, Qy, Py, base, fdig, Df, v, t, rc);
-#pragma unroll
-      for (int q = 0; q < NL; ++q) {
-        const C ny = mkc(t[q].x + h[q].x, t[q].y + h[q].y);
-        Py[base + q] = ny;
-        acc[q] = rfma(ak, ny, acc[q]);
-      }
-    }
-    __syncthreads();
-    C *t1 = Pz; Pz = Qz; Qz = t1;
-    C *t2 = Py; Py = Qy; Qy = t2;
+  if (!sm.flag[3]) return;
+  __threadfence();
+  const int chunk = ((int)gridDim.x + blockDim.x - 1) / blockDim.x;
+  const int t0 = threadIdx.x * chunk, t1 = min((int)gridDim.x, t0 + chunk);
+  for (int c = 0; c < g.n_ctrl; ++c) {
+    double v = 0.0;
+    for (int t = t0; t < t1; ++t) v += __ldcg(a.partials + (size_t)t * g.n_ctrl + c);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sm.red[(threadIdx.x >> 5) * 8 + c] = v;
   }
-  apply_phase<R, NL>(g, sm, 0, acc, [&](int q) { return Df.lo + acs_kd<R>(im, q).lo; });
+  __syncthreads();
+  if (threadIdx.x < g.n_ctrl) {
+    double s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sm.red[w * 8 + threadIdx.x];
+    const double gr = -2.0 / (double)g.M * s;
+    a.grad[(size_t)threadIdx.x * a.nt + (j - 1)] = gr;
+    if (!isfinite(gr)) set_status(a.status, KT_DEV_NONFINITE);
+  }
+  if (threadIdx.x == 0) *a.counter = 0u;
 }
 
-// NL = 0: strided items (EPT per thread); NL = 9 with ACS = 4: fiber mapping, tile width 1,
-// cavity structure with real / imaginary coupling classes.
-template <typename R, int EPT, int NL, int ACS>
-__global__ void __launch_bounds__(NL > 0 ? 96 : (EPT == 4 ? 256 : 1024), NL > 0 ? 5 : 1)
+// One step of the reverse series on the thread's fiber (tile width 1): out[q] = h (B^dag b)[q] + add[q], b's own values
+// in bk, add[q] = m W[q] + prev[base + q]; and dot[i] += h sum_q Re(conj(b at the drive neighbour of node i) y[q]) for the
+// outer nodes, dl[.] the same for the last node, one slot per e_n and r_n row.
+template <typename R, int NC>
+__device__ __forceinline__ void adj_step(const KtGeom &g, const KtGenImage &im, const Smem &sm,
+                                         const typename C2<R>::T *__restrict__ v, const typename C2<R>::T *prev, int base,
+                                         uint32_t fdig, Diag<R> Df, const RowCache<R> &rc, R h, R m,
+                                         const typename C2<R>::T (&w)[3 * (NC + 1)], typename C2<R>::T (&bk)[3 * (NC + 1)],
+                                         const typename C2<R>::T *__restrict__ ysrc, int ystride, R (&dot)[3],
+                                         R (&dl)[2 * (NC + 1)]) {
+  typedef typename C2<R>::T C;
+  constexpr int NP = NC + 1, NL = 3 * NP;
+  const C *pv = (const C *)sm.pair_val;
+  const C *ld = (const C *)sm.ldense;
+  const int last = g.n_nodes - 1;
+  C y[NL], out[NL];
+#pragma unroll
+  for (int q = 0; q < NL; ++q) y[q] = ysrc[(size_t)q * ystride];
+#pragma unroll
+  for (int q = 0; q < NL; ++q) {
+    const R re = Df.re + acs_kd<R>(im, q).re;
+    out[q] = mkc(re * bk[q].x, re * bk[q].y);
+  }
+#pragma unroll
+  for (int n = 1; n <= NC; ++n) {
+    const int qr = 2 * NP + n - 1, qg = n;
+    out[qr] = ifma(acs_kc<R>(im)[n - 1], bk[qg], out[qr]);
+    out[qg] = ifma(acs_kc<R>(im)[NC + n - 1], bk[qr], out[qg]);
+  }
+#pragma unroll
+  for (int n = 0; n <= NC; ++n) {
+    const int qr = 2 * NP + n, qe = NP + n;
+    out[qr] = rfma(ld[qr * NL + qe].x, bk[qe], out[qr]);
+    out[qe] = rfma(ld[qe * NL + qr].x, bk[qr], out[qe]);
+    dl[n] = fma(h, bk[qr].x * y[qe].x + bk[qr].y * y[qe].y, dl[n]);               // row e_n, neighbour r_n
+    dl[NP + n] = fma(h, bk[qe].x * y[qr].x + bk[qe].y * y[qr].y, dl[NP + n]);     // row r_n, neighbour e_n
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (rc.off0[i]) {
+#pragma unroll
+      for (int q = 0; q < NL; ++q) out[q] = ifma(rc.a[i], v[base + rc.off0[i] + q], out[q]);
+    }
+    if (rc.off1[i]) {
+      R s = (R)0;
+#pragma unroll
+      for (int q = 0; q < NL; ++q) {
+        const C x = v[base + rc.off1[i] + q];
+        out[q] = rfma(rc.b[i], x, out[q]);
+        s = fma(x.x, y[q].x, s);
+        s = fma(x.y, y[q].y, s);
+      }
+      dot[i] = fma(h, s, dot[i]);
+    }
+  }
+  for (int p = 0; p < g.n_pairs; ++p) {
+    const int pd = im.pair_dst[p], ps = im.pair_src[p];
+    if (pd != last && ps != last) {
+      const int e = p * NL * NL + ((fdig >> (4 * pd)) & 15) * NL + ((fdig >> (4 * ps)) & 15);
+      const int off = sm.pair_off[e];
+      if (off) {
+        const R b = pv[e].x;
+#pragma unroll
+        for (int q = 0; q < NL; ++q) out[q] = rfma(b, v[base + off + q], out[q]);
+      }
+    } else if (pd == last) {
+      const int xs = (fdig >> (4 * ps)) & 15;
+      if (xs % NP < NC) {
+        const int off = g.stride[ps];
+        const R cb = acs_kp<R>(im)[p] * sqrt_n<R>(xs % NP + 1);
+#pragma unroll
+        for (int q = 0; q < NL; ++q)
+          if (q % NP != 0) out[q] = rfma(cb * sqrt_n<R>(q % NP), v[base + off + q - 1], out[q]);
+      }
+    } else {
+      const int xd = (fdig >> (4 * pd)) & 15;
+      if (xd % NP >= 1) {
+        const int off = -g.stride[pd];
+        const R cb = acs_kp<R>(im)[p] * sqrt_n<R>(xd % NP);
+#pragma unroll
+        for (int q = 0; q < NL; ++q)
+          if (q % NP != NC) out[q] = rfma(cb * sqrt_n<R>(q % NP + 1), v[base + off + q + 1], out[q]);
+      }
+    }
+  }
+  // the small terms first, as in the forward series
+#pragma unroll
+  for (int q = 0; q < NL; ++q) {
+    const R hi = h * (Df.hi + acs_kd<R>(im, q).hi);
+    const C old = prev[base + q];
+    C s = mkc(h * out[q].x, h * out[q].y);
+    s = rfma(m, w[q], s);
+    s.x += old.x;
+    s.y += old.y;
+    bk[q] = mkc(fma(-hi, bk[q].y, s.x), fma(hi, bk[q].x, s.y));
+  }
+}
+
+// Reverse gradient of interval j and the co-state at its start (see above).  One CTA per trajectory, one thread per
+// last-node fiber.
+template <typename R, int NC, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
+    grad_adj_kernel(KtGeom g, int T_layout, int tel, KtGenImage imf, KtGenImage imb, KtOps ops, GradArgs a) {
+  typedef typename C2<R>::T C;
+  constexpr int NP = NC + 1, NL = 3 * NP;
+  extern __shared__ __align__(16) char smem_raw[];
+  Smem sm;
+  carve(g, sizeof(C), smem_raw, &sm, false);
+  C *A = (C *)sm.bufA, *B = (C *)sm.bufB;
+  const int k = blockIdx.x, j = a.j;
+  const size_t rb = (size_t)k * g.max_jumps;
+  if (threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = a.eps[threadIdx.x * a.nt + (j - 1)];
+  if (threadIdx.x < 8) sm.flag[threadIdx.x] = 0;
+  if (threadIdx.x == 0) {
+    // records of interval j in ascending time: walk down from the backward cursor, then reverse
+    int cur = a.cursor[k], n = 0, idx[12];
+    while (cur >= 0 && a.rec_step[rb + cur] == j && n < 12) idx[n++] = cur--;
+    if (cur >= 0 && a.rec_step[rb + cur] == j) set_status(a.status, KT_DEV_RECORD_FULL);
+    for (int m = 0; m < n; ++m) sm.tin[TI_J0 + m] = idx[n - 1 - m];
+    sm.tin[TI_NJ] = n;
+    a.cursor[k] = cur;
+  }
+  __syncthreads();
+  const int m = sm.tin[TI_NJ];
+  Items<NL, NL> it;
+  load_items<NL, NL>(g, ops, it);
+  const bool ok = it.ok(0);
+  const int base = it.item(0), last = g.n_nodes - 1;
+  const uint32_t fdig = it.dig(0);
+  const size_t tile = (size_t)(k / T_layout) * tel + (k % T_layout);
+  const C *psi = (const C *)a.psi_prev + tile, *chi = (const C *)a.chi_t + tile;
+  C *ybuf = (C *)a.scratch + (size_t)k * g.K * NL * blockDim.x + threadIdx.x;   // y_n element q at [n][q][thread]
+  const int ys = blockDim.x;
+  auto sb = [&](int p) -> double { return p == 0 ? 0.0 : (p > m ? g.dt : a.rec_s[rb + sm.tin[TI_J0 + p - 1]]); };
+  const R *cf = (const R *)sm.coef;
+  R dot[3] = {(R)0, (R)0, (R)0}, dl[2 * NP];
+#pragma unroll
+  for (int q = 0; q < 2 * NP; ++q) dl[q] = (R)0;
+  C w[NL];   // the co-state at the end of the current piece
+#pragma unroll
+  for (int q = 0; q < NL; ++q) w[q] = ok ? chi[(size_t)(base + q) * T_layout] : mkc((R)0, (R)0);
+  for (int q = m; q >= 0; --q) {
+    // ---- Z_q: psi(t_{j-1}) taken forward over pieces 0 .. q-1 and their jumps
+    if (ok) {
+#pragma unroll
+      for (int e = 0; e < NL; ++e) A[base + e] = psi[(size_t)(base + e) * T_layout];
+    }
+    build_tables<R>(g, imf, ops, sm, sm.eps, false);
+    __syncthreads();
+    for (int p = 0; p < q; ++p) {
+      C acc[NL];
+      if (threadIdx.x == 0) tau_coefs<R>(g, sm, 0, g.c_fwd, sb(p + 1) - sb(p));
+      __syncthreads();
+      cheb_run_acs<R, NC, 1, true, false>(g, imf, sm, it, g.K, acc);
+      if (ok) {
+#pragma unroll
+        for (int e = 0; e < NL; ++e) A[base + e] = acc[e];
+      }
+      __syncthreads();
+      const size_t ri = rb + sm.tin[TI_J0 + p];
+      const R cn = (R)a.rec_c[ri];
+      if (ok) {
+#pragma unroll 1
+        for (int e = 0; e < NL; ++e) {
+          const C z = lind_item<R>(g, ops, a.rec_ch[ri], 0, A, base + e, it.dig(e));
+          B[base + e] = mkc(cn * z.x, cn * z.y);
+        }
+      }
+      __syncthreads();
+      if (ok) {
+#pragma unroll
+        for (int e = 0; e < NL; ++e) A[base + e] = B[base + e];
+      }
+      __syncthreads();
+    }
+    // ---- y_0 .. y_{K-2} of piece q, each thread's fiber to its place in ybuf
+    if (m == 0) uniform_coefs<R>(g, sm, imf, j);
+    else if (threadIdx.x == 0) tau_coefs<R>(g, sm, 0, g.c_fwd, sb(q + 1) - sb(q));
+    RowCache<R> rc;
+    Diag<R> Df{(R)0, (R)0, (R)0};
+    if (ok) {
+      load_rows<R, NL>(g, sm, fdig, rc);
+      for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
+    }
+    {
+      C vk[NL], t[NL];
+      C *P = B, *Q = A;
+      if (ok) {
+#pragma unroll
+        for (int e = 0; e < NL; ++e) {
+          vk[e] = A[base + e];
+          ybuf[(size_t)e * ys] = vk[e];
+        }
+      }
+      for (int n = 1; n < g.K - 1; ++n) {
+        if (ok) {
+          if (n == 1) {
+            apply_acs<R, NC, 1, true, true, false>(g, imf, sm, Q, Q, base, fdig, Df, vk, t, rc);
+#pragma unroll
+            for (int e = 0; e < NL; ++e) t[e] = mkc((R)0.5 * t[e].x, (R)0.5 * t[e].y);
+          } else {
+            apply_acs<R, NC, 1, true, true, true>(g, imf, sm, Q, P, base, fdig, Df, vk, t, rc);
+          }
+#pragma unroll
+          for (int e = 0; e < NL; ++e) {
+            vk[e] = t[e];
+            P[base + e] = t[e];
+            ybuf[((size_t)n * NL + e) * ys] = t[e];
+          }
+        }
+        __syncthreads();
+        C *tmp = P; P = Q; Q = tmp;
+      }
+      __syncthreads();   // every read of the forward tables and of the coefficients' phase is done
+    }
+    // ---- the reverse series under B^dag (the backward direction's B), its phase the forward one's conjugate
+    if (threadIdx.x == 0) {
+      C *ph = (C *)sm.phase;
+      ph[0].y = -ph[0].y;
+      if (sizeof(R) == 4) ph[1].y = -ph[1].y;
+    }
+    build_tables<R>(g, imb, ops, sm, sm.eps, false);
+    __syncthreads();
+    if (ok) {
+      load_rows<R, NL>(g, sm, fdig, rc);
+      Df = Diag<R>{(R)0, (R)0, (R)0};
+      for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
+    }
+    apply_phase<R, NL>(g, sm, 0, w, [&](int e) { return Df.lo + acs_kd<R>(imb, e).lo; });
+    {
+      C bk[NL];
+      const R mk = cf[g.K - 1];
+      C *P = B, *Q = A;
+      if (ok) {
+#pragma unroll
+        for (int e = 0; e < NL; ++e) {
+          bk[e] = mkc(mk * w[e].x, mk * w[e].y);
+          Q[base + e] = bk[e];
+          P[base + e] = mkc((R)0, (R)0);
+        }
+      }
+      __syncthreads();
+      for (int n = g.K - 2; n >= 0; --n) {
+        if (ok) {
+          adj_step<R, NC>(g, imb, sm, Q, P, base, fdig, Df, rc, n == 0 ? (R)0.5 : (R)1, cf[n], w, bk,
+                          ybuf + (size_t)n * NL * ys, ys, dot, dl);
+#pragma unroll
+          for (int e = 0; e < NL; ++e) P[base + e] = bk[e];
+        }
+        __syncthreads();
+        C *tmp = P; P = Q; Q = tmp;
+      }
+      if (q > 0) {
+        // the jump that starts piece q: c L^dag (b_0 is in Q)
+        const size_t ri = rb + sm.tin[TI_J0 + q - 1];
+        const R cn = (R)a.rec_c[ri];
+        if (ok) {
+#pragma unroll 1
+          for (int e = 0; e < NL; ++e) {
+            const C z = lind_item<R>(g, ops, a.rec_ch[ri], 1, Q, base + e, it.dig(e));
+            P[base + e] = mkc(cn * z.x, cn * z.y);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < NL; ++e) w[e] = ok ? P[base + e] : mkc((R)0, (R)0);
+        __syncthreads();
+      } else {
+#pragma unroll
+        for (int e = 0; e < NL; ++e) w[e] = ok ? bk[e] : mkc((R)0, (R)0);
+      }
+    }
+  }
+  if (ok) {
+    C *out = (C *)a.chi_out + tile;
+#pragma unroll
+    for (int e = 0; e < NL; ++e) out[(size_t)(base + e) * T_layout] = w[e];
+  }
+  // the bilinear forms weighted with the control terms' entries (per unit eps, real: slot 1 of their node's rows)
+  double part[KT_MAX_CTRL];
+  const int nls = NL * g.S;
+#pragma unroll
+  for (int c = 0; c < KT_MAX_CTRL; ++c) {
+    part[c] = 0.0;
+    if (c >= g.n_ctrl || !ok) continue;
+    const int node = g.ctrl_node[c];
+    const KtCplx *slot = imb.ctrl_slot + (size_t)c * nls;
+    if (node == last) {
+#pragma unroll
+      for (int e = 0; e < 2 * NP; ++e) part[c] += (double)(R)slot[(NP + e) * g.S + 1].re * (double)dl[e];
+    } else {
+      R d = dot[0];
+      if (node == 1) d = dot[1];
+      if (node == 2) d = dot[2];
+      part[c] = (double)(R)slot[((fdig >> (4 * node)) & 15) * g.S + 1].re * (double)d;
+    }
+  }
+  grad_finish(g, sm, a, part);
+}
+
+// Strided items (EPT per thread): any model.
+template <typename R, int EPT>
+__global__ void __launch_bounds__(EPT == 4 ? 256 : 1024)
     grad_kernel(KtGeom g, int T_layout, int tel, KtGenImage imf, KtGenImage imb, KtOps ops, GradArgs a) {
   typedef typename C2<R>::T C;
   extern __shared__ __align__(16) char smem_raw[];
@@ -235,8 +476,8 @@ __global__ void __launch_bounds__(NL > 0 ? 96 : (EPT == 4 ? 256 : 1024), NL > 0 
   }
   __syncthreads();
   const int m = sm.tin[TI_NJ];
-  Items<EPT, NL> it;
-  load_items<EPT, NL>(g, ops, it);
+  Items<EPT, 0> it;
+  load_items<EPT, 0>(g, ops, it);
   const C *psi_t = (const C *)a.psi_prev;
   const C *chi_t = (const C *)a.chi_t;
   // piece boundaries s_0 = 0 < s_1 < ... < s_m < s_{m+1} = dt
@@ -300,8 +541,7 @@ __global__ void __launch_bounds__(NL > 0 ? 96 : (EPT == 4 ? 256 : 1024), NL > 0 
       for (int qq = 0; qq < EPT; ++qq)
         if (it.ok(qq)) A[it.item(qq)] = zq[qq];
       __syncthreads();
-      if constexpr (ACS == 4) aug_run_acs<R, NL / 3 - 1>(g, imf, sm, it, g.K, c, D, acc);
-      else aug_run<R, EPT>(g, imf, sm, it, g.K, c, D, acc);
+      aug_run<R, EPT>(g, imf, sm, it, g.K, c, D, acc);
       double sacc = 0.0;
 #pragma unroll
       for (int qq = 0; qq < EPT; ++qq)
@@ -309,66 +549,50 @@ __global__ void __launch_bounds__(NL > 0 ? 96 : (EPT == 4 ? 256 : 1024), NL > 0 
       part[c] += sacc;
     }
   }
-  reduce_tau<KT_MAX_CTRL>(part, g, sm.red, sm.tsc + TS_V0 * g.T);
-  if (threadIdx.x < g.n_ctrl) a.partials[(size_t)k * g.n_ctrl + threadIdx.x] = sm.tsc[TS_V0 * g.T + threadIdx.x];
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned ticket = atomicAdd(a.counter, 1u);
-    sm.flag[3] = (ticket == (unsigned)(gridDim.x - 1));
-  }
-  __syncthreads();
-  if (!sm.flag[3]) return;
-  __threadfence();
-  const int chunk = ((int)gridDim.x + blockDim.x - 1) / blockDim.x;
-  const int t0 = threadIdx.x * chunk, t1 = min((int)gridDim.x, t0 + chunk);
-  for (int c = 0; c < g.n_ctrl; ++c) {
-    double v = 0.0;
-    for (int t = t0; t < t1; ++t) v += __ldcg(a.partials + (size_t)t * g.n_ctrl + c);
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sm.red[(threadIdx.x >> 5) * 8 + c] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < g.n_ctrl) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sm.red[w * 8 + threadIdx.x];
-    const double gr = -2.0 / (double)g.M * s;
-    a.grad[(size_t)threadIdx.x * a.nt + (j - 1)] = gr;
-    if (!isfinite(gr)) set_status(a.status, KT_DEV_NONFINITE);
-  }
-  if (threadIdx.x == 0) *a.counter = 0u;
+  grad_finish(g, sm, a, part);
 }
 
-template <typename R, int EPT, int NL, int ACS>
+template <typename R, int EPT>
 static cudaError_t launch_grad_t(const KtGeom &g1, int T_layout, int tel, const KtGenImage &imf,
                                  const KtGenImage &imb, const KtOps &ops, const GradArgs &a, cudaStream_t st) {
-  const cudaError_t attr = kt_allow_large_smem((const void *)grad_kernel<R, EPT, NL, ACS>);
+  const cudaError_t attr = kt_allow_large_smem((const void *)grad_kernel<R, EPT>);
   if (attr != cudaSuccess) return attr;
   const size_t smem = grad_carve(g1, sizeof(typename C2<R>::T), nullptr, nullptr, nullptr);
-  grad_kernel<R, EPT, NL, ACS><<<g1.M, g1.nthreads, smem, st>>>(g1, T_layout, tel, imf, imb, ops, a);
+  grad_kernel<R, EPT><<<g1.M, g1.nthreads, smem, st>>>(g1, T_layout, tel, imf, imb, ops, a);
+  return cudaGetLastError();
+}
+
+template <typename R, int NC, int MAXT>
+static cudaError_t launch_adj_t(const KtGeom &g1, int T_layout, int tel, const KtGenImage &imf,
+                                const KtGenImage &imb, const KtOps &ops, const GradArgs &a, cudaStream_t st) {
+  const cudaError_t attr = kt_allow_large_smem((const void *)grad_adj_kernel<R, NC, MAXT>);
+  if (attr != cudaSuccess) return attr;
+  const size_t smem = carve(g1, sizeof(typename C2<R>::T), nullptr, nullptr, false);
+  grad_adj_kernel<R, NC, MAXT><<<g1.M, g1.nthreads, smem, st>>>(g1, T_layout, tel, imf, imb, ops, a);
   return cudaGetLastError();
 }
 
 }  // namespace kt
 
-size_t kt_grad_smem_bytes(const KtGeom &g1, int elem_bytes) {
-  return kt::grad_carve(g1, elem_bytes, nullptr, nullptr, nullptr);
+size_t kt_grad_smem_bytes(const KtGeom &g1, int elem_bytes, bool reverse) {
+  return reverse ? kt::carve(g1, elem_bytes, nullptr, nullptr, false)
+                 : kt::grad_carve(g1, elem_bytes, nullptr, nullptr, nullptr);
 }
 
+// ept 4, 8: strided; -6, -9: the reverse kernel for that local dimension
 cudaError_t kt_launch_grad(int fp64, int ept, const KtGeom &g1, int T_layout, int tel, const KtGenImage &imf,
                            const KtGenImage &imb, const KtOps &ops, const GradArgs &a, cudaStream_t st) {
-  if (fp64) {
-    switch (ept) {
-      case 4: return kt::launch_grad_t<double, 4, 0, 0>(g1, T_layout, tel, imf, imb, ops, a, st);
-      case 8: return kt::launch_grad_t<double, 8, 0, 0>(g1, T_layout, tel, imf, imb, ops, a, st);
-      case -409: return kt::launch_grad_t<double, 9, 9, 4>(g1, T_layout, tel, imf, imb, ops, a, st);
-    }
-  } else {
-    switch (ept) {
-      case 4: return kt::launch_grad_t<float, 4, 0, 0>(g1, T_layout, tel, imf, imb, ops, a, st);
-      case 8: return kt::launch_grad_t<float, 8, 0, 0>(g1, T_layout, tel, imf, imb, ops, a, st);
-      case -409: return kt::launch_grad_t<float, 9, 9, 4>(g1, T_layout, tel, imf, imb, ops, a, st);
-    }
+  const bool small = g1.nthreads <= 96;
+#define ADJ(R, NC) (small ? kt::launch_adj_t<R, NC, 96>(g1, T_layout, tel, imf, imb, ops, a, st) \
+                          : kt::launch_adj_t<R, NC, 736>(g1, T_layout, tel, imf, imb, ops, a, st))
+  switch (ept) {
+    case 4: return fp64 ? kt::launch_grad_t<double, 4>(g1, T_layout, tel, imf, imb, ops, a, st)
+                        : kt::launch_grad_t<float, 4>(g1, T_layout, tel, imf, imb, ops, a, st);
+    case 8: return fp64 ? kt::launch_grad_t<double, 8>(g1, T_layout, tel, imf, imb, ops, a, st)
+                        : kt::launch_grad_t<float, 8>(g1, T_layout, tel, imf, imb, ops, a, st);
+    case -6: return fp64 ? ADJ(double, 1) : ADJ(float, 1);
+    case -9: return fp64 ? ADJ(double, 2) : ADJ(float, 2);
   }
+#undef ADJ
   return cudaErrorInvalidValue;
 }

@@ -270,7 +270,7 @@ kt_status kt_fail(kt_status s, const char *msg) { return fail(s, "%s", msg); }
 struct kt_problem {
   KtGeom g{};
   int fp64 = 1, ept = 4, cross = 0, density = 0, items_reported = 0;
-  bool cavity_ri = false;
+  bool grad_reverse = false;
   size_t esz = 16;
   // trajectory sharding: this problem holds trajectories [traj_offset, traj_offset + M) of M_total,
   // tiles [tile_off, tile_off + n_tiles) of n_tiles_total; the per-interval update sums the tile
@@ -330,7 +330,8 @@ struct kt_problem {
   int Kg = 0, grad_ept = 4;
   KtGeom g1{};                  // the geometry re-cut to one trajectory per CTA
   void *psi_ck = nullptr;       // [nt/Kg + 1] states: psi(t_{s Kg}), s >= 1 (s = 0 is psi_init)
-  void *psi_seg = nullptr;      // [Kg] replayed states of one segment
+  void *psi_seg = nullptr;      // [Kg] replayed states of one segment (Kg = nt: written by the forward sweep itself)
+  void *yscratch = nullptr;     // reverse kernel: the terms of every trajectory's forward series
   void *chi_run[2] = {nullptr, nullptr};
   double *gpart = nullptr, *dgrad = nullptr;
   int *fcursor = nullptr;
@@ -598,8 +599,10 @@ kt_status fwd_step(kt_problem *p, int update, cudaStream_t st, bool save_psi, Fw
       (s = recompute_segment(p, seg_a, seg_end(p, seg_a), st)) != KT_OK)
     return s;
   a.j = j;
-  a.psi_in = (j == 1) ? p->psi_init : p->psi[(j - 1) & 1];
-  a.psi_out = p->psi[j & 1];
+  // a sweep that keeps every state for the gradient writes psi(t_j) to its place
+  const bool direct = save_psi && p->Kg == p->nt;
+  a.psi_in = (j == 1) ? p->psi_init : direct ? state_slot(p, p->psi_seg, j - 2) : p->psi[(j - 1) & 1];
+  a.psi_out = direct && j < p->nt ? state_slot(p, p->psi_seg, j - 1) : p->psi[j & 1];
   a.chi_t = (update && j < p->nt) ? chi_at(p, j, seg_a) : nullptr;
   if ((s = prof_begin(p, KT_PROF_FWD, st)) != KT_OK) return s;
   KT_CUDA(kt_launch_fwd(p->fp64, p->ept, p->g, p->im_fwd, p->ops, a, st));
@@ -699,21 +702,24 @@ kt_status grad_setup(kt_problem *p, cudaStream_t st) {
   g1.M_pad = p->M;
   g1.tile_elems = (g1.d + 3) / 4 * 4;
   g1.prefetch_chi = 0;
-  // cavity structure with real / imaginary coupling classes, n_loc = 9, up to 96 fibers (the
-  // compiled block size): one thread per last-node fiber; otherwise 4 items per thread up to 256
-  // threads, else 8 up to 1024
-  int ept;
-  if (p->cavity_ri && g1.n_loc == 9 && g1.d / 9 <= 96) {
-    ept = -409;
-    g1.nthreads = std::max(32, (g1.d / 9 + 31) / 32 * 32);
-  } else {
-    ept = (g1.d + 3) / 4 <= 256 ? 4 : 8;
-    if ((g1.d + ept - 1) / ept > 1024) return fail(KT_ERR_UNSUPPORTED, "dimension too large for the gradient kernel");
-    g1.nthreads = std::max(32, ((g1.d + ept - 1) / ept + 31) / 32 * 32);
+  // cavity structure with real / imaginary coupling classes and drive controls: the reverse kernel, one thread per
+  // last-node fiber, its series' terms in global memory; otherwise 4 items per thread up to 256 threads, else 8
+  // up to 1024
+  int ept = -g1.n_loc;
+  g1.nthreads = std::max(32, (g1.d / g1.n_loc + 31) / 32 * 32);
+  bool reverse = p->grad_reverse && g1.nthreads <= 736 && kt_grad_smem_bytes(g1, (int)p->esz, true) <= 227 * 1024;
+  KtGeom gs = g1;               // the strided kernel's geometry
+  const int epts = (g1.d + 3) / 4 <= 256 ? 4 : 8;
+  gs.nthreads = std::max(32, ((g1.d + epts - 1) / epts + 31) / 32 * 32);
+  const bool strided_fits = (g1.d + epts - 1) / epts <= 1024 && kt_grad_smem_bytes(gs, (int)p->esz, false) <= 227 * 1024;
+  if (!reverse) {
+    if ((g1.d + epts - 1) / epts > 1024) return fail(KT_ERR_UNSUPPORTED, "dimension too large for the gradient kernel");
+    if (!strided_fits)
+      return fail(KT_ERR_UNSUPPORTED, "the gradient needs four state buffers of d = %d in shared memory (%s)", g1.d,
+                  p->fp64 ? "use FP32-mixed" : "too large");
+    ept = epts;
+    g1 = gs;
   }
-  if (kt_grad_smem_bytes(g1, (int)p->esz) > 227 * 1024)
-    return fail(KT_ERR_UNSUPPORTED, "the gradient needs four state buffers of d = %d in shared memory (%s)", g1.d,
-                p->fp64 ? "use FP32-mixed" : "too large");
   p->g1 = g1;
   p->grad_ept = ept;
   // forward states kept every Kg intervals: the co-state spacing if one was given; with automatic
@@ -730,6 +736,13 @@ kt_status grad_setup(kt_problem *p, cudaStream_t st) {
   if ((s = dev_alloc(p, (void **)&p->dgrad, (size_t)p->g.n_ctrl * p->nt * sizeof(double))) != KT_OK) return s;
   if ((s = dev_alloc(p, (void **)&p->fcursor, (size_t)p->g.M_pad * sizeof(int))) != KT_OK) return s;
   KT_CUDA(cudaMemsetAsync(p->dgrad, 0, (size_t)p->g.n_ctrl * p->nt * sizeof(double), st));
+  if (reverse &&
+      (s = dev_alloc(p, &p->yscratch, (size_t)p->M * g1.K * g1.n_loc * g1.nthreads * p->esz)) != KT_OK) {
+    if (!strided_fits) return s;
+    cudaGetLastError();         // no room for the series' terms: the strided kernel needs none
+    p->g1 = gs;
+    p->grad_ept = epts;
+  }
   return KT_OK;
 }
 
@@ -760,7 +773,7 @@ kt_status gradient_sweep(kt_problem *p, cudaStream_t st) {
   ga.status = p->status;
   for (int seg_b = p->nt; seg_b > 0;) {
     const int seg_a = ((seg_b - 1) / p->Kg) * p->Kg;
-    if (seg_b - 1 > seg_a) {
+    if (seg_b - 1 > seg_a && p->Kg < p->nt) {
       KT_CUDA(kt_launch_cursor_seek_fwd(p->g, p->rec_step[prev], p->jcount[prev], seg_a + 1, p->fcursor, st));
       for (int j = seg_a + 1; j <= seg_b - 1; ++j) {
         BwdArgs b = bwd_args(p);
@@ -780,10 +793,13 @@ kt_status gradient_sweep(kt_problem *p, cudaStream_t st) {
       ga.j = j;
       ga.psi_prev = psi_at(p, j - 1, seg_a);
       ga.chi_t = p->chi_run[j & 1];
+      ga.chi_out = p->chi_run[(j - 1) & 1];
+      ga.scratch = p->yscratch;
       kt_status s = prof_begin(p, KT_PROF_GRAD, st);
       if (s != KT_OK) return s;
       KT_CUDA(kt_launch_grad(p->fp64, p->grad_ept, p->g1, p->g.T, p->g.tile_elems, p->im_fwd, p->im_bwd, p->ops, ga, st));
       if ((s = prof_end(p, st)) != KT_OK) return s;
+      if (p->grad_ept < 0) continue;   // the reverse kernel has propagated the co-state
       s = launch_bwd_step(p, j, p->chi_run[j & 1], p->chi_run[(j - 1) & 1], st);
       if (s != KT_OK) return s;
     }
@@ -1007,7 +1023,7 @@ struct HostPlan {
   KtGeom g{};
   int fp64 = 1, ept = 4, ckpt = 0, ckpt_dense = 0, cross = 0, density = 0;
   int sharded = 0, tile_off = 0, n_tiles_total = 0, M_total = 0;
-  bool cavity_ri = false;      // cavity structure with real / imaginary coupling classes
+  bool grad_reverse = false;   // cavity structure with real / imaginary coupling classes, the controls its drives
   bool sweeps = false;         // mapping whose sweeps may run as one launch
   int items_reported = 0;      // kt_info::items_per_thread
   std::vector<double> psi0;    // density: vec(rho_0) [d][2]; empty otherwise (the model's psi0 is used)
@@ -1688,7 +1704,15 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
   P.tgt.resize(d);
   for (int x = 0; x < d; ++x) P.tgt[x] = KtCplx{psi_t[x].real(), psi_t[x].imag()};
   P.density = density ? 1 : 0;
-  P.cavity_ri = ri;
+  P.grad_reverse = ri && !density;
+  for (int t = 0; t < nterm && P.grad_reverse; ++t)
+    for (int x = 0; x < nl; ++x) {
+      const size_t e = ((size_t)t * nl + x) * g.S;
+      if (P.bwd.cslot[e].re != 0.0 || P.bwd.cslot[e].im != 0.0 || P.bwd.cslot[e + 1].im != 0.0 ||
+          P.bwd.cdg[(size_t)t * nl + x].re != 0.0 || P.bwd.cdg[(size_t)t * nl + x].im != 0.0 ||
+          (g.cterm_node[t] == N - 1 && x < nl / 3 && P.bwd.cslot[e + 1].re != 0.0))
+        P.grad_reverse = false;
+    }
   P.items_reported = fiber || (row && !few && cfg->items_per_thread == 0) ? 0 : ipt > 0 ? ipt : P.ept;
   P.sweeps = !fiber && (few || g.nthreads <= 256 || cfg->items_per_thread > 0 || !row);
   g.density = P.density;
@@ -1790,7 +1814,7 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
   p->g = P.g;
   p->fp64 = P.fp64;
   p->ept = P.ept;
-  p->cavity_ri = P.cavity_ri;
+  p->grad_reverse = P.grad_reverse;
   p->items_reported = P.items_reported;
   p->cross = P.cross;
   p->density = P.density;

@@ -151,7 +151,7 @@ struct GradArgs {
   const void *psi_prev;  // tile-layout psi(t_{j-1}) of the recorded forward pass
   const void *chi_t;     // tile-layout chi~(t_j)
   const double *eps;     // [n_ctrl][nt]
-  const int *cursor;     // [M_pad] latest record with interval <= j (backward cursor, not advanced)
+  int *cursor;           // [M_pad] latest record with interval <= j (backward cursor; the reverse kernel advances it)
   const int *rec_step;
   const int *rec_ch;
   const double *rec_s;
@@ -159,10 +159,12 @@ struct GradArgs {
   double *partials;      // [M][n_ctrl]
   unsigned *counter;
   double *grad;          // [n_ctrl][nt]: dJ_T/deps of interval j written by the last CTA
+  void *chi_out;         // reverse kernel: tile-layout chi~(t_{j-1})
+  void *scratch;         // reverse kernel: [M][K][n_loc][nthreads] the forward series' terms
   int *status;
 };
 // g1: the problem geometry re-cut to one trajectory per CTA (T = 1)
-size_t kt_grad_smem_bytes(const KtGeom &g1, int elem_bytes);
+size_t kt_grad_smem_bytes(const KtGeom &g1, int elem_bytes, bool reverse);
 cudaError_t kt_launch_grad(int fp64, int ept, const KtGeom &g1, int T_layout, int tile_elems_layout,
                            const KtGenImage &im_fwd, const KtGenImage &im_bwd, const KtOps &ops, const GradArgs &a,
                            cudaStream_t st);
