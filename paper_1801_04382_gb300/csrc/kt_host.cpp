@@ -271,6 +271,8 @@ struct kt_problem {
   KtGeom g{};
   int fp64 = 1, ept = 4, cross = 0, density = 0, items_reported = 0;
   bool grad_reverse = false;
+  int dens_ctas = 0;            // density matrix on a cluster of this many CTAs (0: the interval kernels)
+  KtGeom dens_g{};              // its geometry, re-cut to one CTA's elements
   size_t esz = 16;
   // trajectory sharding: this problem holds trajectories [traj_offset, traj_offset + M) of M_total,
   // tiles [tile_off, tile_off + n_tiles) of n_tiles_total; the per-interval update sums the tile
@@ -507,6 +509,43 @@ BwdArgs bwd_args(kt_problem *p) {
   return b;
 }
 
+// Forward / backward launches of a problem: the interval kernels, or the cluster kernel of a density matrix.
+cudaError_t run_fwd(kt_problem *p, const FwdArgs &a, cudaStream_t st) {
+  if (!p->dens_ctas) return kt_launch_fwd(p->fp64, p->ept, p->g, p->im_fwd, p->ops, a, st);
+  DensArgs d{};
+  d.j = a.j;
+  d.j_last = a.sweep ? p->nt : a.j;
+  d.nt = p->nt;
+  d.update = a.update;
+  d.ctas = p->dens_ctas;
+  d.in = a.psi_in;
+  d.out = a.sweep ? a.psi_ring[p->nt & 1] : a.psi_out;
+  d.chi = a.sweep ? a.chi_slots : a.chi_t;
+  d.slot_bytes = a.sweep ? a.slot_bytes : 0;
+  d.eps_old = a.eps_old;
+  d.eps_new = a.eps_new;
+  d.deps = a.deps;
+  d.shape = a.shape;
+  d.tau = a.tau;
+  d.norm2 = a.norm2;
+  d.status = a.status;
+  return kt_launch_density(p->fp64, 0, p->dens_g, p->im_fwd, p->ops, d, st);
+}
+cudaError_t run_bwd(kt_problem *p, const BwdArgs &b, cudaStream_t st) {
+  if (!p->dens_ctas) return kt_launch_bwd(p->fp64, p->ept, p->g, p->im_bwd, p->ops, b, st);
+  DensArgs d{};
+  d.j = b.j;
+  d.j_last = b.sweep ? 1 : b.j;
+  d.nt = p->nt;
+  d.ctas = p->dens_ctas;
+  d.in = b.chi_in;
+  d.out = b.sweep ? b.chi_slots : b.chi_out;
+  d.slot_bytes = b.sweep ? b.slot_bytes : 0;
+  d.eps_old = b.eps;
+  d.status = b.status;
+  return kt_launch_density(p->fp64, 1, p->dens_g, p->im_bwd, p->ops, d, st);
+}
+
 kt_status launch_bwd_step(kt_problem *p, int j, const void *in, void *out, cudaStream_t st) {
   BwdArgs b = bwd_args(p);
   b.j = j;
@@ -514,7 +553,7 @@ kt_status launch_bwd_step(kt_problem *p, int j, const void *in, void *out, cudaS
   b.chi_out = out;
   kt_status s = prof_begin(p, KT_PROF_BWD, st);
   if (s != KT_OK) return s;
-  KT_CUDA(kt_launch_bwd(p->fp64, p->ept, p->g, p->im_bwd, p->ops, b, st));
+  KT_CUDA(run_bwd(p, b, st));
   return prof_end(p, st);
 }
 
@@ -585,7 +624,7 @@ kt_status fwd_begin(kt_problem *p, int update, cudaStream_t st, FwdArgs &a) {
     a.chi_t = ckpt_slot(p, 0);
     kt_status s = prof_begin(p, KT_PROF_FWD, st);
     if (s != KT_OK) return s;
-    KT_CUDA(kt_launch_fwd(p->fp64, p->ept, p->g, p->im_fwd, p->ops, a, st));
+    KT_CUDA(run_fwd(p, a, st));
     if ((s = prof_end(p, st)) != KT_OK) return s;
   }
   return KT_OK;
@@ -605,7 +644,7 @@ kt_status fwd_step(kt_problem *p, int update, cudaStream_t st, bool save_psi, Fw
   a.psi_out = direct && j < p->nt ? state_slot(p, p->psi_seg, j - 1) : p->psi[j & 1];
   a.chi_t = (update && j < p->nt) ? chi_at(p, j, seg_a) : nullptr;
   if ((s = prof_begin(p, KT_PROF_FWD, st)) != KT_OK) return s;
-  KT_CUDA(kt_launch_fwd(p->fp64, p->ept, p->g, p->im_fwd, p->ops, a, st));
+  KT_CUDA(run_fwd(p, a, st));
   if ((s = prof_end(p, st)) != KT_OK) return s;
   if (update && p->cross && j < p->nt && (s = launch_cross(p, j, p->psi[j & 1], chi_at(p, j, seg_a), st)) != KT_OK)
     return s;
@@ -651,7 +690,7 @@ kt_status enqueue_forward(kt_problem *p, int update, cudaStream_t st, bool save_
     }
     kt_status s = prof_begin(p, KT_PROF_FWD, st);
     if (s != KT_OK) return s;
-    KT_CUDA(kt_launch_fwd(p->fp64, p->ept, p->g, p->im_fwd, p->ops, a, st));
+    KT_CUDA(run_fwd(p, a, st));
     return prof_end(p, st);
   }
   FwdArgs a;
@@ -826,7 +865,7 @@ kt_status enqueue_backward(kt_problem *p, cudaStream_t st) {
     b.slot_bytes = p->state_bytes;
     kt_status s = prof_begin(p, KT_PROF_BWD, st);
     if (s != KT_OK) return s;
-    KT_CUDA(kt_launch_bwd(p->fp64, p->ept, p->g, p->im_bwd, p->ops, b, st));
+    KT_CUDA(run_bwd(p, b, st));
     return prof_end(p, st);
   }
   const void *in = chiT;
@@ -1024,6 +1063,7 @@ struct HostPlan {
   int fp64 = 1, ept = 4, ckpt = 0, ckpt_dense = 0, cross = 0, density = 0;
   int sharded = 0, tile_off = 0, n_tiles_total = 0, M_total = 0;
   bool grad_reverse = false;   // cavity structure with real / imaginary coupling classes, the controls its drives
+  int dens_ctas = 0;
   bool sweeps = false;         // mapping whose sweeps may run as one launch
   int items_reported = 0;      // kt_info::items_per_thread
   std::vector<double> psi0;    // density: vec(rho_0) [d][2]; empty otherwise (the model's psi0 is used)
@@ -1461,7 +1501,11 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
   const bool row = N <= 3 && npair <= 3 && S <= 2 && (long long)d * std::max(1, cfg->tile_traj) <= row_max && (N <= 2 || d <= 256) &&
                    (autom || cfg->items_per_thread == 1) &&
                    (ri || ri_classes(gf, gb, lo_val, ra_val, cols, false));
-  if (ri || row) S = 2;
+  // density matrix of two nodes: the cluster kernel (real / imaginary classes, two slots per node row, at most six pair terms,
+  // one element per thread of at most eight CTAs)
+  const bool cluster = density && N == 4 && npair <= 6 && S <= 2 && d > 736 && d <= 8 * 832 && !cfg->inject_copy_timeout &&
+                       (ri || ri_classes(gf, gb, lo_val, ra_val, cols, false));
+  if (ri || row || cluster) S = 2;
   const bool small = few && autom;
   const int ipt = cfg->items_per_thread > 0 ? cfg->items_per_thread : (small || row ? 1 : 0);
   const bool fiber = (nl == 6 || nl == 9) && ipt == 0;
@@ -1714,7 +1758,9 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
         P.grad_reverse = false;
     }
   P.items_reported = fiber || (row && !few && cfg->items_per_thread == 0) ? 0 : ipt > 0 ? ipt : P.ept;
-  P.sweeps = !fiber && (few || g.nthreads <= 256 || cfg->items_per_thread > 0 || !row);
+  if (cluster)
+    for (P.dens_ctas = 1; P.dens_ctas < 8 && P.dens_ctas * 416 < d;) P.dens_ctas *= 2;
+  P.sweeps = cluster || (!fiber && (few || g.nthreads <= 256 || cfg->items_per_thread > 0 || !row));
   g.density = P.density;
   if (density) {
     P.psi0.resize((size_t)2 * d);
@@ -1815,6 +1861,12 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
   p->fp64 = P.fp64;
   p->ept = P.ept;
   p->grad_reverse = P.grad_reverse;
+  p->dens_ctas = P.dens_ctas;
+  p->dens_g = P.g;
+  if (P.dens_ctas) {
+    p->dens_g.tile_elems = (P.g.d + P.dens_ctas - 1) / P.dens_ctas;
+    p->dens_g.nthreads = (p->dens_g.tile_elems + 31) / 32 * 32;
+  }
   p->items_reported = P.items_reported;
   p->cross = P.cross;
   p->density = P.density;
@@ -1918,7 +1970,8 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
     if (!cfg->per_interval_launches && P.sweeps && p->ckpt == 0 && !p->sharded && !p->cross &&
         cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        kt_fwd_blocks_per_sm(p->fp64, p->ept, g, &per) == cudaSuccess && (long long)per * sms >= g.n_tiles) {
+        (p->dens_ctas > 0 ||
+         (kt_fwd_blocks_per_sm(p->fp64, p->ept, g, &per) == cudaSuccess && (long long)per * sms >= g.n_tiles))) {
       TRY(dev_alloc(p, (void **)&p->wpart, (size_t)nt * g.n_tiles * nc * sizeof(double)));
       p->whole_sweep = 1;
     }

@@ -84,6 +84,25 @@ struct BwdArgs {
   size_t slot_bytes;
 };
 
+// Density-matrix state of two nodes on a cluster of `ctas` CTAs (kt_density.cu), in the geometry re-cut to
+// tile_elems elements and nthreads threads per CTA.  Forward: intervals j .. j_last (j = 0: the overlap at t_0 first),
+// out = psi(t_{j_last}), co-states chi(t_j) at chi + j * slot_bytes; backward: intervals j down to j_last, chi(t_{j-1}) to
+// out + (j-1) * slot_bytes.  slot_bytes = 0 with j = j_last: one interval with its own pointers.
+struct DensArgs {
+  int j, j_last, nt, update, ctas;
+  const void *in, *chi;
+  void *out;
+  size_t slot_bytes;
+  const double *eps_old;
+  double *eps_new, *deps;
+  const double *shape;
+  KtCplx *tau;
+  double *norm2;
+  int *status;
+};
+cudaError_t kt_launch_density(int fp64, int backward, const KtGeom &g, const KtGenImage &im, const KtOps &ops,
+                              const DensArgs &a, cudaStream_t st);
+
 #include "../../include/krotov_traj.h"
 
 // Record msg as the calling thread's last error (krotov_last_error) and return s.
