@@ -89,6 +89,9 @@ __global__ void __launch_bounds__(832) density_kernel(KtGeom g, KtGenImage im, K
 #pragma unroll
     for (int e = 0; e < DSLOTS; ++e) row.w[e] = (R)0;
   }
+  unsigned any = 0;
+#pragma unroll
+  for (int e = 0; e < DSLOTS; ++e) any |= (__any_sync(0xffffffffu, adr[e] != 0) ? 1u : 0u) << e;
   C cur = ok ? ((const C *)a.in)[x] : mkc((R)0, (R)0);
   if (ok) A[threadIdx.x] = cur;
   const R *cf = (const R *)sm.coef;
@@ -122,27 +125,30 @@ __global__ void __launch_bounds__(832) density_kernel(KtGeom g, KtGenImage im, K
       C prev = mkc((R)0, (R)0), acc = mkc(cf[0] * cur.x, cf[0] * cur.y);
       uint32_t src = 0;
       C *dst = B;
+      C s = diag_init(D, cur, prev);   // of the next term, formed before the barrier
       for (int k = 1; k < g.K; ++k) {
         if (ok) {
           C v[DSLOTS];
 #pragma unroll
           for (int e = 0; e < DSLOTS; ++e) v[e] = ld_cluster(adr[e], src, (C *)nullptr);
-          C s = diag_init(D, cur, prev), z = mkc((R)0, (R)0);
+          C z = mkc((R)0, (R)0);
 #pragma unroll
-          for (int e = 0; e < 2 * DNN; e += 2) {
-            s = ifma(row.w[e], v[e], s);
-            z = rfma(row.w[e + 1], v[e + 1], z);
+          for (int e = 0; e < DSLOTS; ++e) {
+            if (sizeof(R) == 8 && !(any >> e & 1)) continue;   // FP64: an FMA that no lane of the warp needs
+            C &t = sizeof(R) == 4 && (e >= 2 * DNN || e % 2) ? z : s;
+            t = (e < 2 * DNN && e % 2 == 0) ? ifma(row.w[e], v[e], t) : rfma(row.w[e], v[e], t);
           }
-#pragma unroll
-          for (int e = 2 * DNN; e < DSLOTS; ++e) z = rfma(row.w[e], v[e], z);
-          s.x += z.x;
-          s.y += z.y;
+          if (sizeof(R) == 4) {
+            s.x += z.x;
+            s.y += z.y;
+          }
           s = diag_done(D, cur, prev, s);
           if (k == 1) s = mkc((R)0.5 * s.x, (R)0.5 * s.y);
+          dst[threadIdx.x] = s;
           prev = cur;
           cur = s;
-          dst[threadIdx.x] = s;
-          acc = rfma(cf[k], s, acc);
+          acc = rfma(cf[k], cur, acc);
+          s = diag_init(D, cur, prev);
         }
         cluster_sync();
         src = shift - src;

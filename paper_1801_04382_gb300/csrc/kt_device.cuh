@@ -300,7 +300,7 @@ __device__ __forceinline__ void reduce_tau(double (&v)[NV], const KtGeom &g, dou
 // --------------------------------------------------------------------------------------
 // Diagonal of B: re + i (hi + lo), lo only in FP32 (kt_split).  diag_init starts a row's sum, diag_done
 // adds y_{k-1} and the diagonal: in FP32 the smallest terms come first and only the last two additions
-// round at the size of the result.  lo turns an element by r s lo / 2 ~ 1e-7 over a series: apply_phase turns the
+// round at the size of the result; in FP64 they come first, off the path from the neighbours' loads to the result.  lo turns an element by r s lo / 2 ~ 1e-7 over a series: apply_phase turns the
 // result by it once (what the order of that turn and the couplings leaves out is a hundred times smaller).
 template <typename R> struct Diag { R re, hi, lo; };
 
@@ -325,18 +325,15 @@ __device__ __forceinline__ void keep_in_loop(Diag<float> &D) { asm volatile("" :
 __device__ __forceinline__ void keep_in_loop(Diag<double> &D) { asm volatile("" : "+d"(D.re), "+d"(D.hi)); }
 template <typename R, typename C> __device__ __forceinline__ C diag_init(Diag<R> D, C v, C old) {
   if constexpr (sizeof(R) == 4) return mkc(D.re * v.x, D.re * v.y);
-  else return old;
+  else return mkc(fma(-D.hi, v.y, fma(D.re, v.x, old.x)), fma(D.hi, v.x, fma(D.re, v.y, old.y)));
 }
 template <typename R, typename C> __device__ __forceinline__ C diag_done(Diag<R> D, C v, C old, C s) {
   if constexpr (sizeof(R) == 4) {
     s.x += old.x;
     s.y += old.y;
-  } else {
-    s.x = fma(D.re, v.x, s.x);
-    s.y = fma(D.re, v.y, s.y);
+    s.x = fma(-D.hi, v.y, s.x);
+    s.y = fma(D.hi, v.x, s.y);
   }
-  s.x = fma(-D.hi, v.y, s.x);
-  s.y = fma(D.hi, v.x, s.y);
   return s;
 }
 
@@ -1380,30 +1377,45 @@ __device__ void cheb_run_row(const KtGeom &g, const KtGenImage &im, const Smem &
 #pragma unroll
     for (int e = 0; e < 2 * NN + NPR; ++e) r.off[e] = 0;
   }
+  unsigned any = 0;
+  if (sizeof(R) == 8 && NN >= 3) {
+#pragma unroll
+    for (int e = 0; e < 2 * NN + NPR; ++e) any |= (__any_sync(0xffffffffu, r.off[e] != 0) ? 1u : 0u) << e;
+  }
   const R c0 = cf[tau];
   acc[0] = mkc(c0 * cur.x, c0 * cur.y);
   R a = K > 1 ? cf[g.T + tau] : (R)0;
+  C s = diag_init(D, cur, prev);   // of the next term: formed before the barrier, from the thread's own values
   for (int k = 1; k < K; ++k) {
     if (ok) {
       C v[2 * NN + NPR];
 #pragma unroll
       for (int e = 0; e < 2 * NN + NPR; ++e) v[e] = ld_if(Q + item, r.off[e]);
-      C s = diag_init(D, cur, prev), z = mkc((R)0, (R)0);   // two chains: an FP64 FMA's latency is what a term waits for
+      if constexpr (sizeof(R) == 4) {
+        C z = mkc((R)0, (R)0);   // two chains, for latency
 #pragma unroll
-      for (int e = 0; e < 2 * NN; e += 2) {
-        s = ifma(r.w[e], v[e], s);
-        z = rfma(r.w[e + 1], v[e + 1], z);
+        for (int e = 0; e < 2 * NN; e += 2) {
+          s = ifma(r.w[e], v[e], s);
+          z = rfma(r.w[e + 1], v[e + 1], z);
+        }
+#pragma unroll
+        for (int e = 2 * NN; e < 2 * NN + NPR; ++e) z = rfma(r.w[e], v[e], z);
+        s.x += z.x;
+        s.y += z.y;
+      } else {
+        // FP64: an FMA takes a warp 64 cycles of its scheduler's share of the FP64 unit, so the count decides; with three
+        // nodes most warps have slots that no lane needs
+#pragma unroll
+        for (int e = 0; e < 2 * NN + NPR; ++e)
+          if (NN < 3 || (any >> e & 1)) s = (e < 2 * NN && e % 2 == 0) ? ifma(r.w[e], v[e], s) : rfma(r.w[e], v[e], s);
       }
-#pragma unroll
-      for (int e = 2 * NN; e < 2 * NN + NPR; ++e) z = rfma(r.w[e], v[e], z);
-      s.x += z.x;
-      s.y += z.y;
       s = diag_done(D, cur, prev, s);
       if (k == 1) s = mkc((R)0.5 * s.x, (R)0.5 * s.y);
+      P[item] = s;
       prev = cur;
       cur = s;
-      P[item] = s;
-      acc[0] = rfma(a, s, acc[0]);
+      acc[0] = rfma(a, cur, acc[0]);
+      s = diag_init(D, cur, prev);
     }
     a = k + 1 < K ? cf[(k + 1) * g.T + tau] : (R)0;
     __syncthreads();

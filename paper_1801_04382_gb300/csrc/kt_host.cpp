@@ -1498,7 +1498,7 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
   const bool few = (nl == 6 || nl == 9) && d / nl < 16;
   const bool autom = cfg->items_per_thread == 0 && (cfg->tile_traj <= 0 || (density && few));
   const int row_max = N <= 2 && npair <= 1 ? (cfg->prec == KT_FP64 ? 512 : 1024) : 736;   // its launch bounds
-  const bool row = N <= 3 && npair <= 3 && S <= 2 && (long long)d * std::max(1, cfg->tile_traj) <= row_max && (N <= 2 || d <= 256) &&
+  const bool row = N <= 3 && npair <= 3 && S <= 2 && (long long)d * std::max(1, cfg->tile_traj) <= row_max && (N <= 2 || d <= 256 || cfg->prec == KT_FP64) &&
                    (autom || cfg->items_per_thread == 1) &&
                    (ri || ri_classes(gf, gb, lo_val, ra_val, cols, false));
   // density matrix of two nodes: the cluster kernel (real / imaginary classes, two slots per node row, at most six pair terms,
