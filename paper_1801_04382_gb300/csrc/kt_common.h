@@ -119,6 +119,7 @@ struct KtGenImage {
   const double *cheb_full;    // [sets][K] full-step coefficients lambda_s (2 - delta_k0) J_k(r dt)
   const KtCplx *phase_full;   // [sets] exp(-i c dt) / lambda_s
   int sets;                   // interval j takes set j % sets (a power of two)
+  int quick_pulse;            // each node carries at most one control term and no control touches a diagonal
   const KtCplx *pair_coef;    // [P] coefficient of pair term p (value = coef * a^dag a entries)
   int pair_dst[KT_MAX_PAIRS]; // node raised by pair term p of this direction
   int pair_src[KT_MAX_PAIRS]; // node lowered by pair term p of this direction

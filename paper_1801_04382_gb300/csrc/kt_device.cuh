@@ -747,6 +747,79 @@ __device__ void uniform_coefs(const KtGeom &g, const Smem &sm, const KtGenImage 
     store_phase<R>(g, sm, t, im.phase_full[set].re, im.phase_full[set].im, g.dt);
 }
 
+// What a whole sweep keeps from interval to interval: its thread's entry of the node factors with the control term on
+// it, and (tile width 1) the coefficient sets, behind the carve.  Rebuilding the tables from global memory, with the
+// last node's dense factor and the two-float diagonal that the small problems' mappings do not use or that no control
+// changes, and loading the coefficients again took a third of a d = 81 interval.
+struct SweepKeep {
+  double base_re, base_im, slot_re, slot_im;
+  int ctrl;          // control of this thread's entry, -1: none (or no entry)
+  bool quick, sets;
+};
+
+__host__ __device__ inline size_t sweep_keep_bytes(const KtGeom &g, int esz, int sets) {
+  return g.T == 1 ? (size_t)esz / 2 * (((size_t)sets * g.K + 7) / 8 * 8) + (size_t)esz * 3 * sets : 0;
+}
+
+template <typename R>
+__device__ __forceinline__ void sweep_keep_init(const KtGeom &g, const KtGenImage &im, char *extra, SweepKeep &kp) {
+  typedef typename C2<R>::T C;
+  const int nls = g.n_loc * g.S, e = threadIdx.x;
+  kp.quick = im.quick_pulse && g.n_nodes * nls <= (int)blockDim.x;
+  kp.sets = g.T == 1;
+  kp.ctrl = -1;
+  if (kp.quick && e < g.n_nodes * nls) {
+    const int i = e / nls, rem = e % nls;
+    kp.base_re = im.loc_base[e].re;
+    kp.base_im = im.loc_base[e].im;
+    for (int t = 0; t < g.n_cterms; ++t)
+      if (g.cterm_node[t] == i) {
+        kp.slot_re = im.ctrl_slot[t * nls + rem].re;
+        kp.slot_im = im.ctrl_slot[t * nls + rem].im;
+        if (kp.slot_re != 0.0 || kp.slot_im != 0.0) kp.ctrl = g.cterm_ctrl[t];
+      }
+  }
+  if (kp.sets) {
+    R *cf = (R *)extra;
+    C *ph = (C *)(cf + (im.sets * g.K + 7) / 8 * 8);
+    for (int q = threadIdx.x; q < im.sets * g.K; q += blockDim.x) cf[q] = (R)im.cheb_full[q];
+    for (int q = threadIdx.x; q < im.sets; q += blockDim.x) {
+      Smem t;
+      t.phase = ph + 3 * q;
+      store_phase<R>(g, t, 0, im.phase_full[q].re, im.phase_full[q].im, g.dt);
+    }
+  }
+}
+
+// Tables of the next interval (sm.eps is synchronised; a barrier must follow before they are read).
+template <typename R>
+__device__ __forceinline__ void sweep_tables(const KtGeom &g, const KtGenImage &im, const KtOps &ops, const Smem &sm,
+                                             const SweepKeep &kp) {
+  typedef typename C2<R>::T C;
+  if (!kp.quick) {
+    build_tables<R>(g, im, ops, sm, sm.eps, false, true);
+  } else if (kp.ctrl >= 0) {
+    const double e = sm.eps[kp.ctrl];
+    ((C *)sm.loc_val)[threadIdx.x] = mkc((R)(kp.base_re + e * kp.slot_re), (R)(kp.base_im + e * kp.slot_im));
+  }
+}
+
+// Full-step coefficients and phase of interval j: the kept set, or loaded into the carve's own (coef0, phase0).
+template <typename R>
+__device__ __forceinline__ void sweep_coefs(const KtGeom &g, const KtGenImage &im, Smem &sm, const SweepKeep &kp, char *extra,
+                                            int j, void *coef0, void *phase0) {
+  typedef typename C2<R>::T C;
+  sm.coef = coef0;
+  sm.phase = phase0;
+  if (kp.sets) {
+    const int set = j & (im.sets - 1);
+    sm.coef = (R *)extra + set * g.K;
+    sm.phase = (C *)((R *)extra + (im.sets * g.K + 7) / 8 * 8) + 3 * set;
+  } else {
+    uniform_coefs<R>(g, sm, im, j);
+  }
+}
+
 template <typename R, int EPT, class IT>
 __device__ __forceinline__ void load_tile(const KtGeom &g, const IT &it, const typename C2<R>::T *src,
                                           typename C2<R>::T *dst) {
@@ -1506,7 +1579,8 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
   // a compile-time switch, so that the per-interval kernels carry none of the sweep's state.
   constexpr bool sweep = SWEEP;
   const bool persist = !sweep && g.fwd_grid > 0;
-  carve(g, sizeof(C), smem_raw, &sm, g.prefetch_chi != 0, persist);
+  char *const extra = smem_raw + carve(g, sizeof(C), smem_raw, &sm, g.prefetch_chi != 0, persist);
+  void *const coef0 = sm.coef, *const phase0 = sm.phase;
   const int tau = threadIdx.x % g.T;
   // error allowed to the jump time: 2^-50 dt in FP64 (near the rounding of the FP64 norm that decides it),
   // 2^-32 dt in FP32-mixed (far below the FP32 norm's own error)
@@ -1545,13 +1619,18 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
   build_tables<R>(g, im, ops, sm, sm.eps, a.overlap != 0);
   Items<EPT, NL> it;
   load_items<EPT, NL>(g, ops, it);
+  SweepKeep keep;
+  if constexpr (SWEEP) sweep_keep_init<R>(g, im, extra, keep);
   bool store_pending = false;
   unsigned nchi = 0;        // chi loads waited for on barrier [1] (the n-th completes phase n & 1)
   C acc[EPT];
+  double eps_ahead = 0.0;   // guess sweep: the next interval's pulse, read an interval ahead
   for (;; ++j) {            // intervals: one unless sweep
     const bool need_chi = a.overlap && j < a.nt;
     // sweep: the update's pulse-independent factors for the finisher, read now, off its critical path
     // (the per-interval kernels read them in the finisher: registers held across the tiles spill there)
+    const double eps_next = eps_ahead;
+    if (sweep && !a.update && j < a.nt && threadIdx.x < g.n_ctrl) eps_ahead = a.eps_old[threadIdx.x * a.nt + j];
     double fin_scale = 0.0, fin_eold = 0.0;
     if (sweep && need_chi && threadIdx.x < g.n_ctrl) {
       const size_t idx = (size_t)threadIdx.x * a.nt + j;   // interval j+1 (0-based index j)
@@ -1562,12 +1641,12 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
       // sweep: the next interval.  Its pulse is in sm.eps (guess sweep: eps_old; updating: the value
       // the barrier's finisher formed), its chi goes to the third buffer once every thread is done
       // with the previous one, and the tables are rebuilt for the new pulse.
-      if (!a.update && threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = a.eps_old[threadIdx.x * a.nt + (j - 1)];
+      if (!a.update && threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = eps_next;
       fence_proxy_async_smem();
       __syncthreads();
       if (threadIdx.x == 0 && need_chi && g.prefetch_chi)
         bulk_load(sm.bufC, chi_of(j, blockIdx.x), tile_bytes, &sm.mbar[1]);
-      build_tables<R>(g, im, ops, sm, sm.eps, a.overlap != 0, true);
+      if constexpr (SWEEP) sweep_tables<R>(g, im, ops, sm, keep);
     }
     int tile = blockIdx.x;
     for (int use = 0; tile < g.n_tiles; tile += gridDim.x, ++use) {
@@ -1588,8 +1667,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
         // sweep: psi(t_{j-1}) is the previous interval's result, still in registers
     #pragma unroll
         for (int q = 0; q < EPT; ++q)
-          if (it.ok(q)) A[it.item(q)] = acc[q];
-        __syncthreads();
+          if (it.ok(q)) A[it.item(q)] = acc[q];   // synchronised before the series
       } else if (!tile_wait((use & 1) ? &sm.mbar[3] : &sm.mbar[0], (use >> 1) & 1, &sm.flag[4], a.status,
                             g.inject_timeout ? &sm.mbar[2] : nullptr)) {
         // psi of this tile: load number `use`, barrier [0] / [3] in turn, phase parity (use >> 1) & 1
@@ -1646,8 +1724,11 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
             if (sm.flag[1] == 0) phase = PH_SSTAR;
           }
           if (phase == PH_MAIN) {
-            uniform_coefs<R>(g, sm, im, j);
+            if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, keep, extra, j, coef0, phase0);
+            else uniform_coefs<R>(g, sm, im, j);
           } else {
+            sm.coef = coef0;
+            sm.phase = phase0;
             if (threadIdx.x < g.T) {
               const int t = threadIdx.x;
               const bool act = sm.tin[TI_ACT * g.T + t] != 0;
@@ -2169,7 +2250,8 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
   Smem sm;
   constexpr bool sweep = SWEEP;   // a.sweep, compiled in
   const bool persist = !sweep && g.bwd_grid > 0;
-  carve(g, sizeof(C), smem_raw, &sm, persist);
+  char *const extra = smem_raw + carve(g, sizeof(C), smem_raw, &sm, persist);
+  void *const coef0 = sm.coef, *const phase0 = sm.phase;
   const int tau = threadIdx.x % g.T;
   const int j_first = a.j, j_last = sweep ? 1 : a.j;
   if (threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = a.eps[threadIdx.x * a.nt + (j_first - 1)];
@@ -2189,6 +2271,10 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
   const bool fw = a.forward_replay != 0;
   Items<EPT, NL> it;
   load_items<EPT, NL>(g, ops, it);
+  SweepKeep keep;
+  if constexpr (SWEEP) sweep_keep_init<R>(g, im, extra, keep);
+  int cur = -1, cur_step = 0;      // the trajectory's latest unprocessed record (forward replay: the next) and its interval
+  double eps_ahead = 0.0;          // sweep: the next interval's pulse
   bool store_pending = false;
   for (int use = 0; tile < g.n_tiles; tile += gridDim.x, ++use) {
     // this tile's input: load number `use`, on barrier use & 1 with phase parity (use >> 1) & 1
@@ -2201,55 +2287,58 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
     if (persist && next < g.n_tiles && threadIdx.x == 0)   // the third buffer is free: prefetch the next input
       bulk_load(sm.bufC, (const C *)a.chi_in + (size_t)next * g.tile_elems, tile_bytes, &sm.mbar[(use + 1) & 1]);
     for (int j = j_first; j >= j_last; --j) {
-      if (j != j_first) {
-        // whole sweep: the pulse and the tables of the next interval (every read of the previous
-        // interval's tables ended at the barrier after its store)
-        if (threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = a.eps[threadIdx.x * a.nt + (j - 1)];
-        __syncthreads();
-        build_tables<R>(g, im, ops, sm, sm.eps, false, true);
-      }
       C *chi_out = sweep ? (C *)((char *)a.chi_slots + (size_t)(j - 1) * a.slot_bytes) + (size_t)tile * g.tile_elems
                          : (C *)a.chi_out + (size_t)tile * g.tile_elems;
+      if (sweep && threadIdx.x < g.n_ctrl) {
+        if (j != j_first) sm.eps[threadIdx.x] = eps_ahead;
+        if (j > 1) eps_ahead = a.eps[threadIdx.x * a.nt + (j - 2)];
+      }
       if (threadIdx.x == 0) sm.flag[0] = 0;
       if (threadIdx.x == 0 && store_pending) bulk_store_wait();   // A still feeds the previous tile's store
       store_pending = false;
-      __syncthreads();
+      int nj = 0;
       if (threadIdx.x < g.T) {
         const int t = threadIdx.x, k = tile * g.T + t;
-        int nj = 0;
         if (k < g.M) {
-          int cur = a.cursor[k];
-          if (fw) {
-            const int cnt = a.jcount[k];
-            while (cur < cnt && a.rec_step[(size_t)k * g.max_jumps + cur] == j && nj < 12) {
-              sm.tin[(TI_J0 + nj) * g.T + t] = cur;  // ascending in time
-              ++nj;
-              ++cur;
-            }
-            if (cur < cnt && a.rec_step[(size_t)k * g.max_jumps + cur] == j) set_status(a.status, KT_DEV_RECORD_FULL);
-          } else {
-            while (cur >= 0 && a.rec_step[(size_t)k * g.max_jumps + cur] == j && nj < 12) {
-              sm.tin[(TI_J0 + nj) * g.T + t] = cur;  // descending in time
-              ++nj;
-              --cur;
-            }
-            if (cur >= 0 && a.rec_step[(size_t)k * g.max_jumps + cur] == j) set_status(a.status, KT_DEV_RECORD_FULL);
+          const int cnt = fw ? a.jcount[k] : 0;
+          auto held = [&]() { return fw ? cur < cnt : cur >= 0; };
+          if (j == j_first) {
+            cur = a.cursor[k];
+            cur_step = held() ? a.rec_step[(size_t)k * g.max_jumps + cur] : 0;
           }
-          if (a.advance_cursor) a.cursor[k] = cur;
+          while (held() && cur_step == j && nj < 12) {
+            sm.tin[(TI_J0 + nj) * g.T + t] = cur;   // forward replay ascending in time, backward descending
+            ++nj;
+            cur += fw ? 1 : -1;
+            cur_step = held() ? a.rec_step[(size_t)k * g.max_jumps + cur] : 0;
+          }
+          if (held() && cur_step == j) set_status(a.status, KT_DEV_RECORD_FULL);
+          if (a.advance_cursor && j == j_last) a.cursor[k] = cur;
         }
         sm.tin[TI_NJ * g.T + t] = nj;
-        atomicMax(&sm.flag[0], nj);
       }
-      __syncthreads();
+      // most intervals hold no jump: one barrier then says so (and covers the pulse and flag[0] above)
+      int rounds = __syncthreads_or(nj);
+      if (rounds) {
+        if (threadIdx.x < g.T) atomicMax(&sm.flag[0], nj);
+        __syncthreads();
+        rounds = sm.flag[0];
+      }
+      if constexpr (SWEEP) {
+        // the next interval's tables (every read of the previous one's ended with its series)
+        if (j != j_first) sweep_tables<R>(g, im, ops, sm, keep);
+      }
       C *A = (C *)sm.bufA;
       C *B = (C *)sm.bufB;
-      const int rounds = sm.flag[0];
       C acc[EPT];
       for (int rnd = 0; rnd <= rounds; ++rnd) {
+        sm.coef = coef0;
+        sm.phase = phase0;
         if (rounds == 0) {
-          uniform_coefs<R>(g, sm, im, j);
+          if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, keep, extra, j, coef0, phase0);
+          else uniform_coefs<R>(g, sm, im, j);
         } else if (threadIdx.x < g.T) {
-          const int t = threadIdx.x, k = tile * g.T + t, nj = sm.tin[TI_NJ * g.T + t];
+          const int t = threadIdx.x, k = tile * g.T + t;
           double len = 0.0;
           if (rnd <= nj) {
             const double *rs = a.rec_s + (size_t)k * g.max_jumps;
@@ -2265,10 +2354,12 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
           }
           tau_coefs<R>(g, sm, t, fw ? g.c_fwd : g.c_bwd, len);
         }
-        // B holds the vector to propagate
+        // B holds the vector to propagate (a sweep's later intervals start with it in A)
+        if (!sweep || j == j_first || rnd > 0) {
   #pragma unroll
-        for (int q = 0; q < EPT; ++q)
-          if (it.ok(q)) A[it.item(q)] = B[it.item(q)];
+          for (int q = 0; q < EPT; ++q)
+            if (it.ok(q)) A[it.item(q)] = B[it.item(q)];
+        }
         __syncthreads();
         cheb_dispatch<R, EPT, NL, ACS, false>(g, im, sm, it, g.K, acc);
         if (rnd == rounds) break;
@@ -2276,13 +2367,13 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
         for (int q = 0; q < EPT; ++q)
           if (it.ok(q)) A[it.item(q)] = acc[q];
         __syncthreads();
-        const int nj = sm.tin[TI_NJ * g.T + tau];
+        const int njt = sm.tin[TI_NJ * g.T + tau];
         const int k = tile * g.T + tau;
   #pragma unroll (NL > 0 ? 1 : EPT)
         for (int q = 0; q < EPT; ++q) {
           if (!it.ok(q)) continue;
           C y = A[it.item(q)];
-          if (rnd < nj) {
+          if (rnd < njt) {
             const size_t ri = (size_t)k * g.max_jumps + sm.tin[(TI_J0 + rnd) * g.T + tau];
             const C z = lind_item<R>(g, ops, a.rec_ch[ri], fw ? 0 : 1, A, it.item(q), it.dig(q));
             const R cn = (R)a.rec_c[ri];
@@ -2292,20 +2383,20 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
         }
         __syncthreads();
       }
-      // chi(t_{j-1}) of the whole tile: into A, then one bulk store (completed before A is reused)
+      // chi(t_{j-1}) of the whole tile: into A, then one bulk store (completed before A is reused); a sweep starts its
+      // next interval from A and stores from its registers, which nothing has to wait for
   #pragma unroll
       for (int q = 0; q < EPT; ++q)
-        if (it.ok(q)) A[it.item(q)] = acc[q];
-      if (sweep && j > j_last) {
-        // the next interval starts from this result (B's last reads ended at the rounds' barrier)
-  #pragma unroll
-        for (int q = 0; q < EPT; ++q)
-          if (it.ok(q)) B[it.item(q)] = acc[q];
+        if (it.ok(q)) {
+          A[it.item(q)] = acc[q];
+          if (sweep) chi_out[it.item(q)] = acc[q];
+        }
+      if (!sweep) {
+        fence_proxy_async_smem();
+        __syncthreads();
+        if (threadIdx.x == 0) bulk_store(chi_out, A, tile_bytes);
+        store_pending = true;
       }
-      fence_proxy_async_smem();
-      __syncthreads();
-      if (threadIdx.x == 0) bulk_store(chi_out, A, tile_bytes);
-      store_pending = true;
     }   // intervals
     // the prefetched input becomes this CTA's input buffer; the old one (free) the next prefetch target
     void *tmp = sm.bufB;

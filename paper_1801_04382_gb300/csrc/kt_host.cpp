@@ -1053,6 +1053,7 @@ struct HostImage {
   std::vector<KtCplx> base, cslot, dg, cdg, pval, pc;
   std::vector<double> cf;
   std::vector<KtCplx> phase;
+  int quick_pulse = 0;
   int pdst[KT_MAX_PAIRS], psrc[KT_MAX_PAIRS];
   double kd[2 * KT_MAX_NL] = {}, kc[4] = {}, kp[KT_MAX_PAIRS] = {};   // constants of the real / imaginary kernels
   double kh[5][2] = {};                                              // and of the block mapping
@@ -1654,6 +1655,13 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
         im.cdg[(size_t)t * nl + x] = KtCplx{dv.real(), dv.imag()};
       }
     }
+    im.quick_pulse = 1;
+    for (int t = 0; t < nterm; ++t)
+      for (int x = 0; x < nl; ++x)
+        if (im.cdg[(size_t)t * nl + x].re != 0.0 || im.cdg[(size_t)t * nl + x].im != 0.0) im.quick_pulse = 0;
+    for (int t = 0; t < nterm; ++t)
+      for (int u = 0; u < t; ++u)
+        if (gen.ctrl_node[t] == gen.ctrl_node[u]) im.quick_pulse = 0;
     const int nl2 = nl * nl;
     im.pc.assign((size_t)std::max(1, g.n_pairs), KtCplx{0, 0});
     im.poff.assign((size_t)g.n_pairs * nl2, 0);
@@ -1791,6 +1799,7 @@ kt_status upload_image(kt_problem *p, const HostImage &h, KtGenImage &im, cudaSt
   }
   if ((t = upload(p, (KtCplx **)&im.phase_full, h.phase.data(), h.phase.size(), st)) != KT_OK) return t;
   im.sets = (int)h.phase.size();
+  im.quick_pulse = h.quick_pulse;
   for (int q = 0; q < 2 * KT_MAX_NL; ++q) im.kd64[q] = h.kd[q];
   for (int q = 0; q < KT_MAX_NL; ++q) {
     im.kd32[3 * q] = (float)h.kd[2 * q];

@@ -116,12 +116,14 @@ size_t kt_smem_bytes(const KtGeom &g, int elem_bytes, bool with_chi_buffer, bool
 
 cudaError_t kt_launch_fwd(int fp64, int ept, const KtGeom &g, const KtGenImage &im, const KtOps &ops,
                           const FwdArgs &a, cudaStream_t st) {
-  const size_t smem = kt_smem_bytes(g, fp64 ? 16 : 8, g.prefetch_chi != 0, g.fwd_grid > 0 && !a.sweep);
+  const size_t smem = kt_smem_bytes(g, fp64 ? 16 : 8, g.prefetch_chi != 0, g.fwd_grid > 0 && !a.sweep) +
+                      (a.sweep ? kt::sweep_keep_bytes(g, fp64 ? 16 : 8, im.sets) : 0);
   return fp64 ? kt_launch_fwd_f64(ept, g, im, ops, a, smem, st) : kt_launch_fwd_f32(ept, g, im, ops, a, smem, st);
 }
 
 cudaError_t kt_fwd_blocks_per_sm(int fp64, int ept, const KtGeom &g, int *blocks) {
-  const size_t smem = kt_smem_bytes(g, fp64 ? 16 : 8, g.prefetch_chi != 0, false);
+  const size_t smem = kt_smem_bytes(g, fp64 ? 16 : 8, g.prefetch_chi != 0, false) +
+                      kt::sweep_keep_bytes(g, fp64 ? 16 : 8, fp64 ? 1 : KT_COEF_SETS);
   KtGenImage im{};
   KtOps ops{};
   FwdArgs a{};
@@ -131,7 +133,8 @@ cudaError_t kt_fwd_blocks_per_sm(int fp64, int ept, const KtGeom &g, int *blocks
 
 cudaError_t kt_launch_bwd(int fp64, int ept, const KtGeom &g, const KtGenImage &im, const KtOps &ops,
                           const BwdArgs &a, cudaStream_t st) {
-  const size_t smem = kt_smem_bytes(g, fp64 ? 16 : 8, g.bwd_grid > 0 && !a.sweep);
+  const size_t smem = kt_smem_bytes(g, fp64 ? 16 : 8, g.bwd_grid > 0 && !a.sweep) +
+                      (a.sweep ? kt::sweep_keep_bytes(g, fp64 ? 16 : 8, im.sets) : 0);
   return fp64 ? kt_launch_bwd_f64(ept, g, im, ops, a, smem, st) : kt_launch_bwd_f32(ept, g, im, ops, a, smem, st);
 }
 
