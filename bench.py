@@ -88,9 +88,9 @@ def fp32_peak_tflops(clk_mhz: float) -> float:
 def executed_flops_per_elem_term(nnz: float, ri: bool) -> float:
     """FP32 flops one element of one Chebyshev term executes: every off-diagonal coupling of the
     cavity network is purely real or purely imaginary, so the kernels apply it with two FMAs
-    (4 flops) instead of a complex multiply-add (8); the diagonal is a complex product (6), the
-    recurrence 2 T_k - T_{k-1} 4 and the running sum a complex FMA 8."""
-    return (4.0 if ri else 8.0) * (nnz - 1.0) + 6.0 + 4.0 + 8.0
+    (4 flops) instead of a complex multiply-add (8); the diagonal takes 8 (the sum of its node parts 2, real
+    part 2, imaginary part 4), the term before last 2 and the running sum with real coefficients 4."""
+    return (4.0 if ri else 8.0) * (nnz - 1.0) + 8.0 + 2.0 + 4.0
 
 
 def measured_peaks():
@@ -400,10 +400,10 @@ def run_grad(args, rank, world):
     fp32_peak = fp32_peak_tflops(clk_max)
     K = info.cheb_terms
     nnz = avg_row_nonzeros(net)
-    # per control a 2d-dimensional propagation: the state's and the derivative's recurrences, plus
-    # the control factor (one entry per row) applied to the state in every term
+    # reverse differentiation of the series: the state's recurrence, the adjoint one and, per control, a
+    # real bilinear form over the rows with a drive entry (two thirds of them, four flops) in every term
     g_ms, g_n = prof["grad"]
-    flops_grad = net.n_ctrl * K * (2 * (8.0 * nnz + 12.0) + 8.0) * wl.d * wl.M
+    flops_grad = K * (2 * (4.0 * (nnz - 1.0) + 14.0) + net.n_ctrl * 4.0 * 2.0 / 3.0) * wl.d * wl.M
     achieved = flops_grad / (g_ms / max(g_n, 1) / 1000.0) / 1e12
     per_s = world * 1000.0 / ms_step
     line = {

@@ -1,7 +1,7 @@
 // Cross-trajectory Krotov update (Eq. cross_traj_update): at the start of interval j+1,
 //   Delta eps_c = S_c / (M^2 lambda_c) sum_{k,k'} Im[<xi_k|h_c|psi_k'> <psi_k'|xi_k>],
-// all pairs of trajectories at time t_j.  The states are transposed to [x][k] (k padded to a
-// multiple of 32 with zeros), then 32 x 32 pair tiles accumulate G_kk' = <xi_k|psi_k'> and
+// all pairs of trajectories at time t_j.  32 x 32 pair tiles read the states from their tile layout (k padded to a
+// multiple of 32 with zeros), apply the control factors to psi on the way and accumulate G_kk' = <xi_k|psi_k'> and
 // A_c,kk' = <xi_k|h_c|psi_k'> over slices of x in the state precision (like every per-trajectory
 // partial sum of the FP32-mixed path), the slice sums are added in slice order, and the pair terms
 // Im[A conj(G)] -- the cross-trajectory sum -- are formed and summed in FP64 in a fixed order: per
@@ -14,63 +14,46 @@ namespace kt {
 
 constexpr int XC = 8;   // elements per staged chunk
 
-template <typename C>
-__global__ void cross_prep_kernel(KtGeom g, KtOps ops, const C *psi, const C *xi, C *X, C *P, C *HP, int Mp) {
-  typedef decltype(C().x) R;
-  const size_t n = (size_t)g.d * Mp;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(e / Mp), k = (int)(e % Mp);
-    const bool ok = k < g.M;
-    const size_t base = ok ? (size_t)(k / g.T) * g.tile_elems + (k % g.T) : 0;
-    X[e] = ok ? xi[base + (size_t)x * g.T] : mkc((R)0, (R)0);
-    P[e] = ok ? psi[base + (size_t)x * g.T] : mkc((R)0, (R)0);
-    const uint32_t dig = ops.digits[x];
-    for (int c = 0; c < g.n_ctrl; ++c) {
-      // (h_c psi_k)[x]: the control factor (unscaled) on its node, as in the update overlap
-      C h = mkc((R)0, (R)0);
-      if (ok) {
-        const int node = g.ctrl_node[c];
-        const int b = (c * g.n_loc + ((dig >> (4 * node)) & 15)) * g.SH;
-        for (int s = 0; s < g.SH; ++s) {
-          const KtCplx w = ops.hc_val[b + s];
-          if (w.re == 0.0 && w.im == 0.0) continue;
-          const int y = x + ops.hc_dl[b + s] * g.stride[node];
-          h = cfma(mkc((R)w.re, (R)w.im), psi[base + (size_t)y * g.T], h);
-        }
-      }
-      HP[(size_t)c * n + e] = h;
-    }
-  }
-}
-
 // Pair tile sums over a slice of the elements: one CTA per 32 x 32 tile of pairs and slice z
 // (blockIdx.z) of the x range, one pair per thread (k = 32 blockIdx.y + tid / 32,
 // k' = 32 blockIdx.x + tid % 32).  Writes the slice sums of G_kk' and A_c,kk' to
 // buf[tile][z][1 + n_ctrl][1024] (coalesced).
 template <typename C>
-__global__ void __launch_bounds__(1024) cross_slice_kernel(KtGeom g, CrossArgs a, int Mp, int xlen) {
+__global__ void __launch_bounds__(1024) cross_slice_kernel(KtGeom g, KtOps ops, CrossArgs a, int xlen) {
   typedef decltype(C().x) R;
-  __shared__ C sX[XC][32], sP[XC][32], sH[KT_MAX_CTRL][XC][32];
-  const C *X = (const C *)a.X, *P = (const C *)a.P, *HP = (const C *)a.HP;
+  __shared__ C sX[XC][33], sP[XC][33], sH[KT_MAX_CTRL][XC][33];
+  const C *xi = (const C *)a.xi, *psi = (const C *)a.psi;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int kb = blockIdx.y * 32, kpb = blockIdx.x * 32;
   const int nc = g.n_ctrl;
-  const size_t n = (size_t)g.d * Mp;
   const int xa = blockIdx.z * xlen, xb = min(g.d, xa + xlen);
   R G[2] = {0, 0};
   R A[KT_MAX_CTRL][2];
 #pragma unroll
   for (int c = 0; c < KT_MAX_CTRL; ++c) A[c][0] = A[c][1] = 0;
   for (int x0 = xa; x0 < xb; x0 += XC) {
-    if (threadIdx.x < XC * 32) {
-      const int xx = threadIdx.x / 32, kk = threadIdx.x % 32, x = x0 + xx;
-      const bool ok = x < xb;
-      const size_t r = (size_t)x * Mp;
-      sX[xx][kk] = ok ? X[r + kb + kk] : mkc((R)0, (R)0);
-      sP[xx][kk] = ok ? P[r + kpb + kk] : mkc((R)0, (R)0);
-#pragma unroll
-      for (int c = 0; c < KT_MAX_CTRL; ++c)
-        if (c < nc) sH[c][xx][kk] = ok ? HP[(size_t)c * n + r + kpb + kk] : mkc((R)0, (R)0);
+    // 256 threads each for xi, psi and every control factor; eight consecutive elements of four trajectories per warp
+    for (int role = threadIdx.x / (XC * 32); role < 2 + nc; role += 1024 / (XC * 32)) {
+      const int e = threadIdx.x % (XC * 32), xx = e % XC, kk = e / XC, x = x0 + xx, k = (role == 0 ? kb : kpb) + kk;
+      C v = mkc((R)0, (R)0);
+      if (x < xb && k < g.M) {
+        const C *src = (role == 0 ? xi : psi) + (size_t)(k / g.T) * g.tile_elems + (k % g.T);
+        if (role < 2) {
+          v = src[(size_t)x * g.T];
+        } else {
+          // (h_c psi_k)[x]: the control factor (unscaled) on its node, as in the update overlap
+          const int c = role - 2, node = g.ctrl_node[c];
+          const int b = (c * g.n_loc + ((ops.digits[x] >> (4 * node)) & 15)) * g.SH;
+          for (int s = 0; s < g.SH; ++s) {
+            const KtCplx w = ops.hc_val[b + s];
+            if (w.re == 0.0 && w.im == 0.0) continue;
+            v = cfma(mkc((R)w.re, (R)w.im), src[(size_t)(x + ops.hc_dl[b + s] * g.stride[node]) * g.T], v);
+          }
+        }
+      }
+      if (role == 0) sX[xx][kk] = v;
+      else if (role == 1) sP[xx][kk] = v;
+      else sH[role - 2][xx][kk] = v;
     }
     __syncthreads();
     R gr = 0, gi = 0;
@@ -176,27 +159,17 @@ __global__ void __launch_bounds__(1024) cross_final_kernel(KtGeom g, CrossArgs a
 template <typename C>
 cudaError_t launch_cross_t(const KtGeom &g, const KtOps &ops, const CrossArgs &a, cudaStream_t st) {
   const int Mp = (g.M + 31) / 32 * 32;
-  const size_t n = (size_t)g.d * Mp;
-  const int blocks = (int)std::min<size_t>((n + 255) / 256, 152 * 16);
-  cross_prep_kernel<C><<<blocks, 256, 0, st>>>(g, ops, (const C *)a.psi, (const C *)a.xi, (C *)a.X, (C *)a.P,
-                                                (C *)a.HP, Mp);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   const int nz = kt_cross_slices(g);
   const int chunks = (g.d + XC - 1) / XC;
   const int xlen = (chunks + nz - 1) / nz * XC;
-  cross_slice_kernel<C><<<dim3(Mp / 32, Mp / 32, nz), 1024, 0, st>>>(g, a, Mp, xlen);
+  cross_slice_kernel<C><<<dim3(Mp / 32, Mp / 32, nz), 1024, 0, st>>>(g, ops, a, xlen);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cross_final_kernel<C><<<dim3(Mp / 32, Mp / 32), 1024, 0, st>>>(g, a, nz);
   return cudaGetLastError();
 }
 
 }  // namespace kt
-
-size_t kt_cross_work_bytes(const KtGeom &g, int elem_bytes) {
-  const size_t Mp = (size_t)(g.M + 31) / 32 * 32;
-  return (size_t)g.d * Mp * (2 + g.n_ctrl) * elem_bytes;
-}
 
 // slices of the x range: about two CTAs per SM in all, at most one chunk of XC elements each
 int kt_cross_slices(const KtGeom &g) {

@@ -310,6 +310,7 @@ struct kt_problem {
   unsigned *counter = nullptr;
   // whole-sweep launches (kt_config.per_interval_launches): wpart = the tile partials of every interval
   int whole_sweep = 0;
+  bool whole_plain = false;     // backward sweeps and forward sweeps without update as one launch (whole_sweep, or the cross rule)
   double *wpart = nullptr;
   KtCplx *tau = nullptr;
   double *norm2 = nullptr;
@@ -319,8 +320,7 @@ struct kt_problem {
   long long passes = 0;         // completed forward sweeps since the uniforms were uploaded
   long long sweeps = 0;         // completed forward sweeps since krotov_init (never reset)
   double *nu = nullptr;         // device [KT_MAX_CTRL]: pulse noise (krotov_pulse_noise)
-  void *cwork = nullptr;        // cross-trajectory update: [x][k] states and control products
-  double *cpart = nullptr;      // its per-tile partial sums
+  double *cpart = nullptr;      // cross-trajectory update: per-tile partial sums
   double *cpair = nullptr;      // its per-slice pair sums
   unsigned *ccounter = nullptr;
   double *nu_ref = nullptr;     // device [n_ctrl][nt]: its reference pulse
@@ -579,15 +579,11 @@ const void *chi_at(const kt_problem *p, int j, int seg_a) {
 // Cross-trajectory update of interval j+1 from psi(t_j) and xi(t_j).
 kt_status launch_cross(kt_problem *p, int j, const void *psi, const void *xi, cudaStream_t st) {
   const KtGeom &g = p->g;
-  const size_t Mp = (size_t)(g.M + 31) / 32 * 32, n = (size_t)g.d * Mp;
   CrossArgs c{};
   c.j = j;
   c.nt = p->nt;
   c.psi = psi;
   c.xi = xi;
-  c.X = p->cwork;
-  c.P = (char *)p->cwork + n * p->esz;
-  c.HP = (char *)p->cwork + 2 * n * p->esz;
   c.pairbuf = p->cpair;
   c.partials = p->cpart;
   c.counter = p->ccounter;
@@ -671,7 +667,7 @@ kt_status enqueue_forward(kt_problem *p, int update, cudaStream_t st, bool save_
   if (p->sharded && !p->nccl_comm)
     return fail(KT_ERR_STATE, "a trajectory shard runs through its group (krotov_group_update) or over NCCL "
                               "(krotov_shard_nccl)");
-  if (p->whole_sweep && !save_psi) {
+  if ((update ? p->whole_sweep != 0 : p->whole_plain) && !save_psi) {
     // the whole sweep as one cooperative launch: interval 0 (the update overlap at t_0) when
     // updating, then 1 .. nt, psi(t_j) in psi[j & 1] as on the per-interval path
     KT_CUDA(kt_launch_init_pass(p->g, p->U, p->pass, p->rstate, p->jcount[p->cur], st));
@@ -854,7 +850,7 @@ kt_status enqueue_backward(kt_problem *p, cudaStream_t st) {
   // chi_k(T) = tau_k |tgt>; the cross-trajectory xi_k(T) = |tgt>; a density matrix's P(T) = P_tgt
   KT_CUDA(kt_launch_chi_boundary(p->fp64, p->g, p->ops, (p->cross || p->density) ? nullptr : p->tau, chiT, st));
   KT_CUDA(kt_launch_cursor_seek(p->g, p->rec_step[prev], p->jcount[prev], p->nt, p->cursor, st));
-  if (p->whole_sweep) {
+  if (p->whole_plain) {
     // the whole sweep as one launch: chi(t_{j-1}) of interval j into co-state slot j-1
     BwdArgs b = bwd_args(p);
     b.j = p->nt;
@@ -1956,7 +1952,6 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
   TRY(dev_alloc(p, (void **)&p->status, sizeof(int)));
   TRY(dev_alloc(p, (void **)&p->pass, 3 * sizeof(int)));
   if (p->cross && !probe) {
-    TRY(dev_alloc(p, &p->cwork, kt_cross_work_bytes(g, (int)p->esz)));
     TRY(dev_alloc(p, (void **)&p->cpart, kt_cross_partials(g) * sizeof(double)));
     TRY(dev_alloc(p, (void **)&p->cpair, kt_cross_pair_bytes(g)));
     TRY(dev_alloc(p, (void **)&p->ccounter, sizeof(unsigned)));
@@ -1973,16 +1968,19 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
     if (p->ckpt > 0) TRY(dev_alloc(p, &p->seg, p->state_bytes * (p->ckpt + 1)));
     // whole-sweep launches: the strided mapping (the small problems' mapping; the sweep kernels are
     // compiled for it only), every tile resident at once (the forward sweep's exchange of partials), every
-    // co-state kept (each interval's co-state has its slot), no exchange with other shards and no
-    // pair sums between intervals
+    // co-state kept (each interval's co-state has its slot), no exchange with other shards; the
+    // cross-trajectory rule's updating sweep keeps one launch per interval, for the pair sums in between
     int dev = 0, sms = 0, per = 0;
-    if (!cfg->per_interval_launches && P.sweeps && p->ckpt == 0 && !p->sharded && !p->cross &&
+    if (!cfg->per_interval_launches && P.sweeps && p->ckpt == 0 && !p->sharded &&
         cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         (p->dens_ctas > 0 ||
          (kt_fwd_blocks_per_sm(p->fp64, p->ept, g, &per) == cudaSuccess && (long long)per * sms >= g.n_tiles))) {
-      TRY(dev_alloc(p, (void **)&p->wpart, (size_t)nt * g.n_tiles * nc * sizeof(double)));
-      p->whole_sweep = 1;
+      p->whole_plain = true;
+      if (!p->cross) {
+        TRY(dev_alloc(p, (void **)&p->wpart, (size_t)nt * g.n_tiles * nc * sizeof(double)));
+        p->whole_sweep = 1;
+      }
     }
     cudaGetLastError();   // an occupancy query that failed leaves per-interval launches
   }

@@ -139,14 +139,12 @@ cudaError_t kt_launch_cursor_seek(const KtGeom &g, const int *rec_step, const in
 cudaError_t kt_launch_cursor_seek_fwd(const KtGeom &g, const int *rec_step, const int *jcount, int from,
                                       int *cursor, cudaStream_t st);
 // Cross-trajectory update of interval j+1 (Eq. cross_traj_update) from psi(t_j), xi(t_j) in tile
-// layout: transposes both to [x][k] (k padded to a multiple of 32), applies the control factors,
-// sums Im[<xi_k|h_c|psi_k'><psi_k'|xi_k>] over all pairs in 32 x 32 pair tiles and, in the last
+// layout: applies the control factors, sums Im[<xi_k|h_c|psi_k'><psi_k'|xi_k>] over all pairs in 32 x 32 pair tiles and, in the last
 // CTA, writes deps / eps_new of interval j+1 (0-based index j).
 struct CrossArgs {
   int j, nt;
   const void *psi;       // tile layout, t_j
   const void *xi;        // tile layout, t_j
-  void *X, *P, *HP;      // [d][Mp], [d][Mp], [n_ctrl][d][Mp] work arrays
   double *pairbuf;       // [slices][Mp][Mp][1 + n_ctrl] FP64 complex slice sums of G and A_c
   double *partials;      // [(Mp/32)^2][n_ctrl]
   unsigned *counter;
@@ -155,7 +153,6 @@ struct CrossArgs {
   const double *shape;
   int *status;
 };
-size_t kt_cross_work_bytes(const KtGeom &g, int elem_bytes);   // X + P + HP
 size_t kt_cross_partials(const KtGeom &g);                     // entries of CrossArgs::partials
 int kt_cross_slices(const KtGeom &g);                          // slices of the element range
 size_t kt_cross_pair_bytes(const KtGeom &g);                   // CrossArgs::pairbuf
