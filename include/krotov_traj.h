@@ -173,8 +173,8 @@ typedef struct {
                                one whose CTAs exchange their partial sums after each interval to form the
                                update (Sec. 2.2: the update of interval j+1 needs every trajectory's
                                state at t_j); bit-identical to the per-interval launches.  Not used for
-                               shards, the updating sweeps of the cross-trajectory rule, the sweeps that keep states
-                               for the gradient, or the problems of a batch.  1 = one launch per interval. */
+                               shards, the sweeps that keep states for the gradient, or the updating
+                               sweeps of the cross-trajectory rule and of the problems of a batch.  1 = one launch per interval. */
 } kt_config;
 
 /* Create a problem: validate, assemble H_eff in structured form (a1), choose the Chebyshev

@@ -804,17 +804,16 @@ __device__ __forceinline__ void sweep_tables(const KtGeom &g, const KtGenImage &
   }
 }
 
-// Full-step coefficients and phase of interval j: the kept set, or loaded into the carve's own (coef0, phase0).
+// Full-step coefficients and phase of interval j: the kept set (in run, the copy of sm that the series takes: sm's own
+// places stay known to the jump phases), or loaded.
 template <typename R>
-__device__ __forceinline__ void sweep_coefs(const KtGeom &g, const KtGenImage &im, Smem &sm, const SweepKeep &kp, char *extra,
-                                            int j, void *coef0, void *phase0) {
+__device__ __forceinline__ void sweep_coefs(const KtGeom &g, const KtGenImage &im, const Smem &sm, Smem &run,
+                                            const SweepKeep &kp, char *extra, int j) {
   typedef typename C2<R>::T C;
-  sm.coef = coef0;
-  sm.phase = phase0;
   if (kp.sets) {
     const int set = j & (im.sets - 1);
-    sm.coef = (R *)extra + set * g.K;
-    sm.phase = (C *)((R *)extra + (im.sets * g.K + 7) / 8 * 8) + 3 * set;
+    run.coef = (R *)extra + set * g.K;
+    run.phase = (C *)((R *)extra + (im.sets * g.K + 7) / 8 * 8) + 3 * set;
   } else {
     uniform_coefs<R>(g, sm, im, j);
   }
@@ -1580,7 +1579,6 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
   constexpr bool sweep = SWEEP;
   const bool persist = !sweep && g.fwd_grid > 0;
   char *const extra = smem_raw + carve(g, sizeof(C), smem_raw, &sm, g.prefetch_chi != 0, persist);
-  void *const coef0 = sm.coef, *const phase0 = sm.phase;
   const int tau = threadIdx.x % g.T;
   // error allowed to the jump time: 2^-50 dt in FP64 (near the rounding of the FP64 norm that decides it),
   // 2^-32 dt in FP32-mixed (far below the FP32 norm's own error)
@@ -1714,6 +1712,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
       int vstride = 8, voff = 1;
       for (;;) {
         if (phase != PH_DONE) {
+          Smem run = sm;
           // ---- choose the propagation of this round
           if (phase == PH_ROOT) {
             if (threadIdx.x == 0) sm.flag[1] = 0;
@@ -1724,11 +1723,9 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
             if (sm.flag[1] == 0) phase = PH_SSTAR;
           }
           if (phase == PH_MAIN) {
-            if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, keep, extra, j, coef0, phase0);
+            if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, run, keep, extra, j);
             else uniform_coefs<R>(g, sm, im, j);
           } else {
-            sm.coef = coef0;
-            sm.phase = phase0;
             if (threadIdx.x < g.T) {
               const int t = threadIdx.x;
               const bool act = sm.tin[TI_ACT * g.T + t] != 0;
@@ -1741,7 +1738,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
             load_tile<R, EPT>(g, it, psi_out, A);   // the main round's tile came by bulk copy
           }
           __syncthreads();
-          cheb_dispatch<R, EPT, NL, ACS, false>(g, im, sm, it, g.K, acc);
+          cheb_dispatch<R, EPT, NL, ACS, false>(g, im, run, it, g.K, acc);
         }
         if (phase == PH_MAIN || phase == PH_DONE) {
           // ---- norm of the result and update overlap at t_j, g_c = sum_k Im <chi_k|hc_c|psi_k>, in one reduction.
@@ -2251,7 +2248,6 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
   constexpr bool sweep = SWEEP;   // a.sweep, compiled in
   const bool persist = !sweep && g.bwd_grid > 0;
   char *const extra = smem_raw + carve(g, sizeof(C), smem_raw, &sm, persist);
-  void *const coef0 = sm.coef, *const phase0 = sm.phase;
   const int tau = threadIdx.x % g.T;
   const int j_first = a.j, j_last = sweep ? 1 : a.j;
   if (threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = a.eps[threadIdx.x * a.nt + (j_first - 1)];
@@ -2332,10 +2328,9 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
       C *B = (C *)sm.bufB;
       C acc[EPT];
       for (int rnd = 0; rnd <= rounds; ++rnd) {
-        sm.coef = coef0;
-        sm.phase = phase0;
+        Smem run = sm;
         if (rounds == 0) {
-          if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, keep, extra, j, coef0, phase0);
+          if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, run, keep, extra, j);
           else uniform_coefs<R>(g, sm, im, j);
         } else if (threadIdx.x < g.T) {
           const int t = threadIdx.x, k = tile * g.T + t;
@@ -2361,7 +2356,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
             if (it.ok(q)) A[it.item(q)] = B[it.item(q)];
         }
         __syncthreads();
-        cheb_dispatch<R, EPT, NL, ACS, false>(g, im, sm, it, g.K, acc);
+        cheb_dispatch<R, EPT, NL, ACS, false>(g, im, run, it, g.K, acc);
         if (rnd == rounds) break;
   #pragma unroll
         for (int q = 0; q < EPT; ++q)

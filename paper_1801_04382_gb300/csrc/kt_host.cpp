@@ -1976,11 +1976,10 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         (p->dens_ctas > 0 ||
          (kt_fwd_blocks_per_sm(p->fp64, p->ept, g, &per) == cudaSuccess && (long long)per * sms >= g.n_tiles))) {
+      // (no room for the partials of every interval: one launch per interval, which needs one interval's)
       p->whole_plain = true;
-      if (!p->cross) {
-        TRY(dev_alloc(p, (void **)&p->wpart, (size_t)nt * g.n_tiles * nc * sizeof(double)));
+      if (!p->cross && dev_alloc(p, (void **)&p->wpart, (size_t)nt * g.n_tiles * nc * sizeof(double)) == KT_OK)
         p->whole_sweep = 1;
-      }
     }
     cudaGetLastError();   // an occupancy query that failed leaves per-interval launches
   }
