@@ -118,6 +118,8 @@ struct KtGenImage {
   const KtCplx *pair_val;     // [P][n_loc*n_loc]
   const double *cheb_full;    // [sets][K] full-step coefficients lambda_s (2 - delta_k0) J_k(r dt)
   const KtCplx *phase_full;   // [sets] exp(-i c dt) / lambda_s
+  const double *piece;        // [n_piece][K] Chebyshev coefficients in u = s / dt of m_k(s), 0 <= s <= dt (pieces of an interval)
+  int n_piece;
   int sets;                   // interval j takes set j % sets (a power of two)
   int quick_pulse;            // each node carries at most one control term and no control touches a diagonal
   const KtCplx *pair_coef;    // [P] coefficient of pair term p (value = coef * a^dag a entries)

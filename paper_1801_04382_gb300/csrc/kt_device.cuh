@@ -211,7 +211,7 @@ __host__ __device__ inline size_t carve(const KtGeom &g, int esz, char *base, Sm
   char *cf = take((size_t)esz / 2 * g.K * g.T);
   char *phs = take((size_t)esz * 3 * g.T);
   char *rd = take(sizeof(double) * nwarps * g.T * 8);
-  char *ts = take(sizeof(double) * 17 * g.T);
+  char *ts = take(sizeof(double) * 18 * g.T);
   char *ti = take(sizeof(int) * 16 * g.T);
   char *ep = take(sizeof(double) * KT_MAX_CTRL);
   char *fl = take(sizeof(int) * 8);
@@ -229,7 +229,7 @@ __host__ __device__ inline size_t carve(const KtGeom &g, int esz, char *base, Sm
 }
 
 // per-trajectory scalar slots in Smem::tsc / Smem::tin
-enum { TS_R = 0, TS_LO, TS_HI, TS_S0, TS_S, TS_PS, TS_PP, TS_C, TS_LEN, TS_V0 };   // TS_V0: 8 values per trajectory
+enum { TS_R = 0, TS_LO, TS_HI, TS_S0, TS_S, TS_PS, TS_PP, TS_C, TS_LEN, TS_X, TS_V0 };   // TS_V0: 8 values per trajectory
 enum { TI_ACT = 0, TI_BUSY, TI_CH, TI_NJ, TI_J0, TI_J1, TI_J2, TI_J3, TI_J4, TI_J5, TI_J6, TI_J7,
        TI_J8, TI_J9, TI_J10, TI_J11 };
 
@@ -724,17 +724,32 @@ __device__ void cheb_run(const KtGeom &g, const KtGenImage &im, const Smem &sm, 
   apply_phase<R, EPT>(g, sm, tau, acc, [&](int q) { return it.ok(q) ? dv[q].lo : (R)0; });
 }
 
-// Coefficients of exp(-i G s) for trajectory tau (called by one thread per trajectory):
-// m_k = (2 - delta_k0) J_k(r s) and the phase exp(-i c s).
+// Coefficients of exp(-i G s) for every trajectory, s in sm.tsc[TS_X] (synchronised): m_k = (2 - delta_k0) J_k(r s) and the
+// phase exp(-i c s).  Called by the whole block, one thread per coefficient: its Chebyshev series in s / dt by Clenshaw's
+// recurrence.  (One thread running Miller's recurrence for all orders took longer than a series of a small problem in
+// FP64, where an instruction costs a warp 64 cycles however few of its lanes work: passes with several jumps per
+// trajectory at d = 81 28.5 -> 25.3 ms, d = 216 FP32 9.9 -> 8.3 ms, d = 729 FP32 26.9 -> 25.4 ms.)
 template <typename R>
-__device__ void tau_coefs(const KtGeom &g, const Smem &sm, int tau, double c_gen, double s) {
+__device__ void piece_coefs(const KtGeom &g, const KtGenImage &im, const Smem &sm, double c_gen) {
   R *cf = (R *)sm.coef;
-  double J[KT_MAX_K];
-  kt_bessel_miller(g.r * s, g.K, J);
-  double sn, cs;
-  sincos(-c_gen * s, &sn, &cs);
-  store_phase<R>(g, sm, tau, cs, sn, s);
-  for (int k = 0; k < g.K; ++k) cf[k * g.T + tau] = (R)((k == 0 ? 1.0 : 2.0) * J[k]);
+  for (int e = threadIdx.x; e < g.K * g.T; e += blockDim.x) {
+    const int k = e / g.T;
+    const double y = 2.0 * (sm.tsc[TS_X * g.T + e % g.T] / g.dt) - 1.0, y2 = 2.0 * y;
+    double b1 = 0.0, b2 = 0.0;
+    for (int j = im.n_piece - 1; j >= 1; --j) {
+      const double b = fma(y2, b1, im.piece[j * g.K + k] - b2);
+      b2 = b1;
+      b1 = b;
+    }
+    cf[e] = (R)fma(y, b1, im.piece[k] - b2);
+  }
+  const int t = blockDim.x - 1 - threadIdx.x;   // the phases on the last warp
+  if (t < g.T) {
+    const double s = sm.tsc[TS_X * g.T + t];
+    double sn, cs;
+    sincos(-c_gen * s, &sn, &cs);
+    store_phase<R>(g, sm, t, cs, sn, s);
+  }
 }
 
 template <typename R>
@@ -1733,9 +1748,11 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
               if (phase == PH_ROOT) len = act && sm.tin[TI_BUSY * g.T + t] ? sm.tsc[TS_S * g.T + t] : 0.0;
               else if (phase == PH_SSTAR) len = act ? sm.tsc[TS_HI * g.T + t] : 0.0;
               else len = act ? g.dt - sm.tsc[TS_S0 * g.T + t] : 0.0;
-              tau_coefs<R>(g, sm, t, g.c_fwd, len);
+              sm.tsc[TS_X * g.T + t] = len;
             }
             load_tile<R, EPT>(g, it, psi_out, A);   // the main round's tile came by bulk copy
+            __syncthreads();
+            piece_coefs<R>(g, im, sm, g.c_fwd);
           }
           __syncthreads();
           cheb_dispatch<R, EPT, NL, ACS, false>(g, im, run, it, g.K, acc);
@@ -2347,7 +2364,11 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
               len = hi - lo;
             }
           }
-          tau_coefs<R>(g, sm, t, fw ? g.c_fwd : g.c_bwd, len);
+          sm.tsc[TS_X * g.T + t] = len;
+        }
+        if (rounds > 0) {
+          __syncthreads();
+          piece_coefs<R>(g, im, sm, fw ? g.c_fwd : g.c_bwd);
         }
         // B holds the vector to propagate (a sweep's later intervals start with it in A)
         if (!sweep || j == j_first || rnd > 0) {

@@ -302,7 +302,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
     __syncthreads();
     for (int p = 0; p < q; ++p) {
       C acc[NL];
-      if (threadIdx.x == 0) tau_coefs<R>(g, sm, 0, g.c_fwd, sb(p + 1) - sb(p));
+      if (threadIdx.x == 0) sm.tsc[TS_X] = sb(p + 1) - sb(p);
+      __syncthreads();
+      piece_coefs<R>(g, imf, sm, g.c_fwd);
       __syncthreads();
       cheb_run_acs<R, NC, 1, true, false>(g, imf, sm, it, g.K, acc);
       if (ok) {
@@ -327,8 +329,13 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
       __syncthreads();
     }
     // ---- y_0 .. y_{K-2} of piece q, each thread's fiber to its place in ybuf
-    if (m == 0) uniform_coefs<R>(g, sm, imf, j);
-    else if (threadIdx.x == 0) tau_coefs<R>(g, sm, 0, g.c_fwd, sb(q + 1) - sb(q));
+    if (m == 0) {
+      uniform_coefs<R>(g, sm, imf, j);
+    } else {
+      if (threadIdx.x == 0) sm.tsc[TS_X] = sb(q + 1) - sb(q);
+      __syncthreads();
+      piece_coefs<R>(g, imf, sm, g.c_fwd);
+    }
     RowCache<R> rc;
     Diag<R> Df{(R)0, (R)0, (R)0};
     if (ok) {
@@ -497,7 +504,9 @@ __global__ void __launch_bounds__(EPT == 4 ? 256 : 1024)
       __syncthreads();
       for (int step = 0; step < np; ++step) {
         const int p = adj ? m - step : step;
-        if (threadIdx.x == 0) tau_coefs<R>(g, sm, 0, adj ? g.c_bwd : g.c_fwd, sb(p + 1) - sb(p));
+        if (threadIdx.x == 0) sm.tsc[TS_X] = sb(p + 1) - sb(p);
+        __syncthreads();
+        piece_coefs<R>(g, imd, sm, adj ? g.c_bwd : g.c_fwd);
         __syncthreads();
         cheb_run<R, EPT>(g, imd, sm, it, g.K, acc);
 #pragma unroll
@@ -527,14 +536,12 @@ __global__ void __launch_bounds__(EPT == 4 ? 256 : 1024)
       __syncthreads();
     }
     // ---- derivative of piece q along every control: <W_q| dP(tau_q)/deps_c |Z_q>
-    if (threadIdx.x == 0) {
-      if (m == 0) {
-        const int set = j & (imf.sets - 1);
-        for (int e = 0; e < g.K; ++e) ((R *)sm.coef)[e] = (R)imf.cheb_full[(size_t)set * g.K + e];
-        store_phase<R>(g, sm, 0, imf.phase_full[set].re, imf.phase_full[set].im, g.dt);
-      } else {
-        tau_coefs<R>(g, sm, 0, g.c_fwd, sb(q + 1) - sb(q));
-      }
+    if (m == 0) {
+      uniform_coefs<R>(g, sm, imf, j);
+    } else {
+      if (threadIdx.x == 0) sm.tsc[TS_X] = sb(q + 1) - sb(q);
+      __syncthreads();
+      piece_coefs<R>(g, imf, sm, g.c_fwd);
     }
     for (int c = 0; c < g.n_ctrl; ++c) {
 #pragma unroll
