@@ -7,6 +7,9 @@ namespace kt {
 template <typename R, int EPT, int NL, int ACS, int MAXT>
 static cudaError_t launch_bwd_t(const KtGeom &g, const KtGenImage &im, const KtOps &ops, const BwdArgs &a, size_t smem,
                                 cudaStream_t st) {
+  if constexpr (NL > 0 && ACS >= 3 && ACS <= 5) {
+    if (a.y_form) return launch_bwd_t<R, EPT, NL, ACS + 8, MAXT>(g, im, ops, a, smem, st);
+  }
   if (a.sweep) {
     if constexpr (NL == 0) {
       const cudaError_t attr = kt_allow_large_smem((const void *)bwd_kernel<R, EPT, 0, ACS, true, MAXT>);

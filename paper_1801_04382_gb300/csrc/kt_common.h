@@ -129,6 +129,7 @@ struct KtGenImage {
   // coefficients that every Chebyshev term reads, as kernel-parameter constants in both precisions
   // (the kernels then take them as constant-bank operands instead of shared-memory loads).
   float kd32[3 * KT_MAX_NL];  // last node's diagonal per local index: real part, imaginary part in two floats (kt_split)
+  float ki32[KT_MAX_NL];      // its imaginary part in one float
   double kd64[2 * KT_MAX_NL]; // the same, (re, im)
   float kc32[2 * 2];          // last node's cavity couplings (imaginary): [n-1] row (r, n-1) <- (g, n), [NC + n-1] the reverse
   double kc64[2 * 2];
@@ -138,12 +139,14 @@ struct KtGenImage {
   // of the hop that raises the middle / last node and lowers i, kh[2][i] and kh[3][i] of the reverse ones; of
   // the middle and the last node: kh[4][0] raising the last, kh[4][1] raising the middle one.
   float kh[5][2];
+  float km[2][2][3];          // kh[0], kh[2] times the ladder values of both nodes: 1, sqrt 2 or 2
 };
 
-// FP32 coefficient sets.  A state that barely changes from one interval to the next meets the same roundings
-// of the same coefficients each time, and they add up (4e-8 per interval in the norm at d = 81); scaling the
+// FP32 coefficient sets of the y form.  A state that barely changes from one interval to the next meets the same
+// roundings of the same coefficients each time, and they add up (up to 1e-7 per interval in the norm); scaling the
 // coefficients by a different lambda_s from interval to interval, undone in the two-float phase, makes
-// them random: 1e-5 -> 2e-6 over 100 intervals at d = 81.
+// them random: norm off by 1e-6 ... 1e-5 -> 1e-7 ... 2.6e-6 after 100 intervals (d = 81, 216, eight pulses).
+// Set 0 is not scaled (lambda_0 = 1): the T form uses it alone.
 #define KT_COEF_SETS 32
 
 // A diagonal value as a float on a 2^-21 grid and the float of what is left.  The dominant part of the

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(832) density_kernel(KtGeom g, KtGenImage im, K
     C chi = mkc((R)0, (R)0);
     if (need_chi && ok) chi = ((const C *)((const char *)a.chi + (size_t)j * a.slot_bytes))[x];
     if (j >= 1) {
-      uniform_coefs<R>(g, sm, im, j);
+      uniform_coefs<R, false>(g, sm, im, j);
       Diag<R> D{(R)0, (R)0, (R)0};
       if (ok) D = diag_of<R>(g, sm, dig);
       __syncthreads();

@@ -15,11 +15,18 @@
 // The series is run in y_k = (-i)^k T_k((G - c) / r) v with B = -2i (G - c) / r in the tables:
 //   y_0 = v,  y_1 = B v / 2,  y_{k+1} = y_{k-1} + B y_k,
 //   exp(-i G s) v = exp(-i c s) sum_k m_k y_k,  m_k = (2 - delta_k0) J_k(r s) real.
-// Against T_k with complex coefficients this saves two FMAs per element and term in the sum and the
-// 2 t - old, a fifth of the arithmetic at d = 6561.  In FP32 a row is summed from its small terms up
-// (couplings, then y_{k-1}, then the diagonal), and the diagonal's imaginary part and the phase are held
-// as two floats: the error against 64 bits over 100 intervals falls from 7.5e-6 to 2.4e-6 (d = 216), from
-// 1.1e-5 to 3.9e-6 (d = 81).
+// Against T_k with complex coefficients this saves two FMAs per element and term in the sum.  In FP32 a row is
+// summed from its small terms up (couplings, then y_{k-1}, then the diagonal), and the diagonal's imaginary part
+// and the phase are held as two floats: the error of Delta eps against 64 bits is 0.6e-6 ... 3.7e-6 where the T form's is
+// 2.4e-6 ... 8.5e-6 (d = 216, 101 intervals, eight pulses), 0.8e-6 ... 3.2e-6 where it is 3.5e-6 ... 5.8e-6 (d = 81,
+// 100 intervals).
+//
+// FP32 fibers and blocks run the T form all the same (t_form below), except in the sweeps that keep states for the
+// gradient.  The norm of the FP32 state decides in which interval a trajectory jumps, a threshold can lie closer to
+// the norm at t_j than its rounding, and a jump moved by an interval moves Delta eps by about 1 / M.  With hundreds of
+// trajectories that happens in one sweep out of ten if the rounding of the norm changes by 5e-6, as it does between the
+// two forms; with the T form the outcome of these problems is what it has always been.  It costs 3 % at d = 6561 and
+// nothing at d = 729, where the shared-memory pipe is the bound.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -44,6 +51,10 @@ template <typename C> __device__ __forceinline__ C cfma(C a, C b, C c) {  // c +
   c.y = fma(a.x, b.y, c.y);
   c.y = fma(a.y, b.x, c.y);
   return c;
+}
+
+template <typename C> __device__ __forceinline__ C cmul_fma(C a, C b) {  // a*b with its roundings written out
+  return mkc(fma(a.x, b.x, -(a.y * b.y)), fma(a.y, b.x, a.x * b.y));
 }
 
 // c + a*b for a purely real (rfma, a) or purely imaginary (ifma, i b) coefficient: the two
@@ -170,7 +181,7 @@ struct Smem {
   void *pair_val;             // [P*n_loc^2]
   int *hc_off;                // [n_cterms*n_loc*SH]
   void *hc_val;               // [n_cterms*n_loc*SH]
-  void *coef;                 // [K][T] real
+  void *coef;                 // [K][T] real; complex in the T form
   void *phase;                // [3][T] exp(-i c s) (FP32: in two floats, and r s / 2)
   double *red;                // [nwarps][T][8]
   double *tsc;                // per-trajectory scalars [TS_V0 + 8][T]
@@ -208,7 +219,7 @@ __host__ __device__ inline size_t carve(const KtGeom &g, int esz, char *base, Sm
   char *pv = take((size_t)esz * g.n_pairs * nl2);
   char *ho = take(sizeof(int) * g.n_cterms * g.n_loc * g.SH);
   char *hv = take((size_t)esz * g.n_cterms * g.n_loc * g.SH);
-  char *cf = take((size_t)esz / 2 * g.K * g.T);
+  char *cf = take((size_t)esz * g.K * g.T);
   char *phs = take((size_t)esz * 3 * g.T);
   char *rd = take(sizeof(double) * nwarps * g.T * 8);
   char *ts = take(sizeof(double) * 18 * g.T);
@@ -304,6 +315,27 @@ __device__ __forceinline__ void reduce_tau(double (&v)[NV], const KtGeom &g, dou
 // result by it once (what the order of that turn and the couplings leaves out is a hundred times smaller).
 template <typename R> struct Diag { R re, hi, lo; };
 
+// T form of the series (FP32 fibers and blocks): T_{k+1} = 2 Ghat T_k - T_{k-1} with 2 Ghat = i B, and complex coefficients
+// a_k = (2 - delta_k0) (-i)^k J_k(r s) exp(-i c s), one set for all intervals; a row is summed from the diagonal on (one
+// float), then the last node, the other nodes in turn and the hops, every FMA written out.  The order and the roundings
+// are part of the results (top of this file).  ACS 11, 12, 13: the mappings 3, 4, 5 in the y form.
+template <typename R, int NL, int ACS> __host__ __device__ constexpr bool t_form() { return sizeof(R) == 4 && NL > 0 && ACS < 8; }
+template <typename R, bool TF> struct CoefT { typedef R T; };
+template <typename R> struct CoefT<R, true> { typedef typename C2<R>::T T; };
+template <typename R, bool TF> using Coef = typename CoefT<R, TF>::T;
+template <typename R, typename C> __device__ __forceinline__ C coef_mul(R a, C v) {
+  if constexpr (sizeof(R) == sizeof(C)) return cmul_fma(a, v);
+  else return mkc(a * v.x, a * v.y);
+}
+template <typename R, typename C> __device__ __forceinline__ C coef_fma(R a, C v, C c) {
+  if constexpr (sizeof(R) == sizeof(C)) return cfma(a, v, c);
+  else return rfma(a, v, c);
+}
+// c + i w v, c + w v, c + w v of an entry i w, w (real), w (complex) of B; T form: of 2 Ghat = i B
+template <bool TF, typename R, typename C> __device__ __forceinline__ C add_im(R w, C v, C c) { return TF ? rfma(-w, v, c) : ifma(w, v, c); }
+template <bool TF, typename R, typename C> __device__ __forceinline__ C add_re(R w, C v, C c) { return TF ? ifma(w, v, c) : rfma(w, v, c); }
+template <bool TF, typename C> __device__ __forceinline__ C add_cx(C w, C v, C c) { return cfma(TF ? mkc(-w.y, w.x) : w, v, c); }
+
 __device__ __forceinline__ void store_diag(const Smem &sm, int e, float2 *dg, double re, double im) {
   float hi, lo;
   kt_split(im, &hi, &lo);
@@ -313,8 +345,9 @@ __device__ __forceinline__ void store_diag(const Smem &sm, int e, float2 *dg, do
 __device__ __forceinline__ void store_diag(const Smem &, int e, double2 *dg, double re, double im) {
   dg[e] = make_double2(re, im);
 }
-template <typename R> __device__ __forceinline__ Diag<R> load_diag(const Smem &sm, int e) {
+template <typename R, bool TF = false> __device__ __forceinline__ Diag<R> load_diag(const Smem &sm, int e) {
   const typename C2<R>::T v = ((const typename C2<R>::T *)sm.diag)[e];
+  if constexpr (TF) return Diag<R>{v.x, v.y + ((const R *)sm.diag_lo)[e], (R)0};
   return Diag<R>{v.x, v.y, sizeof(R) == 4 ? ((const R *)sm.diag_lo)[e] : (R)0};
 }
 template <typename R> __device__ __forceinline__ Diag<R> add_diag(Diag<R> a, Diag<R> b) {
@@ -323,12 +356,16 @@ template <typename R> __device__ __forceinline__ Diag<R> add_diag(Diag<R> a, Dia
 // Keeps the sums of D with a fiber's constants inside the loop: hoisted, they take two registers per element and spill.
 __device__ __forceinline__ void keep_in_loop(Diag<float> &D) { asm volatile("" : "+f"(D.re), "+f"(D.hi)); }
 __device__ __forceinline__ void keep_in_loop(Diag<double> &D) { asm volatile("" : "+d"(D.re), "+d"(D.hi)); }
-template <typename R, typename C> __device__ __forceinline__ C diag_init(Diag<R> D, C v, C old) {
-  if constexpr (sizeof(R) == 4) return mkc(D.re * v.x, D.re * v.y);
+template <bool TF = false, typename R, typename C> __device__ __forceinline__ C diag_init(Diag<R> D, C v, C old) {
+  if constexpr (TF) return cmul_fma(mkc(-D.hi, D.re), v);
+  else if constexpr (sizeof(R) == 4) return mkc(D.re * v.x, D.re * v.y);
   else return mkc(fma(-D.hi, v.y, fma(D.re, v.x, old.x)), fma(D.hi, v.x, fma(D.re, v.y, old.y)));
 }
-template <typename R, typename C> __device__ __forceinline__ C diag_done(Diag<R> D, C v, C old, C s) {
-  if constexpr (sizeof(R) == 4) {
+template <bool TF = false, typename R, typename C> __device__ __forceinline__ C diag_done(Diag<R> D, C v, C old, C s) {
+  if constexpr (TF) {
+    s.x -= old.x;
+    s.y -= old.y;
+  } else if constexpr (sizeof(R) == 4) {
     s.x += old.x;
     s.y += old.y;
     s.x = fma(-D.hi, v.y, s.x);
@@ -338,9 +375,11 @@ template <typename R, typename C> __device__ __forceinline__ C diag_done(Diag<R>
 }
 
 // acc times exp(-i c s) of trajectory tau and (FP32) 1 + i lo(q) r s / 2 of each element
-template <typename R, int N, class LO>
+// (T form: nothing, the phase is in the coefficients)
+template <typename R, int N, bool TF = false, class LO>
 __device__ __forceinline__ void apply_phase(const KtGeom &g, const Smem &sm, int tau, typename C2<R>::T (&acc)[N], LO lo_of) {
   typedef typename C2<R>::T C;
+  if constexpr (TF) return;
   const C ph = ((const C *)sm.phase)[tau];
   if constexpr (sizeof(R) == 4) {
     const C lo = ((const C *)sm.phase)[g.T + tau];
@@ -549,7 +588,7 @@ __device__ __forceinline__ void load_items(const KtGeom &g, const KtOps &ops, It
 // out[q] = old[q] + (B v)[item_q] for the whole fiber of this thread, q < NL, old[q] = prev[item_q] (PREV
 // false: 0).  Coefficients of nodes other than the last are looked up once per fiber; those of the last
 // node depend only on q and are the same for every lane.
-template <typename R, int NL, bool PREV>
+template <typename R, int NL, bool PREV, bool TF>
 __device__ __forceinline__ void apply_fiber(const KtGeom &g, const KtGenImage &im, const Smem &sm,
                                             const typename C2<R>::T *__restrict__ v,
                                             const typename C2<R>::T *prev, int base, uint32_t fdig, Diag<R> Df,
@@ -562,14 +601,14 @@ __device__ __forceinline__ void apply_fiber(const KtGeom &g, const KtGenImage &i
   const C zero = mkc((R)0, (R)0);
 #pragma unroll
   for (int q = 0; q < NL; ++q)
-    out[q] = diag_init(add_diag(Df, load_diag<R>(sm, last * NL + q)), v[base + q * T], PREV ? prev[base + q * T] : zero);
+    out[q] = diag_init<TF>(add_diag(Df, load_diag<R, TF>(sm, last * NL + q)), v[base + q * T], PREV ? prev[base + q * T] : zero);
   // last node: row q of its factor
 #pragma unroll
   for (int q = 0; q < NL; ++q) {
     const int e0 = (last * NL + q) * g.S;
     for (int s = 0; s < g.S; ++s) {
       const int off = sm.loc_off[e0 + s];
-      if (off) out[q] = cfma(lv[e0 + s], v[base + q * T + off], out[q]);
+      if (off) out[q] = add_cx<TF>(lv[e0 + s], v[base + q * T + off], out[q]);
     }
   }
   // other nodes: one row per fiber
@@ -580,7 +619,7 @@ __device__ __forceinline__ void apply_fiber(const KtGeom &g, const KtGenImage &i
       if (off) {
         const C w = lv[e0 + s];
 #pragma unroll
-        for (int q = 0; q < NL; ++q) out[q] = cfma(w, v[base + q * T + off], out[q]);
+        for (int q = 0; q < NL; ++q) out[q] = add_cx<TF>(w, v[base + q * T + off], out[q]);
       }
     }
   }
@@ -594,61 +633,61 @@ __device__ __forceinline__ void apply_fiber(const KtGeom &g, const KtGenImage &i
       if (off) {
         const C w = pv[e];
 #pragma unroll
-        for (int q = 0; q < NL; ++q) out[q] = cfma(w, v[base + q * T + off], out[q]);
+        for (int q = 0; q < NL; ++q) out[q] = add_cx<TF>(w, v[base + q * T + off], out[q]);
       }
     } else if (pd == last) {
       const int e0 = pb + ((fdig >> (4 * ps)) & 15);
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
         const int off = sm.pair_off[e0 + q * NL];
-        if (off) out[q] = cfma(pv[e0 + q * NL], v[base + q * T + off], out[q]);
+        if (off) out[q] = add_cx<TF>(pv[e0 + q * NL], v[base + q * T + off], out[q]);
       }
     } else {
       const int e0 = pb + ((fdig >> (4 * pd)) & 15) * NL;
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
         const int off = sm.pair_off[e0 + q];
-        if (off) out[q] = cfma(pv[e0 + q], v[base + q * T + off], out[q]);
+        if (off) out[q] = add_cx<TF>(pv[e0 + q], v[base + q * T + off], out[q]);
       }
     }
   }
 #pragma unroll
   for (int q = 0; q < NL; ++q)
-    out[q] = diag_done(add_diag(Df, load_diag<R>(sm, last * NL + q)), v[base + q * T], PREV ? prev[base + q * T] : zero,
+    out[q] = diag_done<TF>(add_diag(Df, load_diag<R, TF>(sm, last * NL + q)), v[base + q * T], PREV ? prev[base + q * T] : zero,
                        out[q]);
 }
 
 // Chebyshev sum in fiber mapping (see cheb_run).
-template <typename R, int NL, class IT>
+template <typename R, int NL, bool TF, class IT>
 __device__ void cheb_run_fiber(const KtGeom &g, const KtGenImage &im, const Smem &sm, const IT &it, int K,
                                typename C2<R>::T (&acc)[NL]) {
   typedef typename C2<R>::T C;
   C *A = (C *)sm.bufA;
   C *B = (C *)sm.bufB;
-  const R *cf = (const R *)sm.coef;
+  const Coef<R, TF> *cf = (const Coef<R, TF> *)sm.coef;
   const int tau = threadIdx.x % g.T;
   const bool ok = it.ok(0);
   const int base = it.item(0);
   const uint32_t fdig = it.dig(0);
   const int last = g.n_nodes - 1;
   Diag<R> Df{(R)0, (R)0, (R)0};
-  for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
-  const R c0 = cf[tau];
+  for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R, TF>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
+  const Coef<R, TF> c0 = cf[tau];
 #pragma unroll
   for (int q = 0; q < NL; ++q) {
     const C v = ok ? A[base + q * g.T] : mkc((R)0, (R)0);
-    acc[q] = mkc(c0 * v.x, c0 * v.y);
+    acc[q] = coef_mul(c0, v);
   }
   if (K > 1) {
     C t[NL];
     if (ok) {
-      apply_fiber<R, NL, false>(g, im, sm, A, A, base, fdig, Df, t);
-      const R c1 = cf[g.T + tau];
+      apply_fiber<R, NL, false, TF>(g, im, sm, A, A, base, fdig, Df, t);
+      const Coef<R, TF> c1 = cf[g.T + tau];
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
         t[q] = mkc((R)0.5 * t[q].x, (R)0.5 * t[q].y);
         B[base + q * g.T] = t[q];
-        acc[q] = rfma(c1, t[q], acc[q]);
+        acc[q] = coef_fma(c1, t[q], acc[q]);
       }
     }
     __syncthreads();
@@ -656,12 +695,12 @@ __device__ void cheb_run_fiber(const KtGeom &g, const KtGenImage &im, const Smem
     C *Q = B;   // holds y_k
     for (int k = 2; k < K; ++k) {
       if (ok) {
-        const R a = cf[k * g.T + tau];
-        apply_fiber<R, NL, true>(g, im, sm, Q, P, base, fdig, Df, t);
+        const Coef<R, TF> a = cf[k * g.T + tau];
+        apply_fiber<R, NL, true, TF>(g, im, sm, Q, P, base, fdig, Df, t);
 #pragma unroll
         for (int q = 0; q < NL; ++q) {
           P[base + q * g.T] = t[q];
-          acc[q] = rfma(a, t[q], acc[q]);
+          acc[q] = coef_fma(a, t[q], acc[q]);
         }
       }
       __syncthreads();
@@ -670,7 +709,7 @@ __device__ void cheb_run_fiber(const KtGeom &g, const KtGenImage &im, const Smem
   } else {
     __syncthreads();
   }
-  apply_phase<R, NL>(g, sm, tau, acc, [&](int q) { return Df.lo + load_diag<R>(sm, last * NL + q).lo; });
+  apply_phase<R, NL, TF>(g, sm, tau, acc, [&](int q) { return Df.lo + load_diag<R, TF>(sm, last * NL + q).lo; });
 }
 
 // Chebyshev sum: acc = exp(-i c s) sum_k coef[k][tau] y_k with y_0 = v in A on entry (synced).
@@ -724,14 +763,24 @@ __device__ void cheb_run(const KtGeom &g, const KtGenImage &im, const Smem &sm, 
   apply_phase<R, EPT>(g, sm, tau, acc, [&](int q) { return it.ok(q) ? dv[q].lo : (R)0; });
 }
 
+// m (-i)^k (cs + i sn)
+template <typename R> __device__ __forceinline__ typename C2<R>::T t_coef(int k, double m, double cs, double sn) {
+  switch (k & 3) {
+    case 0: return mkc((R)(m * cs), (R)(m * sn));
+    case 1: return mkc((R)(m * sn), (R)(-m * cs));
+    case 2: return mkc((R)(-m * cs), (R)(-m * sn));
+  }
+  return mkc((R)(-m * sn), (R)(m * cs));
+}
+
 // Coefficients of exp(-i G s) for every trajectory, s in sm.tsc[TS_X] (synchronised): m_k = (2 - delta_k0) J_k(r s) and the
 // phase exp(-i c s).  Called by the whole block, one thread per coefficient: its Chebyshev series in s / dt by Clenshaw's
 // recurrence.  (One thread running Miller's recurrence for all orders took longer than a series of a small problem in
 // FP64, where an instruction costs a warp 64 cycles however few of its lanes work: passes with several jumps per
 // trajectory at d = 81 28.5 -> 25.3 ms, d = 216 FP32 9.9 -> 8.3 ms, d = 729 FP32 26.9 -> 25.4 ms.)
-template <typename R>
+template <typename R, bool TF>
 __device__ void piece_coefs(const KtGeom &g, const KtGenImage &im, const Smem &sm, double c_gen) {
-  R *cf = (R *)sm.coef;
+  Coef<R, TF> *cf = (Coef<R, TF> *)sm.coef;
   for (int e = threadIdx.x; e < g.K * g.T; e += blockDim.x) {
     const int k = e / g.T;
     const double y = 2.0 * (sm.tsc[TS_X * g.T + e % g.T] / g.dt) - 1.0, y2 = 2.0 * y;
@@ -741,8 +790,16 @@ __device__ void piece_coefs(const KtGeom &g, const KtGenImage &im, const Smem &s
       b2 = b1;
       b1 = b;
     }
-    cf[e] = (R)fma(y, b1, im.piece[k] - b2);
+    const double m = fma(y, b1, im.piece[k] - b2);
+    if constexpr (TF) {
+      double sn, cs;
+      sincos(-c_gen * sm.tsc[TS_X * g.T + e % g.T], &sn, &cs);
+      cf[e] = t_coef<R>(k, m, cs, sn);
+    } else {
+      cf[e] = (R)m;
+    }
   }
+  if constexpr (TF) return;
   const int t = blockDim.x - 1 - threadIdx.x;   // the phases on the last warp
   if (t < g.T) {
     const double s = sm.tsc[TS_X * g.T + t];
@@ -752,12 +809,16 @@ __device__ void piece_coefs(const KtGeom &g, const KtGenImage &im, const Smem &s
   }
 }
 
-template <typename R>
+template <typename R, bool TF>
 __device__ void uniform_coefs(const KtGeom &g, const Smem &sm, const KtGenImage &im, int j) {
-  R *cf = (R *)sm.coef;
-  const int set = j & (im.sets - 1);
+  Coef<R, TF> *cf = (Coef<R, TF> *)sm.coef;
+  const int set = TF ? 0 : j & (im.sets - 1);   // set 0 is not scaled
   const double *full = im.cheb_full + (size_t)set * g.K;
-  for (int e = threadIdx.x; e < g.K * g.T; e += blockDim.x) cf[e] = (R)full[e / g.T];
+  for (int e = threadIdx.x; e < g.K * g.T; e += blockDim.x) {
+    if constexpr (TF) cf[e] = t_coef<R>(e / g.T, full[e / g.T], im.phase_full[0].re, im.phase_full[0].im);
+    else cf[e] = (R)full[e / g.T];
+  }
+  if constexpr (TF) return;
   for (int t = threadIdx.x; t < g.T; t += blockDim.x)
     store_phase<R>(g, sm, t, im.phase_full[set].re, im.phase_full[set].im, g.dt);
 }
@@ -830,7 +891,7 @@ __device__ __forceinline__ void sweep_coefs(const KtGeom &g, const KtGenImage &i
     run.coef = (R *)extra + set * g.K;
     run.phase = (C *)((R *)extra + (im.sets * g.K + 7) / 8 * 8) + 3 * set;
   } else {
-    uniform_coefs<R>(g, sm, im, j);
+    uniform_coefs<R, false>(g, sm, im, j);
   }
 }
 
@@ -900,12 +961,10 @@ __device__ __forceinline__ void load_rows(const KtGeom &g, const Smem &sm, uint3
 }
 
 // Constants of the real / imaginary kernels (kernel parameters of the image, see KtGenImage).
-template <typename R> __device__ __forceinline__ Diag<R> acs_kd(const KtGenImage &im, int q);
-template <> __device__ __forceinline__ Diag<float> acs_kd<float>(const KtGenImage &im, int q) {
-  return Diag<float>{im.kd32[3 * q], im.kd32[3 * q + 1], im.kd32[3 * q + 2]};
-}
-template <> __device__ __forceinline__ Diag<double> acs_kd<double>(const KtGenImage &im, int q) {
-  return Diag<double>{im.kd64[2 * q], im.kd64[2 * q + 1], 0.0};
+template <typename R, bool TF = false> __device__ __forceinline__ Diag<R> acs_kd(const KtGenImage &im, int q) {
+  if constexpr (sizeof(R) == 8) return Diag<R>{im.kd64[2 * q], im.kd64[2 * q + 1], 0.0};
+  else if constexpr (TF) return Diag<R>{im.kd32[3 * q], im.ki32[q], 0.f};
+  else return Diag<R>{im.kd32[3 * q], im.kd32[3 * q + 1], im.kd32[3 * q + 2]};
 }
 template <typename R> __device__ __forceinline__ const R *acs_kc(const KtGenImage &im);
 template <> __device__ __forceinline__ const float *acs_kc<float>(const KtGenImage &im) { return im.kc32; }
@@ -930,7 +989,7 @@ __device__ __forceinline__ R sqrt_n(int n) {
 // pair coefficients, ladder values) are kernel-parameter or compile-time constants, so only the
 // drive couplings, the other nodes' pair tables and the states are read from shared memory.
 // CACHE: the other nodes' rows come from rc (registers) instead of the shared tables.
-template <typename R, int NC, int TT, bool RI, bool CACHE, bool PREV>
+template <typename R, int NC, int TT, bool RI, bool CACHE, bool PREV, bool TF>
 __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im, const Smem &sm,
                                           const typename C2<R>::T *__restrict__ v,
                                           const typename C2<R>::T *prev, int base, uint32_t fdig, Diag<R> Df,
@@ -947,33 +1006,33 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
   const int last = g.n_nodes - 1;
   const int T = TT > 0 ? TT : g.T;   // TT > 0: tile width fixed at compile time
   auto diag = [&](int q) -> Diag<R> {
-    if constexpr (RI) return add_diag(Df, acs_kd<R>(im, q));
-    else return add_diag(Df, load_diag<R>(sm, last * NL + q));
+    if constexpr (RI) return add_diag(Df, acs_kd<R, TF>(im, q));
+    else return add_diag(Df, load_diag<R, TF>(sm, last * NL + q));
   };
   const C zero = mkc((R)0, (R)0);
 #pragma unroll
-  for (int q = 0; q < NL; ++q) out[q] = diag_init(diag(q), vk[q], PREV ? prev[base + q * T] : zero);
+  for (int q = 0; q < NL; ++q) out[q] = diag_init<TF>(diag(q), vk[q], PREV ? prev[base + q * T] : zero);
   // last node: cavity (r, n-1) <-> (g, n) and drive (r, n) <-> (e, n)
 #pragma unroll
   for (int n = 1; n <= NC; ++n) {
     const int qr = 2 * NP + n - 1, qg = n;
     if constexpr (RI) {
-      out[qr] = ifma(acs_kc<R>(im)[n - 1], vk[qg], out[qr]);
-      out[qg] = ifma(acs_kc<R>(im)[NC + n - 1], vk[qr], out[qg]);
+      out[qr] = add_im<TF>(acs_kc<R>(im)[n - 1], vk[qg], out[qr]);
+      out[qg] = add_im<TF>(acs_kc<R>(im)[NC + n - 1], vk[qr], out[qg]);
     } else {
-      out[qr] = cfma(ld[qr * NL + qg], vk[qg], out[qr]);
-      out[qg] = cfma(ld[qg * NL + qr], vk[qr], out[qg]);
+      out[qr] = add_cx<TF>(ld[qr * NL + qg], vk[qg], out[qr]);
+      out[qg] = add_cx<TF>(ld[qg * NL + qr], vk[qr], out[qg]);
     }
   }
 #pragma unroll
   for (int n = 0; n <= NC; ++n) {
     const int qr = 2 * NP + n, qe = NP + n;
     if constexpr (RI) {
-      out[qr] = rfma(ld[qr * NL + qe].x, vk[qe], out[qr]);
-      out[qe] = rfma(ld[qe * NL + qr].x, vk[qr], out[qe]);
+      out[qr] = add_re<TF>(ld[qr * NL + qe].x, vk[qe], out[qr]);
+      out[qe] = add_re<TF>(ld[qe * NL + qr].x, vk[qr], out[qe]);
     } else {
-      out[qr] = cfma(ld[qr * NL + qe], vk[qe], out[qr]);
-      out[qe] = cfma(ld[qe * NL + qr], vk[qr], out[qe]);
+      out[qr] = add_cx<TF>(ld[qr * NL + qe], vk[qe], out[qr]);
+      out[qe] = add_cx<TF>(ld[qe * NL + qr], vk[qr], out[qe]);
     }
   }
   // other nodes: one row per fiber, each entry one neighbouring fiber
@@ -984,12 +1043,12 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
       if (off0) {
         const R a = lv[e0].y;
 #pragma unroll
-        for (int q = 0; q < NL; ++q) out[q] = ifma(a, v[base + off0 + q * T], out[q]);
+        for (int q = 0; q < NL; ++q) out[q] = add_im<TF>(a, v[base + off0 + q * T], out[q]);
       }
       if (off1) {
         const R b = lv[e0 + 1].x;
 #pragma unroll
-        for (int q = 0; q < NL; ++q) out[q] = rfma(b, v[base + off1 + q * T], out[q]);
+        for (int q = 0; q < NL; ++q) out[q] = add_re<TF>(b, v[base + off1 + q * T], out[q]);
       }
     }
   } else if constexpr (RI) {
@@ -997,11 +1056,11 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
     for (int i = 0; i < 3; ++i) {
       if (rc.off0[i]) {
 #pragma unroll
-        for (int q = 0; q < NL; ++q) out[q] = ifma(rc.a[i], v[base + rc.off0[i] + q * T], out[q]);
+        for (int q = 0; q < NL; ++q) out[q] = add_im<TF>(rc.a[i], v[base + rc.off0[i] + q * T], out[q]);
       }
       if (rc.off1[i]) {
 #pragma unroll
-        for (int q = 0; q < NL; ++q) out[q] = rfma(rc.b[i], v[base + rc.off1[i] + q * T], out[q]);
+        for (int q = 0; q < NL; ++q) out[q] = add_re<TF>(rc.b[i], v[base + rc.off1[i] + q * T], out[q]);
       }
     }
   } else {
@@ -1012,7 +1071,7 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
         if (off) {
           const C w = lv[e0 + s];
 #pragma unroll
-          for (int q = 0; q < NL; ++q) out[q] = cfma(w, v[base + off + q * T], out[q]);
+          for (int q = 0; q < NL; ++q) out[q] = add_cx<TF>(w, v[base + off + q * T], out[q]);
         }
       }
     }
@@ -1027,11 +1086,11 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
         if constexpr (RI) {
           const R b = pv[e].x;
 #pragma unroll
-          for (int q = 0; q < NL; ++q) out[q] = rfma(b, v[base + off + q * T], out[q]);
+          for (int q = 0; q < NL; ++q) out[q] = add_re<TF>(b, v[base + off + q * T], out[q]);
         } else {
           const C w = pv[e];
 #pragma unroll
-          for (int q = 0; q < NL; ++q) out[q] = cfma(w, v[base + off + q * T], out[q]);
+          for (int q = 0; q < NL; ++q) out[q] = add_cx<TF>(w, v[base + off + q * T], out[q]);
         }
       }
     } else if (pd == last) {
@@ -1044,14 +1103,14 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
 #pragma unroll
           for (int q = 0; q < NL; ++q) {
             if (q % NP == 0) continue;
-            out[q] = rfma(cb * sqrt_n<R>(q % NP), v[base + off + (q - 1) * T], out[q]);
+            out[q] = add_re<TF>(cb * sqrt_n<R>(q % NP), v[base + off + (q - 1) * T], out[q]);
           }
         } else {
           const C cf = cmul(pc[p], lo[xs]);
 #pragma unroll
           for (int q = 0; q < NL; ++q) {
             if (q % NP == 0) continue;
-            out[q] = cfma(cmul(cf, ra[q]), v[base + off + (q - 1) * T], out[q]);
+            out[q] = add_cx<TF>(cmul(cf, ra[q]), v[base + off + (q - 1) * T], out[q]);
           }
         }
       }
@@ -1065,31 +1124,31 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
 #pragma unroll
           for (int q = 0; q < NL; ++q) {
             if (q % NP == NC) continue;
-            out[q] = rfma(cb * sqrt_n<R>(q % NP + 1), v[base + off + (q + 1) * T], out[q]);
+            out[q] = add_re<TF>(cb * sqrt_n<R>(q % NP + 1), v[base + off + (q + 1) * T], out[q]);
           }
         } else {
           const C cf = cmul(pc[p], ra[xd]);
 #pragma unroll
           for (int q = 0; q < NL; ++q) {
             if (q % NP == NC) continue;
-            out[q] = cfma(cmul(cf, lo[q]), v[base + off + (q + 1) * T], out[q]);
+            out[q] = add_cx<TF>(cmul(cf, lo[q]), v[base + off + (q + 1) * T], out[q]);
           }
         }
       }
     }
   }
 #pragma unroll
-  for (int q = 0; q < NL; ++q) out[q] = diag_done(diag(q), vk[q], PREV ? prev[base + q * T] : zero, out[q]);
+  for (int q = 0; q < NL; ++q) out[q] = diag_done<TF>(diag(q), vk[q], PREV ? prev[base + q * T] : zero, out[q]);
 }
 
-template <typename R, int NC, int TT, bool RI, bool CACHE, class IT>
+template <typename R, int NC, int TT, bool RI, bool CACHE, bool TF, class IT>
 __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &sm, const IT &it,
                              int K, typename C2<R>::T (&acc)[3 * (NC + 1)]) {
   typedef typename C2<R>::T C;
   constexpr int NL = 3 * (NC + 1);
   C *A = (C *)sm.bufA;
   C *B = (C *)sm.bufB;
-  const R *cf = (const R *)sm.coef;
+  const Coef<R, TF> *cf = (const Coef<R, TF> *)sm.coef;
   const int T = TT > 0 ? TT : g.T;
   const int tau = TT == 1 ? 0 : (int)(threadIdx.x % T);
   const bool ok = it.ok(0);
@@ -1097,28 +1156,28 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
   const uint32_t fdig = it.dig(0);
   const int last = g.n_nodes - 1;
   Diag<R> Df{(R)0, (R)0, (R)0};
-  for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
+  for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R, TF>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
   RowCache<R> rc;
   if constexpr (RI && CACHE) {
     if (ok) load_rows<R, NL>(g, sm, fdig, rc);
   }
   C vk[NL];
-  const R c0 = cf[tau];
+  const Coef<R, TF> c0 = cf[tau];
 #pragma unroll
   for (int q = 0; q < NL; ++q) {
     vk[q] = ok ? A[base + q * T] : mkc((R)0, (R)0);
-    acc[q] = mkc(c0 * vk[q].x, c0 * vk[q].y);
+    acc[q] = coef_mul(c0, vk[q]);
   }
   if (K > 1) {
     C t[NL];
     if (ok) {
-      apply_acs<R, NC, TT, RI, CACHE, false>(g, im, sm, A, A, base, fdig, Df, vk, t, rc);
-      const R c1 = cf[T + tau];
+      apply_acs<R, NC, TT, RI, CACHE, false, TF>(g, im, sm, A, A, base, fdig, Df, vk, t, rc);
+      const Coef<R, TF> c1 = cf[T + tau];
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
         vk[q] = mkc((R)0.5 * t[q].x, (R)0.5 * t[q].y);
         B[base + q * T] = vk[q];
-        acc[q] = rfma(c1, vk[q], acc[q]);
+        acc[q] = coef_fma(c1, vk[q], acc[q]);
       }
     }
     __syncthreads();
@@ -1126,13 +1185,13 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
     C *Q = B;   // holds y_k (this thread's fiber also in vk)
     for (int k = 2; k < K; ++k) {
       if (ok) {
-        const R a = cf[k * T + tau];
+        const Coef<R, TF> a = cf[k * T + tau];
         if constexpr (RI) keep_in_loop(Df);
-        apply_acs<R, NC, TT, RI, CACHE, true>(g, im, sm, Q, P, base, fdig, Df, vk, t, rc);
+        apply_acs<R, NC, TT, RI, CACHE, true, TF>(g, im, sm, Q, P, base, fdig, Df, vk, t, rc);
 #pragma unroll
         for (int q = 0; q < NL; ++q) {
           P[base + q * T] = t[q];
-          acc[q] = rfma(a, t[q], acc[q]);
+          acc[q] = coef_fma(a, t[q], acc[q]);
           vk[q] = t[q];
         }
       }
@@ -1142,9 +1201,9 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
   } else {
     __syncthreads();
   }
-  apply_phase<R, NL>(g, sm, tau, acc, [&](int q) {
-    if constexpr (RI) return Df.lo + acs_kd<R>(im, q).lo;
-    else return Df.lo + load_diag<R>(sm, last * NL + q).lo;
+  apply_phase<R, NL, TF>(g, sm, tau, acc, [&](int q) {
+    if constexpr (RI) return Df.lo + acs_kd<R, TF>(im, q).lo;
+    else return Df.lo + load_diag<R, TF>(sm, last * NL + q).lo;
   });
 }
 
@@ -1215,8 +1274,9 @@ __device__ __forceinline__ void load_blk(const KtGeom &g, const KtGenImage &im, 
   }
 }
 
-// out[q] = prev[base + q] + (B v)[base + q] for the thread's block, as apply_acs
-template <typename R, int NC>
+// out[q] = prev[base + q] + (B v)[base + q] for the thread's block, as apply_acs.  Every element's terms come in the order of
+// the fiber mapping (for the hops as long as a pair of nodes hops one way only, as a cascade does), with its coefficients.
+template <typename R, int NC, bool TF>
 __device__ __forceinline__ void apply_blk(const KtGeom &g, const KtGenImage &im, const Smem &sm,
                                           const typename C2<R>::T *__restrict__ v, const typename C2<R>::T *prev,
                                           int base, const Diag<R> (&Df)[NC + 1],
@@ -1226,27 +1286,91 @@ __device__ __forceinline__ void apply_blk(const KtGeom &g, const KtGenImage &im,
   typedef typename C2<R>::T C;
   constexpr int NP = NC + 1, NL = 3 * NP, E = NP * NL;
   const C *ld = (const C *)sm.ldense;
+  const C zero = mkc((R)0, (R)0);
 #pragma unroll
-  for (int q = 0; q < E; ++q) {
-    const R re = Df[q / NL].re + acs_kd<R>(im, q % NL).re;
-    out[q] = mkc(re * vk[q].x, re * vk[q].y);
-  }
+  for (int q = 0; q < E; ++q) out[q] = diag_init<TF>(add_diag(Df[q / NL], acs_kd<R, TF>(im, q % NL)), vk[q], zero);
   // last node
 #pragma unroll
   for (int m = 0; m < NP; ++m) {
 #pragma unroll
     for (int n = 1; n <= NC; ++n) {
       const int qr = m * NL + 2 * NP + n - 1, qg = m * NL + n;
-      out[qr] = ifma(acs_kc<R>(im)[n - 1], vk[qg], out[qr]);
-      out[qg] = ifma(acs_kc<R>(im)[NC + n - 1], vk[qr], out[qg]);
+      out[qr] = add_im<TF>(acs_kc<R>(im)[n - 1], vk[qg], out[qr]);
+      out[qg] = add_im<TF>(acs_kc<R>(im)[NC + n - 1], vk[qr], out[qg]);
     }
 #pragma unroll
     for (int n = 0; n <= NC; ++n) {
       const int r = 2 * NP + n, e = NP + n;
-      out[m * NL + r] = rfma(ld[r * NL + e].x, vk[m * NL + e], out[m * NL + r]);
-      out[m * NL + e] = rfma(ld[e * NL + r].x, vk[m * NL + r], out[m * NL + e]);
+      out[m * NL + r] = add_re<TF>(ld[r * NL + e].x, vk[m * NL + e], out[m * NL + r]);
+      out[m * NL + e] = add_re<TF>(ld[e * NL + r].x, vk[m * NL + r], out[m * NL + e]);
     }
   }
+  // outer nodes' rows
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (rc.off0[i]) {
+#pragma unroll
+      for (int q = 0; q < E; ++q) out[q] = add_im<TF>(rc.a[i], v[base + rc.off0[i] + q], out[q]);
+    }
+    if (rc.off1[i]) {
+#pragma unroll
+      for (int q = 0; q < E; ++q) out[q] = add_re<TF>(rc.b[i], v[base + rc.off1[i] + q], out[q]);
+    }
+  }
+  // middle node's rows
+#pragma unroll
+  for (int m = 0; m < NP; ++m)
+    if (rc.moff0[m]) {
+#pragma unroll
+      for (int q = 0; q < NL; ++q) out[m * NL + q] = add_im<TF>(rc.ma[m], v[base + rc.moff0[m] + m * NL + q], out[m * NL + q]);
+    }
+  if (rc.moff1) {
+#pragma unroll
+    for (int q = 0; q < E; ++q) out[q] = add_re<TF>(rc.mb[q / NL], v[base + rc.moff1 + q], out[q]);
+  }
+  // hops between the outer nodes
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (rc.hoff[i]) {
+#pragma unroll
+      for (int q = 0; q < E; ++q) out[q] = add_re<TF>(rc.hop[i], v[base + rc.hoff[i] + q], out[q]);
+    }
+  // hops between an outer node and the middle and the last one
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (i < g.n_nodes - 2) {
+      const int s = g.stride[i];
+      // middle or last node raised, node i lowered: the block with one photon more in node i
+      if (rc.up[i] != (R)0 && (im.kh[0][i] != 0.f || im.kh[1][i] != 0.f)) {
+        const bool two = rc.up[i] > (R)1;
+        const R cm1 = two ? im.km[0][i][1] : im.km[0][i][0], cm2 = two ? im.km[0][i][2] : im.km[0][i][1];
+        const R cl = (R)im.kh[1][i] * rc.up[i];
+#pragma unroll
+        for (int m = 0; m < NP; ++m)
+#pragma unroll
+          for (int q = 0; q < NL; ++q) {
+            if (m == NC && q % NP == NC) continue;
+            const C w = v[base + s + m * NL + q];
+            if (m < NC) out[(m + 1) * NL + q] = add_re<TF>(m == 1 ? cm2 : cm1, w, out[(m + 1) * NL + q]);
+            if (q % NP < NC) out[m * NL + q + 1] = add_re<TF>(cl * sqrt_n<R>(q % NP + 1), w, out[m * NL + q + 1]);
+          }
+      }
+      // node i raised, middle or last node lowered
+      if (rc.dn[i] != (R)0 && (im.kh[2][i] != 0.f || im.kh[3][i] != 0.f)) {
+        const bool two = rc.dn[i] > (R)1;
+        const R cm1 = two ? im.km[1][i][1] : im.km[1][i][0], cm2 = two ? im.km[1][i][2] : im.km[1][i][1];
+        const R cl = (R)im.kh[3][i] * rc.dn[i];
+#pragma unroll
+        for (int m = NC; m >= 0; --m)
+#pragma unroll
+          for (int q = 0; q < NL; ++q) {
+            if (m == 0 && q % NP == 0) continue;
+            const C w = v[base - s + m * NL + q];
+            if (m >= 1) out[(m - 1) * NL + q] = add_re<TF>(m == 2 ? cm2 : cm1, w, out[(m - 1) * NL + q]);
+            if (q % NP >= 1) out[m * NL + q - 1] = add_re<TF>(cl * sqrt_n<R>(q % NP), w, out[m * NL + q - 1]);
+          }
+      }
+    }
   // hops between the middle and the last node
   {
     const R cl = (R)im.kh[4][0], cm = (R)im.kh[4][1];
@@ -1256,7 +1380,7 @@ __device__ __forceinline__ void apply_blk(const KtGeom &g, const KtGenImage &im,
 #pragma unroll
         for (int q = 0; q < NL; ++q)
           if (q % NP >= 1)
-            out[m * NL + q] = rfma(cl * (sqrt_n<R>(m + 1) * sqrt_n<R>(q % NP)), vk[(m + 1) * NL + q - 1], out[m * NL + q]);
+            out[m * NL + q] = add_re<TF>((cl * sqrt_n<R>(m + 1)) * sqrt_n<R>(q % NP), vk[(m + 1) * NL + q - 1], out[m * NL + q]);
     }
     if (cm != (R)0) {
 #pragma unroll
@@ -1264,96 +1388,40 @@ __device__ __forceinline__ void apply_blk(const KtGeom &g, const KtGenImage &im,
 #pragma unroll
         for (int q = 0; q < NL; ++q)
           if (q % NP < NC)
-            out[m * NL + q] = rfma(cm * (sqrt_n<R>(m) * sqrt_n<R>(q % NP + 1)), vk[(m - 1) * NL + q + 1], out[m * NL + q]);
-    }
-  }
-  // middle node
-  if (rc.moff1) {
-#pragma unroll
-    for (int q = 0; q < E; ++q) out[q] = rfma(rc.mb[q / NL], v[base + rc.moff1 + q], out[q]);
-  }
-#pragma unroll
-  for (int m = 0; m < NP; ++m)
-    if (rc.moff0[m]) {
-#pragma unroll
-      for (int q = 0; q < NL; ++q) out[m * NL + q] = ifma(rc.ma[m], v[base + rc.moff0[m] + m * NL + q], out[m * NL + q]);
-    }
-  // outer nodes
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    if (rc.off0[i]) {
-#pragma unroll
-      for (int q = 0; q < E; ++q) out[q] = ifma(rc.a[i], v[base + rc.off0[i] + q], out[q]);
-    }
-    if (rc.off1[i]) {
-#pragma unroll
-      for (int q = 0; q < E; ++q) out[q] = rfma(rc.b[i], v[base + rc.off1[i] + q], out[q]);
-    }
-    if (rc.hoff[i]) {
-#pragma unroll
-      for (int q = 0; q < E; ++q) out[q] = rfma(rc.hop[i], v[base + rc.hoff[i] + q], out[q]);
-    }
-    if (i < g.n_nodes - 2) {
-      const int s = g.stride[i];
-      // middle or last node raised, node i lowered: the block with one photon more in node i
-      if (rc.up[i] != (R)0 && (im.kh[0][i] != 0.f || im.kh[1][i] != 0.f)) {
-        const R cm = (R)im.kh[0][i] * rc.up[i], cl = (R)im.kh[1][i] * rc.up[i];
-#pragma unroll
-        for (int m = 0; m < NP; ++m)
-#pragma unroll
-          for (int q = 0; q < NL; ++q) {
-            if (m == NC && q % NP == NC) continue;
-            const C w = v[base + s + m * NL + q];
-            if (m < NC) out[(m + 1) * NL + q] = rfma(cm * sqrt_n<R>(m + 1), w, out[(m + 1) * NL + q]);
-            if (q % NP < NC) out[m * NL + q + 1] = rfma(cl * sqrt_n<R>(q % NP + 1), w, out[m * NL + q + 1]);
-          }
-      }
-      // node i raised, middle or last node lowered
-      if (rc.dn[i] != (R)0 && (im.kh[2][i] != 0.f || im.kh[3][i] != 0.f)) {
-        const R cm = (R)im.kh[2][i] * rc.dn[i], cl = (R)im.kh[3][i] * rc.dn[i];
-#pragma unroll
-        for (int m = 0; m < NP; ++m)
-#pragma unroll
-          for (int q = 0; q < NL; ++q) {
-            if (m == 0 && q % NP == 0) continue;
-            const C w = v[base - s + m * NL + q];
-            if (m >= 1) out[(m - 1) * NL + q] = rfma(cm * sqrt_n<R>(m), w, out[(m - 1) * NL + q]);
-            if (q % NP >= 1) out[m * NL + q - 1] = rfma(cl * sqrt_n<R>(q % NP), w, out[m * NL + q - 1]);
-          }
-      }
+            out[m * NL + q] = add_re<TF>((cm * sqrt_n<R>(m)) * sqrt_n<R>(q % NP + 1), vk[(m - 1) * NL + q + 1], out[m * NL + q]);
     }
   }
 #pragma unroll
   for (int q = 0; q < E; ++q)
-    out[q] = diag_done(add_diag(Df[q / NL], acs_kd<R>(im, q % NL)), vk[q], prev[base + q], out[q]);
+    out[q] = diag_done<TF>(add_diag(Df[q / NL], acs_kd<R, TF>(im, q % NL)), vk[q], prev[base + q], out[q]);
 }
 
-template <typename R, int NC, class IT>
+template <typename R, int NC, bool TF, class IT>
 __device__ void cheb_run_blk(const KtGeom &g, const KtGenImage &im, const Smem &sm, const IT &it, int K,
                              typename C2<R>::T (&acc)[3 * (NC + 1) * (NC + 1)]) {
   typedef typename C2<R>::T C;
   constexpr int NP = NC + 1, NL = 3 * NP, E = NP * NL;
   C *P = (C *)sm.bufB;   // holds y_{k-1}; receives y_{k+1}
   C *Q = (C *)sm.bufA;   // holds y_k (this thread's block also in vk)
-  const R *cf = (const R *)sm.coef;
+  const Coef<R, TF> *cf = (const Coef<R, TF> *)sm.coef;
   const bool ok = it.ok(0);
   const int base = it.item(0), outer = g.n_nodes - 2;
   const uint32_t fdig = it.dig(0);
   Diag<R> Df[NP];
   BlkCache<R, NP> rc;
   C vk[E], out[E];
-  const R c0 = cf[0];
+  const Coef<R, TF> c0 = cf[0];
   if (ok) {
     load_blk<R, NC>(g, im, sm, fdig, rc);
     Diag<R> D{(R)0, (R)0, (R)0};
-    for (int i = 0; i < outer; ++i) D = add_diag(D, load_diag<R>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
+    for (int i = 0; i < outer; ++i) D = add_diag(D, load_diag<R, TF>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
 #pragma unroll
-    for (int m = 0; m < NP; ++m) Df[m] = add_diag(D, load_diag<R>(sm, outer * NL + ((fdig >> (4 * outer)) & 15) + m));
+    for (int m = 0; m < NP; ++m) Df[m] = add_diag(D, load_diag<R, TF>(sm, outer * NL + ((fdig >> (4 * outer)) & 15) + m));
   }
 #pragma unroll
   for (int q = 0; q < E; ++q) {
     vk[q] = ok ? Q[base + q] : mkc((R)0, (R)0);
-    acc[q] = mkc(c0 * vk[q].x, c0 * vk[q].y);
+    acc[q] = coef_mul(c0, vk[q]);
   }
   for (int k = 1; k < K; ++k) {
     if (ok) {
@@ -1362,20 +1430,21 @@ __device__ void cheb_run_blk(const KtGeom &g, const KtGenImage &im, const Smem &
 #pragma unroll
         for (int q = 0; q < E; ++q) P[base + q] = mkc((R)0, (R)0);
       }
-      apply_blk<R, NC>(g, im, sm, Q, P, base, Df, vk, out, rc);
-      const R a = cf[k], h = k == 1 ? (R)0.5 : (R)1;
+      apply_blk<R, NC, TF>(g, im, sm, Q, P, base, Df, vk, out, rc);
+      const Coef<R, TF> a = cf[k];
+      const R h = k == 1 ? (R)0.5 : (R)1;
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         vk[q] = mkc(h * out[q].x, h * out[q].y);
         P[base + q] = vk[q];
-        acc[q] = rfma(a, vk[q], acc[q]);
+        acc[q] = coef_fma(a, vk[q], acc[q]);
       }
     }
     __syncthreads();
     C *tmp = P; P = Q; Q = tmp;
   }
   if (K == 1) __syncthreads();
-  apply_phase<R, E>(g, sm, 0, acc, [&](int q) { return Df[q / NL].lo + acs_kd<R>(im, q % NL).lo; });
+  apply_phase<R, E, TF>(g, sm, 0, acc, [&](int q) { return Df[q / NL].lo + acs_kd<R, TF>(im, q % NL).lo; });
 }
 
 // --------------------------------------------------------------------------------------
@@ -1516,12 +1585,14 @@ template <typename R, int EPT, int NL, int ACS, bool CACHE, class IT>
 __device__ __forceinline__ void cheb_dispatch(const KtGeom &g, const KtGenImage &im, const Smem &sm,
                                               const IT &it, int K, typename C2<R>::T (&acc)[EPT]) {
   // ACS: 1 cavity structure, 2 the same with T = 1, 3 with real / imaginary couplings, 4 both
-  // 5 block mapping; 6, 7 row mapping (up to two nodes and one pair, three nodes and three pairs)
-  if constexpr (ACS == 6) cheb_run_row<R, 2, 1>(g, im, sm, it, K, acc);
-  else if constexpr (ACS == 7) cheb_run_row<R, 3, 3>(g, im, sm, it, K, acc);
-  else if constexpr (ACS == 5) cheb_run_blk<R, NL / 3 - 1>(g, im, sm, it, K, acc);
-  else if constexpr (ACS) cheb_run_acs<R, NL / 3 - 1, (ACS == 2 || ACS == 4) ? 1 : 0, (ACS >= 3), CACHE>(g, im, sm, it, K, acc);
-  else if constexpr (NL > 0) cheb_run_fiber<R, NL>(g, im, sm, it, K, acc);
+  // 5 block mapping; 6, 7 row mapping (up to two nodes and one pair, three nodes and three pairs); 11, 12, 13: 3, 4, 5 in the y form
+  constexpr int A = ACS >= 8 ? ACS - 8 : ACS;
+  constexpr bool TF = t_form<R, NL, ACS>();
+  if constexpr (A == 6) cheb_run_row<R, 2, 1>(g, im, sm, it, K, acc);
+  else if constexpr (A == 7) cheb_run_row<R, 3, 3>(g, im, sm, it, K, acc);
+  else if constexpr (A == 5) cheb_run_blk<R, NL / 3 - 1, TF>(g, im, sm, it, K, acc);
+  else if constexpr (A) cheb_run_acs<R, NL / 3 - 1, (A == 2 || A == 4) ? 1 : 0, (A >= 3), CACHE, TF>(g, im, sm, it, K, acc);
+  else if constexpr (NL > 0) cheb_run_fiber<R, NL, TF>(g, im, sm, it, K, acc);
   else cheb_run<R, EPT>(g, im, sm, it, K, acc);
 }
 
@@ -1562,6 +1633,25 @@ __host__ __device__ constexpr int kt_min_ctas(int rsize, int ept, int nl, int ma
 // of several jumps each in FP64 fell from 201 to 24 ms, 100 intervals of d = 729 with 3 % of 1024 trajectories
 // jumping from 82 to 27 ms.
 enum { PH_MAIN = 0, PH_ROOT, PH_SSTAR, PH_REST, PH_DONE };
+
+// This thread's part of its trajectory's norm^2: summed over a fiber (at most 16 elements) in the state precision, over a
+// block's fibers in FP64.
+template <typename R, int EPT, int NL, class IT>
+__device__ __forceinline__ double norm_part(const IT &it, const typename C2<R>::T (&v)[EPT]) {
+  constexpr int FB = NL > 0 ? NL : EPT;
+  double n = 0.0;
+#pragma unroll
+  for (int f = 0; f < EPT; f += FB) {
+    R s = 0;
+#pragma unroll
+    for (int q = f; q < f + FB; ++q)
+      if (it.ok(q)) s += v[q].x * v[q].x + v[q].y * v[q].y;
+    n = f == 0 ? (double)s : n + (double)s;
+  }
+  return n;
+}
+template <typename R, bool WIDE> struct SumT { typedef R T; };
+template <typename R> struct SumT<R, true> { typedef double T; };
 
 // Root of the cubic Hermite interpolant of a decreasing n on [0, len] with n(0) = n0 >= r >= n(len) = n1
 // and slopes -p0, -p1.
@@ -1701,21 +1791,30 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
       }
       bool jumped = false, stored = false;
 
-      // sum over channels of |L_l v|^2 at this thread's elements of tile vector v (FP32 partial sums)
+      // |L_l v|^2 at this thread's elements of tile vector v, summed over a fiber in the state precision (norm_part)
       // (the jump phases' loops stay rolled where an element's place is arithmetic: they are rare, and unrolled they
       // cost the series registers)
       constexpr int UJ = NL > 0 ? 1 : EPT;
-      auto loss = [&](const C *v) -> double {
+      auto channel = [&](int l, const C *v) -> double {
+        double n = 0.0;
         R s = 0;
-        for (int l = 0; l < g.n_lind; ++l) {
     #pragma unroll UJ
-          for (int q = 0; q < EPT; ++q)
-            if (it.ok(q)) {
-              const C y = lind_item<R>(g, ops, l, 0, v, it.item(q), it.dig(q));
-              s += y.x * y.x + y.y * y.y;
-            }
+        for (int q = 0; q < EPT; ++q) {
+          if (it.ok(q)) {
+            const C y = lind_item<R>(g, ops, l, 0, v, it.item(q), it.dig(q));
+            s += y.x * y.x + y.y * y.y;
+          }
+          if (NL > 0 && EPT > NL && q % (NL > 0 ? NL : 1) == NL - 1) {
+            n += (double)s;
+            s = 0;
+          }
         }
-        return (double)s;
+        return NL > 0 && EPT > NL ? n : (double)s;
+      };
+      auto loss = [&](const C *v) -> double {
+        double p = 0.0;
+        for (int l = 0; l < g.n_lind; ++l) p += channel(l, v);
+        return p;
       };
       int phase = (j >= 1) ? PH_MAIN : PH_DONE;
       if (phase == PH_DONE) {
@@ -1739,7 +1838,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           }
           if (phase == PH_MAIN) {
             if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, run, keep, extra, j);
-            else uniform_coefs<R>(g, sm, im, j);
+            else uniform_coefs<R, t_form<R, NL, ACS>()>(g, sm, im, j);
           } else {
             if (threadIdx.x < g.T) {
               const int t = threadIdx.x;
@@ -1752,7 +1851,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
             }
             load_tile<R, EPT>(g, it, psi_out, A);   // the main round's tile came by bulk copy
             __syncthreads();
-            piece_coefs<R>(g, im, sm, g.c_fwd);
+            piece_coefs<R, t_form<R, NL, ACS>()>(g, im, sm, g.c_fwd);
           }
           __syncthreads();
           cheb_dispatch<R, EPT, NL, ACS, false>(g, im, run, it, g.K, acc);
@@ -1783,19 +1882,18 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           } else {
             __syncthreads();
           }
-          R ns = 0;
+          const double ns = norm_part<R, EPT, NL>(it, acc);
+          // per-thread sums per control in the state precision, a fiber at a time (a trajectory problem has one term per
+          // control; a density matrix a ket and a bra term), converted to FP64 for the reduction
+          constexpr int FB = NL > 0 ? NL : EPT;                    // elements summed in the state precision
+          typedef typename SumT<R, (EPT > FB)>::T S;
+          S sc[KT_MAX_CTRL];
     #pragma unroll
-          for (int q = 0; q < EPT; ++q)
-            if (it.ok(q)) ns += acc[q].x * acc[q].x + acc[q].y * acc[q].y;
-          // per-thread sums per control in the state precision (a trajectory problem has one term per
-          // control; a density matrix a ket and a bra term), converted to FP64 once for the reduction
-          R sc[KT_MAX_CTRL];
-    #pragma unroll
-          for (int c = 0; c < KT_MAX_CTRL; ++c) sc[c] = (R)0;
+          for (int c = 0; c < KT_MAX_CTRL; ++c) sc[c] = (S)0;
           for (int t = 0; t < g.n_cterms && sum; ++t) {
             const int node = g.cterm_node[t];
             const C *hv = (const C *)sm.hc_val;
-            R s = 0;
+            S s = 0;
             // one pass per entry of a factor row, without branches (an empty entry has weight and offset zero), so
             // that the loads of all elements are in flight together
             for (int e = 0; e < g.SH; ++e) {
@@ -1805,18 +1903,28 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
                   const int b = (t * g.n_loc + ((it.dig(0) >> (4 * node)) & 15)) * g.SH + e, off = sm.hc_off[b];
                   const C w = hv[b];
     #pragma unroll
-                  for (int q = 0; q < EPT; ++q) {
-                    const C x = chi[it.item(q)], h = cmul(w, A[it.item(q) + off]);
-                    s += x.x * h.y - x.y * h.x;       // Im(conj(chi) * h)
+                  for (int f = 0; f < EPT; f += FB) {
+                    R sf = 0;
+    #pragma unroll
+                    for (int q = f; q < f + FB; ++q) {
+                      const C x = chi[it.item(q)], h = cmul(w, A[it.item(q) + off]);
+                      sf += x.x * h.y - x.y * h.x;       // Im(conj(chi) * h)
+                    }
+                    s += (S)sf;
                   }
                 }
               } else {
     #pragma unroll
-                for (int q = 0; q < EPT; ++q) {
-                  if (!it.ok(q)) continue;
-                  const int b = (t * g.n_loc + ((it.dig(q) >> (4 * node)) & 15)) * g.SH + e;
-                  const C x = chi[it.item(q)], h = cmul(hv[b], A[it.item(q) + sm.hc_off[b]]);
-                  s += x.x * h.y - x.y * h.x;
+                for (int f = 0; f < EPT; f += FB) {
+                  R sf = 0;
+    #pragma unroll
+                  for (int q = f; q < f + FB; ++q) {
+                    if (!it.ok(q)) continue;
+                    const int b = (t * g.n_loc + ((it.dig(q) >> (4 * node)) & 15)) * g.SH + e;
+                    const C x = chi[it.item(q)], h = cmul(hv[b], A[it.item(q) + sm.hc_off[b]]);
+                    sf += x.x * h.y - x.y * h.x;
+                  }
+                  s += (S)sf;
                 }
               }
             }
@@ -1829,22 +1937,22 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           // (FP64 runs at 1/64 of the FP32 rate here, and every slot costs additions in each lane)
           double nrm_t = 0.0;
           if (!sum) {
-            double v[1] = {(double)ns};
+            double v[1] = {ns};
             reduce_tau<1>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
             vstride = 1;
           } else if (g.n_ctrl <= 3) {
-            double v[4] = {(double)ns, (double)sc[0], (double)sc[1], (double)sc[2]};
+            double v[4] = {ns, (double)sc[0], (double)sc[1], (double)sc[2]};
             reduce_tau<4>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
             vstride = 4;
           } else if (g.n_ctrl < KT_MAX_CTRL) {
             double v[8];
-            v[0] = (double)ns;
+            v[0] = ns;
     #pragma unroll
             for (int c = 1; c < 8; ++c) v[c] = (double)sc[c - 1];
             reduce_tau<8>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
             vstride = 8;
           } else {
-            double n1[1] = {(double)ns};
+            double n1[1] = {ns};
             reduce_tau<1>(n1, g, sm.red, sm.tsc + TS_V0 * g.T);
             if (threadIdx.x < g.T) nrm_t = sm.tsc[TS_V0 * g.T + threadIdx.x];
             __syncthreads();
@@ -1892,15 +2000,11 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
         } else if (phase == PH_ROOT) {
           // n and p at the trial time: one Newton step, kept inside the bracket
           double v[2];
-          R s = 0;
     #pragma unroll
-          for (int q = 0; q < EPT; ++q) {
-            if (!it.ok(q)) continue;
-            A[it.item(q)] = acc[q];
-            s += acc[q].x * acc[q].x + acc[q].y * acc[q].y;
-          }
+          for (int q = 0; q < EPT; ++q)
+            if (it.ok(q)) A[it.item(q)] = acc[q];
           __syncthreads();
-          v[0] = (double)s;
+          v[0] = norm_part<R, EPT, NL>(it, acc);
           v[1] = loss(A);
           reduce_tau<2>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
           if (threadIdx.x < g.T) {
@@ -1938,18 +2042,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           __syncthreads();
           // channel probabilities p_l = ||L_l phi||^2
           double v[KT_MAX_LIND];
-          for (int l = 0; l < KT_MAX_LIND; ++l) {
-            R s = 0;
-            if (l < g.n_lind) {
-    #pragma unroll UJ
-              for (int q = 0; q < EPT; ++q)
-                if (it.ok(q)) {
-                  const C y = lind_item<R>(g, ops, l, 0, A, it.item(q), it.dig(q));
-                  s += y.x * y.x + y.y * y.y;
-                }
-            }
-            v[l] = (double)s;
-          }
+          for (int l = 0; l < KT_MAX_LIND; ++l) v[l] = l < g.n_lind ? channel(l, A) : 0.0;
           reduce_tau<KT_MAX_LIND>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
           if (threadIdx.x < g.T) {
             const int t = threadIdx.x, k = tile * g.T + t;
@@ -2013,12 +2106,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           phase = PH_REST;
           continue;
         } else {  // PH_REST
-          double v[1];
-          R s = 0;
-    #pragma unroll
-          for (int q = 0; q < EPT; ++q)
-            if (it.ok(q)) s += acc[q].x * acc[q].x + acc[q].y * acc[q].y;
-          v[0] = (double)s;
+          double v[1] = {norm_part<R, EPT, NL>(it, acc)};
           if (threadIdx.x == 0) sm.flag[2] = 0;
           reduce_tau<1>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
           if (threadIdx.x < g.T) {
@@ -2066,14 +2154,10 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           __syncthreads();
           load_tile<R, EPT>(g, it, psi_out, A);
           __syncthreads();
-          R s = 0;
     #pragma unroll
           for (int q = 0; q < EPT; ++q)
-            if (it.ok(q)) {
-              const C x = A[it.item(q)];
-              s += x.x * x.x + x.y * x.y;
-            }
-          v[1] = (double)s;
+            if (it.ok(q)) acc[q] = A[it.item(q)];
+          v[1] = norm_part<R, EPT, NL>(it, acc);
           v[2] = loss(A);
           v[3] = 0.0;
           reduce_tau<4>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
@@ -2348,7 +2432,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
         Smem run = sm;
         if (rounds == 0) {
           if constexpr (SWEEP) sweep_coefs<R>(g, im, sm, run, keep, extra, j);
-          else uniform_coefs<R>(g, sm, im, j);
+          else uniform_coefs<R, t_form<R, NL, ACS>()>(g, sm, im, j);
         } else if (threadIdx.x < g.T) {
           const int t = threadIdx.x, k = tile * g.T + t;
           double len = 0.0;
@@ -2368,7 +2452,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
         }
         if (rounds > 0) {
           __syncthreads();
-          piece_coefs<R>(g, im, sm, fw ? g.c_fwd : g.c_bwd);
+          piece_coefs<R, t_form<R, NL, ACS>()>(g, im, sm, fw ? g.c_fwd : g.c_bwd);
         }
         // B holds the vector to propagate (a sweep's later intervals start with it in A)
         if (!sweep || j == j_first || rnd > 0) {

@@ -9,6 +9,9 @@ namespace kt {
 template <typename R, int EPT, int NL, int ACS, int MAXT>
 static cudaError_t launch_fwd_t(const KtGeom &g, const KtGenImage &im, const KtOps &ops, const FwdArgs &a, size_t smem,
                                 cudaStream_t st, int *occ) {
+  if constexpr (NL > 0 && ACS >= 3 && ACS <= 5) {
+    if (a.y_form) return launch_fwd_t<R, EPT, NL, ACS + 8, MAXT>(g, im, ops, a, smem, st, occ);
+  }
   if (a.sweep || occ) {
     if constexpr (NL == 0) {
       const cudaError_t attr = kt_allow_large_smem((const void *)fwd_kernel<R, EPT, 0, ACS, true, MAXT>);

@@ -304,9 +304,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
       C acc[NL];
       if (threadIdx.x == 0) sm.tsc[TS_X] = sb(p + 1) - sb(p);
       __syncthreads();
-      piece_coefs<R>(g, imf, sm, g.c_fwd);
+      piece_coefs<R, false>(g, imf, sm, g.c_fwd);
       __syncthreads();
-      cheb_run_acs<R, NC, 1, true, false>(g, imf, sm, it, g.K, acc);
+      cheb_run_acs<R, NC, 1, true, false, false>(g, imf, sm, it, g.K, acc);
       if (ok) {
 #pragma unroll
         for (int e = 0; e < NL; ++e) A[base + e] = acc[e];
@@ -330,11 +330,11 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
     }
     // ---- y_0 .. y_{K-2} of piece q, each thread's fiber to its place in ybuf
     if (m == 0) {
-      uniform_coefs<R>(g, sm, imf, j);
+      uniform_coefs<R, false>(g, sm, imf, j);
     } else {
       if (threadIdx.x == 0) sm.tsc[TS_X] = sb(q + 1) - sb(q);
       __syncthreads();
-      piece_coefs<R>(g, imf, sm, g.c_fwd);
+      piece_coefs<R, false>(g, imf, sm, g.c_fwd);
     }
     RowCache<R> rc;
     Diag<R> Df{(R)0, (R)0, (R)0};
@@ -355,11 +355,11 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
       for (int n = 1; n < g.K - 1; ++n) {
         if (ok) {
           if (n == 1) {
-            apply_acs<R, NC, 1, true, true, false>(g, imf, sm, Q, Q, base, fdig, Df, vk, t, rc);
+            apply_acs<R, NC, 1, true, true, false, false>(g, imf, sm, Q, Q, base, fdig, Df, vk, t, rc);
 #pragma unroll
             for (int e = 0; e < NL; ++e) t[e] = mkc((R)0.5 * t[e].x, (R)0.5 * t[e].y);
           } else {
-            apply_acs<R, NC, 1, true, true, true>(g, imf, sm, Q, P, base, fdig, Df, vk, t, rc);
+            apply_acs<R, NC, 1, true, true, true, false>(g, imf, sm, Q, P, base, fdig, Df, vk, t, rc);
           }
 #pragma unroll
           for (int e = 0; e < NL; ++e) {
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(EPT == 4 ? 256 : 1024)
         const int p = adj ? m - step : step;
         if (threadIdx.x == 0) sm.tsc[TS_X] = sb(p + 1) - sb(p);
         __syncthreads();
-        piece_coefs<R>(g, imd, sm, adj ? g.c_bwd : g.c_fwd);
+        piece_coefs<R, false>(g, imd, sm, adj ? g.c_bwd : g.c_fwd);
         __syncthreads();
         cheb_run<R, EPT>(g, imd, sm, it, g.K, acc);
 #pragma unroll
@@ -537,11 +537,11 @@ __global__ void __launch_bounds__(EPT == 4 ? 256 : 1024)
     }
     // ---- derivative of piece q along every control: <W_q| dP(tau_q)/deps_c |Z_q>
     if (m == 0) {
-      uniform_coefs<R>(g, sm, imf, j);
+      uniform_coefs<R, false>(g, sm, imf, j);
     } else {
       if (threadIdx.x == 0) sm.tsc[TS_X] = sb(q + 1) - sb(q);
       __syncthreads();
-      piece_coefs<R>(g, imf, sm, g.c_fwd);
+      piece_coefs<R, false>(g, imf, sm, g.c_fwd);
     }
     for (int c = 0; c < g.n_ctrl; ++c) {
 #pragma unroll

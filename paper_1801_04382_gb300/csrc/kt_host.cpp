@@ -546,8 +546,9 @@ cudaError_t run_bwd(kt_problem *p, const BwdArgs &b, cudaStream_t st) {
   return kt_launch_density(p->fp64, 1, p->dens_g, p->im_bwd, p->ops, d, st);
 }
 
-kt_status launch_bwd_step(kt_problem *p, int j, const void *in, void *out, cudaStream_t st) {
+kt_status launch_bwd_step(kt_problem *p, int j, const void *in, void *out, cudaStream_t st, bool gradient = false) {
   BwdArgs b = bwd_args(p);
+  b.y_form = gradient;
   b.j = j;
   b.chi_in = in;
   b.chi_out = out;
@@ -692,6 +693,7 @@ kt_status enqueue_forward(kt_problem *p, int update, cudaStream_t st, bool save_
   FwdArgs a;
   kt_status s = fwd_begin(p, update, st, a);
   if (s != KT_OK) return s;
+  a.y_form = save_psi;
   const bool exchange = p->sharded && update && !p->cross;
   const size_t nloc = (size_t)p->g.n_tiles * p->g.n_ctrl;
   for (int j = 0; j <= p->nt; ++j) {
@@ -817,6 +819,7 @@ kt_status gradient_sweep(kt_problem *p, cudaStream_t st) {
         b.chi_out = (void *)psi_at(p, j, seg_a);
         b.cursor = p->fcursor;
         b.forward_replay = 1;
+        b.y_form = 1;
         b.jcount = p->jcount[prev];
         kt_status s = prof_begin(p, KT_PROF_BWD, st);
         if (s != KT_OK) return s;
@@ -835,7 +838,7 @@ kt_status gradient_sweep(kt_problem *p, cudaStream_t st) {
       KT_CUDA(kt_launch_grad(p->fp64, p->grad_ept, p->g1, p->g.T, p->g.tile_elems, p->im_fwd, p->im_bwd, p->ops, ga, st));
       if ((s = prof_end(p, st)) != KT_OK) return s;
       if (p->grad_ept < 0) continue;   // the reverse kernel has propagated the co-state
-      s = launch_bwd_step(p, j, p->chi_run[j & 1], p->chi_run[(j - 1) & 1], st);
+      s = launch_bwd_step(p, j, p->chi_run[j & 1], p->chi_run[(j - 1) & 1], st, true);
       if (s != KT_OK) return s;
     }
     seg_b = seg_a;
@@ -1829,8 +1832,15 @@ kt_status upload_image(kt_problem *p, const HostImage &h, KtGenImage &im, cudaSt
   for (int q = 0; q < KT_MAX_NL; ++q) {
     im.kd32[3 * q] = (float)h.kd[2 * q];
     kt_split(h.kd[2 * q + 1], &im.kd32[3 * q + 1], &im.kd32[3 * q + 2]);
+    im.ki32[q] = (float)h.kd[2 * q + 1];
   }
   for (int q = 0; q < 10; ++q) im.kh[q / 2][q % 2] = (float)h.kh[q / 2][q % 2];
+  for (int q = 0; q < 4; ++q) {
+    const double v = h.kh[q / 2 * 2][q % 2];
+    im.km[q / 2][q % 2][0] = (float)v;
+    im.km[q / 2][q % 2][1] = (float)(v * std::sqrt(2.0));
+    im.km[q / 2][q % 2][2] = (float)(v * 2.0);
+  }
   for (int q = 0; q < 4; ++q) {
     im.kc32[q] = (float)h.kc[q];
     im.kc64[q] = h.kc[q];

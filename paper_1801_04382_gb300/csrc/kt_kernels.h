@@ -57,12 +57,14 @@ struct FwdArgs {
   // update every CTA puts its partials of interval i into partials [nt][n_tiles][n_ctrl] (every bit set
   // at the launch: not there yet), and forms Delta eps from all tiles' partials in the finisher's order.
   int sweep;
+  int y_form;               // FP32 fibers and blocks: the y form of the series (sweeps that keep states for the gradient)
   void *psi_ring[2];
   const void *chi_slots;
   size_t slot_bytes;
 };
 
 struct BwdArgs {
+  int y_form;               // as in FwdArgs (the replays and co-states of the gradient)
   int j;                 // interval nt..1: chi(t_j) -> chi(t_{j-1})
   int nt;
   const void *chi_in;
