@@ -329,6 +329,7 @@ struct kt_problem {
   int final_buf = 0;
 
   // gradient (krotov_gradient): forward states kept every Kg intervals, replayed per segment
+  bool grad_set = false;        // every buffer below is there (grad_setup)
   int Kg = 0, grad_ept = 4;
   KtGeom g1{};                  // the geometry re-cut to one trajectory per CTA
   void *psi_ck = nullptr;       // [nt/Kg + 1] states: psi(t_{s Kg}), s >= 1 (s = 0 is psi_init)
@@ -729,9 +730,8 @@ kt_status forward_sweep(kt_problem *p, int update, cudaStream_t st, bool save_ps
   return KT_OK;
 }
 
-// Buffers and geometry of the gradient sweep (first use only).
-kt_status grad_setup(kt_problem *p, cudaStream_t st) {
-  if (p->psi_ck) return KT_OK;
+// Buffers and geometry of the gradient sweep.  May leave some of them allocated when it fails.
+kt_status grad_alloc(kt_problem *p, cudaStream_t st) {
   if (p->density) return fail(KT_ERR_UNSUPPORTED, "the frozen-record gradient is defined for trajectory problems");
   KtGeom g1 = p->g;
   g1.T = 1;
@@ -783,6 +783,28 @@ kt_status grad_setup(kt_problem *p, cudaStream_t st) {
   return KT_OK;
 }
 
+// The same on first use, all or nothing: after a failure (no room, most often) the problem holds none of them and the
+// next call starts anew.
+kt_status grad_setup(kt_problem *p, cudaStream_t st) {
+  if (p->grad_set) return KT_OK;
+  const size_t n0 = p->allocs.size(), b0 = p->bytes;
+  const kt_status s = grad_alloc(p, st);
+  if (s == KT_OK) {
+    p->grad_set = true;
+    return KT_OK;
+  }
+  cudaStreamSynchronize(st);    // the gradient's memset may be in flight
+  while (p->allocs.size() > n0) {
+    cudaFree(p->allocs.back());
+    p->allocs.pop_back();
+  }
+  p->bytes = b0;
+  p->psi_ck = p->psi_seg = p->yscratch = p->chi_run[0] = p->chi_run[1] = nullptr;
+  p->gpart = p->dgrad = nullptr;
+  p->fcursor = nullptr;
+  return s;
+}
+
 // state psi(t_j) of the recorded forward pass inside segment [a, b): checkpoint or replayed
 const void *psi_at(const kt_problem *p, int j, int seg_a) {
   if (j == seg_a) return seg_a == 0 ? p->psi_init : state_slot(p, p->psi_ck, seg_a / p->Kg);
@@ -791,7 +813,8 @@ const void *psi_at(const kt_problem *p, int j, int seg_a) {
 
 // dJ_T/deps of the last (mode 2) forward sweep with its jump record frozen.
 kt_status gradient_sweep(kt_problem *p, cudaStream_t st) {
-  if (!p->grad_ready) return fail(KT_ERR_STATE, "krotov_gradient needs propagate_forward(p, 2, ...) first");
+  if (!p->grad_set || !p->grad_ready)
+    return fail(KT_ERR_STATE, "krotov_gradient needs propagate_forward(p, 2, ...) first");
   const int prev = 1 - p->cur;
   KT_CUDA(kt_launch_chi_grad_boundary(p->fp64, p->g, p->ops, p->tau, p->norm2, p->psi[p->final_buf],
                                       p->chi_run[p->nt & 1], st));

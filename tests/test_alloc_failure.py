@@ -1,0 +1,126 @@
+"""Failed device allocations in the gradient's set-up, on the host: the library runs in a child process against a
+stand-in for the CUDA runtime (host memory, kernels that do nothing) whose n-th allocation fails."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+from paper_1801_04382_gb300 import build as pkg_build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+FAKE = r"""
+#include <stdlib.h>
+#include <string.h>
+typedef int E; typedef void *P; typedef size_t Z;
+static int left = -1, made = 0, launches = 0;
+void fake_fail_in(int n) { left = n; }
+int fake_mallocs(void) { return made; }
+int fake_launches(void) { return launches; }
+E cudaMalloc(P *p, Z n) { if (left > 0 && --left == 0) { *p = 0; return 2; } ++made; *p = calloc(1, n); return *p ? 0 : 2; }
+E cudaFree(P p) { free(p); return 0; }
+E cudaMemcpy(P d, const void *s, Z n, int k) { (void)k; if (n && (!d || !s)) return 1; memcpy(d, s, n); return 0; }
+E cudaMemcpyAsync(P d, const void *s, Z n, int k, P st) { (void)st; return cudaMemcpy(d, s, n, k); }
+E cudaMemsetAsync(P d, int v, Z n, P st) { (void)st; if (n && !d) return 1; memset(d, v, n); return 0; }
+E cudaMemGetInfo(Z *f, Z *t) { *f = *t = (Z)8 << 30; return 0; }
+E cudaGetDevice(int *d) { *d = 0; return 0; }
+E cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
+E cudaGetLastError(void) { return 0; }
+const char *cudaGetErrorString(E e) { (void)e; return "stand-in"; }
+E cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
+E cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int b, Z s, unsigned g)
+{ (void)f; (void)b; (void)s; (void)g; *n = 1; return 0; }
+E cudaGetSymbolAddress(P *p, const void *s) { (void)s; static char mem[1 << 20]; *p = mem; return 0; }
+E cudaStreamSynchronize(P s) { (void)s; return 0; }
+E cudaStreamCreateWithFlags(P *s, unsigned f) { (void)f; *s = malloc(1); return 0; }
+E cudaStreamDestroy(P s) { free(s); return 0; }
+E cudaEventCreate(P *s) { *s = malloc(1); return 0; }
+E cudaEventCreateWithFlags(P *s, unsigned f) { (void)f; *s = malloc(1); return 0; }
+E cudaEventDestroy(P s) { free(s); return 0; }
+E cudaLaunchKernelExC(const void *c, const void *f, P *a) { (void)c; (void)f; (void)a; ++launches; return 0; }
+E __cudaLaunchKernel(void) { ++launches; return 0; }
+E __cudaGetKernel(P *k, const void *f) { *k = (P)f; return 0; }
+E __cudaPopCallConfiguration(void) { return 0; }
+E __cudaPushCallConfiguration(void) { return 0; }
+P *__cudaRegisterFatBinary(P f) { (void)f; static P h; return &h; }
+void __cudaRegisterFatBinaryEnd(P *h) { (void)h; }
+void __cudaRegisterFunction(void) {}
+void __cudaRegisterVar(void) {}
+void __cudaUnregisterFatBinary(P *h) { (void)h; }
+"""
+
+CHILD = r"""
+import ctypes as ct, sys
+import numpy as np
+from paper_1801_04382_gb300 import KrotovError, Problem, cascaded_chain
+fake = ct.CDLL(sys.argv[1])
+N, nc, precision, strided = int(sys.argv[2]), int(sys.argv[3]), sys.argv[4], sys.argv[5] == "strided"
+nt, M = 4, 2
+net = cascaded_chain(N, nc)
+
+
+def problem():
+    eps = np.ones((N, nt))
+    return Problem(net, 0.04, nt, M, eps, eps, np.full(N, 10.0), np.full((3, M, 1 + 2 * N * (nc + 1)), 0.5), precision=precision)
+
+
+def gradient(p):
+    out = np.zeros((N, nt))
+    return p._lib.krotov_gradient(p._h, None, out.ctypes.data_as(ct.c_void_p), None)
+
+
+p = problem()
+n0, clean = fake.fake_mallocs(), p.info.device_bytes
+p.forward(keep_for_gradient=True)
+assert gradient(p) == 0
+steps, full = fake.fake_mallocs() - n0, p.get_info().device_bytes
+assert steps >= 7 and full > clean
+p.forward(keep_for_gradient=True)
+assert fake.fake_mallocs() == n0 + steps            # a second sweep allocates nothing
+p.close()
+for n in range(1, steps + 1):
+    p = problem()
+    fake.fake_fail_in(n)
+    try:
+        p.forward(keep_for_gradient=True)
+        assert n == steps and strided, n            # no room for the series' terms: the strided kernel
+        assert gradient(p) == 0
+        p.close()
+        continue
+    except KrotovError as e:
+        assert "KT_ERR_OOM" in str(e), e
+    assert p.get_info().device_bytes == clean       # nothing half set up
+    before, ran = fake.fake_mallocs(), fake.fake_launches()
+    assert gradient(p) != 0 and fake.fake_launches() == ran
+    fake.fake_fail_in(n)                            # again without room: refused again
+    try:
+        p.forward(keep_for_gradient=True)
+        raise SystemExit(f"allocation {n}: the second call went through")
+    except KrotovError as e:
+        assert "KT_ERR_OOM" in str(e), e
+    assert fake.fake_launches() == ran
+    fake.fake_fail_in(-1)
+    before = fake.fake_mallocs()
+    p.forward(keep_for_gradient=True)               # with room: a set-up from the beginning
+    assert fake.fake_mallocs() - before == steps and p.get_info().device_bytes == full
+    assert gradient(p) == 0
+    p.close()
+print("ok")
+"""
+
+
+@pytest.mark.parametrize("N,nc,precision,fallback", [(4, 2, "fp64", "refused"), (3, 2, "fp32", "strided")])
+def test_gradient_setup_is_all_or_nothing(tmp_path, N, nc, precision, fallback):
+    if not shutil.which("gcc"):
+        pytest.skip("no C compiler")
+    if not os.path.exists(pkg_build.lib_path()):
+        pkg_build.build()
+    src, so = tmp_path / "fake_cudart.c", tmp_path / "libfake_cudart.so"
+    src.write_text(FAKE)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-w", str(src), "-o", str(so)], check=True)
+    env = dict(os.environ, LD_PRELOAD=str(so), PYTHONPATH=ROOT)
+    res = subprocess.run([sys.executable, "-c", CHILD, str(so), str(N), str(nc), precision, fallback], env=env,
+                         capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and res.stdout.strip() == "ok", res.stdout + res.stderr
