@@ -730,21 +730,38 @@ kt_status forward_sweep(kt_problem *p, int update, cudaStream_t st, bool save_ps
   return KT_OK;
 }
 
-// Buffers and geometry of the gradient sweep.  May leave some of them allocated when it fails.
-kt_status grad_alloc(kt_problem *p, cudaStream_t st) {
-  if (p->density) return fail(KT_ERR_UNSUPPORTED, "the frozen-record gradient is defined for trajectory problems");
+// Geometry of the gradient kernels: one trajectory per CTA, one thread per last-node fiber (the reverse kernel).
+KtGeom grad_geom(const kt_problem *p) {
   KtGeom g1 = p->g;
   g1.T = 1;
   g1.n_tiles = p->M;
   g1.M_pad = p->M;
   g1.tile_elems = (g1.d + 3) / 4 * 4;
   g1.prefetch_chi = 0;
+  g1.nthreads = std::max(32, (g1.d / g1.n_loc + 31) / 32 * 32);
+  return g1;
+}
+
+// The reverse kernel applies: its structure (plan()), one CTA per trajectory, two state buffers in shared memory.
+bool grad_reverse_fits(const kt_problem *p, const KtGeom &g1) {
+  return p->grad_reverse && g1.nthreads <= 736 && kt_grad_smem_bytes(g1, (int)p->esz, true) <= 227 * 1024;
+}
+
+// Bytes of the reverse kernel's series' terms (0: it does not apply).
+size_t grad_term_bytes(const kt_problem *p) {
+  const KtGeom g1 = grad_geom(p);
+  return grad_reverse_fits(p, g1) ? (size_t)p->M * g1.K * g1.n_loc * g1.nthreads * p->esz : 0;
+}
+
+// Buffers and geometry of the gradient sweep.  May leave some of them allocated when it fails.
+kt_status grad_alloc(kt_problem *p, cudaStream_t st) {
+  if (p->density) return fail(KT_ERR_UNSUPPORTED, "the frozen-record gradient is defined for trajectory problems");
+  KtGeom g1 = grad_geom(p);
   // cavity structure with real / imaginary coupling classes and drive controls: the reverse kernel, one thread per
   // last-node fiber, its series' terms in global memory; otherwise 4 items per thread up to 256 threads, else 8
   // up to 1024
   int ept = -g1.n_loc;
-  g1.nthreads = std::max(32, (g1.d / g1.n_loc + 31) / 32 * 32);
-  bool reverse = p->grad_reverse && g1.nthreads <= 736 && kt_grad_smem_bytes(g1, (int)p->esz, true) <= 227 * 1024;
+  const bool reverse = grad_reverse_fits(p, g1);
   KtGeom gs = g1;               // the strided kernel's geometry
   const int epts = (g1.d + 3) / 4 <= 256 ? 4 : 8;
   gs.nthreads = std::max(32, ((g1.d + epts - 1) / epts + 31) / 32 * 32);
@@ -773,8 +790,7 @@ kt_status grad_alloc(kt_problem *p, cudaStream_t st) {
   if ((s = dev_alloc(p, (void **)&p->dgrad, (size_t)p->g.n_ctrl * p->nt * sizeof(double))) != KT_OK) return s;
   if ((s = dev_alloc(p, (void **)&p->fcursor, (size_t)p->g.M_pad * sizeof(int))) != KT_OK) return s;
   KT_CUDA(cudaMemsetAsync(p->dgrad, 0, (size_t)p->g.n_ctrl * p->nt * sizeof(double), st));
-  if (reverse &&
-      (s = dev_alloc(p, &p->yscratch, (size_t)p->M * g1.K * g1.n_loc * g1.nthreads * p->esz)) != KT_OK) {
+  if (reverse && (s = dev_alloc(p, &p->yscratch, grad_term_bytes(p))) != KT_OK) {
     if (!strided_fits) return s;
     cudaGetLastError();         // no room for the series' terms: the strided kernel needs none
     p->g1 = gs;
@@ -1883,13 +1899,15 @@ namespace {
 // co-state if they fit, else the longest prefix t_0..t_A plus checkpoints every K after it, with
 // (A, K) chosen to recompute the fewest co-states (every co-state not kept is recomputed once per
 // forward sweep, so the count is about nt + 1 minus the slots kept).  A reserve stays free: 2 GiB
-// or 2 % of the device, and room for the forward states a gradient sweep keeps (2 sqrt(nt) + 4).
+// or 2 % of the device, room for the forward states a gradient sweep keeps (2 sqrt(nt) + 4) and, where the reverse
+// gradient kernel applies, for its series' terms (about K states more).
 kt_status choose_storage(kt_problem *p) {
   size_t free_b = 0, total_b = 0;
   KT_CUDA(cudaMemGetInfo(&free_b, &total_b));
   const int nt = p->nt;
   const long long reserve = std::max<long long>(2LL << 30, (long long)(total_b / 50)) +
-                            (long long)(2.0 * std::sqrt((double)nt) + 4.0) * (long long)p->state_bytes;
+                            (long long)(2.0 * std::sqrt((double)nt) + 4.0) * (long long)p->state_bytes +
+                            (long long)grad_term_bytes(p);
   const long long budget = ((long long)free_b - reserve) / (long long)p->state_bytes;
   p->ckpt_auto = true;
   if (budget >= nt + 1) {

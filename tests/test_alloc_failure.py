@@ -1,5 +1,5 @@
-"""Failed device allocations in the gradient's set-up, on the host: the library runs in a child process against a
-stand-in for the CUDA runtime (host memory, kernels that do nothing) whose n-th allocation fails."""
+"""Device memory of the gradient's set-up, on the host: the library runs in a child process against a stand-in for the
+CUDA runtime (host memory, kernels that do nothing) whose n-th allocation fails, or whose memory is small."""
 import os
 import shutil
 import subprocess
@@ -16,15 +16,27 @@ FAKE = r"""
 #include <string.h>
 typedef int E; typedef void *P; typedef size_t Z;
 static int left = -1, made = 0, launches = 0;
+static Z total = (Z)8 << 30, used = 0;
+void fake_set_total(Z n) { total = n; }
 void fake_fail_in(int n) { left = n; }
 int fake_mallocs(void) { return made; }
 int fake_launches(void) { return launches; }
-E cudaMalloc(P *p, Z n) { if (left > 0 && --left == 0) { *p = 0; return 2; } ++made; *p = calloc(1, n); return *p ? 0 : 2; }
-E cudaFree(P p) { free(p); return 0; }
+E cudaMalloc(P *p, Z n)
+{
+  *p = 0;
+  if ((left > 0 && --left == 0) || used + n > total) return 2;
+  Z *h = calloc(1, n + 256);
+  if (!h) return 2;
+  ++made;
+  used += *h = n;
+  *p = (char *)h + 256;
+  return 0;
+}
+E cudaFree(P p) { if (p) { Z *h = (Z *)((char *)p - 256); used -= *h; free(h); } return 0; }
 E cudaMemcpy(P d, const void *s, Z n, int k) { (void)k; if (n && (!d || !s)) return 1; memcpy(d, s, n); return 0; }
 E cudaMemcpyAsync(P d, const void *s, Z n, int k, P st) { (void)st; return cudaMemcpy(d, s, n, k); }
 E cudaMemsetAsync(P d, int v, Z n, P st) { (void)st; if (n && !d) return 1; memset(d, v, n); return 0; }
-E cudaMemGetInfo(Z *f, Z *t) { *f = *t = (Z)8 << 30; return 0; }
+E cudaMemGetInfo(Z *f, Z *t) { *t = total; *f = total - used; return 0; }
 E cudaGetDevice(int *d) { *d = 0; return 0; }
 E cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
 E cudaGetLastError(void) { return 0; }
@@ -111,8 +123,28 @@ print("ok")
 """
 
 
-@pytest.mark.parametrize("N,nc,precision,fallback", [(4, 2, "fp64", "refused"), (3, 2, "fp32", "strided")])
-def test_gradient_setup_is_all_or_nothing(tmp_path, N, nc, precision, fallback):
+ROOM = r"""
+import ctypes as ct, sys
+import numpy as np
+from paper_1801_04382_gb300 import Problem, cascaded_chain
+fake = ct.CDLL(sys.argv[1])
+fake.fake_set_total.argtypes = [ct.c_size_t]
+fake.fake_set_total(14 << 30)
+N, nc, nt, M = 3, 2, 200, 24000
+eps = np.ones((N, nt))
+p = Problem(cascaded_chain(N, nc), 0.025 * nt, nt, M, eps, eps, np.full(N, 10.0), np.full((1, M, 3), 0.5), precision="fp32",
+            ckpt_interval=-1)
+assert 0 < p.info.costate_slots <= nt               # the co-states fill what is left of the device
+before = p.info.device_bytes
+p.forward(keep_for_gradient=True)
+terms = M * p.info.cheb_terms * 9 * 96 * 8          # the reverse kernel's: one place per element, thread and term
+states = (200 // 14 + 1 + 14 + 2) * M * 729 * 8      # kept every 14 intervals, replayed, and two co-states
+assert p.get_info().device_bytes - before >= states + terms, (p.get_info().device_bytes - before, states, terms)
+print("ok")
+"""
+
+
+def run_child(tmp_path, code, *args):
     if not shutil.which("gcc"):
         pytest.skip("no C compiler")
     if not os.path.exists(pkg_build.lib_path()):
@@ -121,6 +153,15 @@ def test_gradient_setup_is_all_or_nothing(tmp_path, N, nc, precision, fallback):
     src.write_text(FAKE)
     subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-w", str(src), "-o", str(so)], check=True)
     env = dict(os.environ, LD_PRELOAD=str(so), PYTHONPATH=ROOT)
-    res = subprocess.run([sys.executable, "-c", CHILD, str(so), str(N), str(nc), precision, fallback], env=env,
+    res = subprocess.run([sys.executable, "-c", code, str(so), *[str(a) for a in args]], env=env,
                          capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and res.stdout.strip() == "ok", res.stdout + res.stderr
+
+
+@pytest.mark.parametrize("N,nc,precision,fallback", [(4, 2, "fp64", "refused"), (3, 2, "fp32", "strided")])
+def test_gradient_setup_is_all_or_nothing(tmp_path, N, nc, precision, fallback):
+    run_child(tmp_path, CHILD, N, nc, precision, fallback)
+
+
+def test_automatic_storage_leaves_room_for_the_gradient(tmp_path):
+    run_child(tmp_path, ROOM)
