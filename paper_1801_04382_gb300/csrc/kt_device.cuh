@@ -1628,7 +1628,8 @@ __host__ __device__ constexpr int kt_min_ctas(int rsize, int ept, int nl, int ma
 // The jump time: the norm falls at the loss rate, dn/ds = -p(s), p = sum_l ||L_l psi(s)||^2, so each trial
 // series gives value and slope.  The first trial is the root of the cubic through (n, p) at both ends of
 // the piece, whose error is of order dt^4; a step is taken as the answer once its own error, curvature times
-// its square, is below tol, and a step that leaves the bracket is replaced by the bracket's middle.  One or two
+// its square, is below tol, and a step that leaves the bracket is replaced by the bracket's middle.  The state at the
+// time taken, which the collapse needs anyway, has to have the norm r; else the search goes on from there.  One or two
 // series where the bisection to 2^-48 dt (2^-40 in FP32) took 48 (40): a Krotov pass over d = 81 with 128 trajectories
 // of several jumps each in FP64 fell from 201 to 24 ms, 100 intervals of d = 729 with 3 % of 1024 trajectories
 // jumping from 82 to 27 ms.
@@ -1686,7 +1687,8 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
   char *const extra = smem_raw + carve(g, sizeof(C), smem_raw, &sm, g.prefetch_chi != 0, persist);
   const int tau = threadIdx.x % g.T;
   // error allowed to the jump time: 2^-50 dt in FP64 (near the rounding of the FP64 norm that decides it),
-  // 2^-32 dt in FP32-mixed (far below the FP32 norm's own error)
+  // 2^-32 dt in FP32-mixed (the FP32 norm's rounding, 2^-24 and more over a loss of 1e-3 ... 1e-2 per interval, leaves
+  // the time uncertain by 1e-5 dt: steps do not get smaller than that, and 2^-40 dt was not reached in 60 trials)
   const double tol = (sizeof(R) == 8 ? 0x1p-50 : 0x1p-32) * g.dt;
   int j = a.j;
 
@@ -1816,6 +1818,27 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
         for (int l = 0; l < g.n_lind; ++l) p += channel(l, v);
         return p;
       };
+      // One step of the root search of trajectory t from n - r = f and the loss rate p at the trial time TS_S, kept inside
+      // the bracket: the next trial, or (TI_BUSY 0) the time taken, in TS_S.
+      auto newton = [&](int t, double f, double p) {
+        const double s0 = sm.tsc[TS_S * g.T + t], ps = sm.tsc[TS_PS * g.T + t], pp = sm.tsc[TS_PP * g.T + t];
+        double lo = sm.tsc[TS_LO * g.T + t], hi = sm.tsc[TS_HI * g.T + t];
+        if (f <= 0.0) hi = s0;
+        else lo = s0;
+        const double step = f / p, next = s0 + step, mid = 0.5 * (lo + hi);
+        const int tries = sm.tin[TI_CH * g.T + t] + 1;
+        const bool in = p > 0.0 && next >= lo && next <= hi;
+        // what Newton's step leaves: |n'' / (2 n')| step^2, n'' from the two latest slopes
+        const double left = fabs((p - pp) / (s0 - ps)) * step * step / p;
+        const bool small = in && (left <= tol || fabs(step) <= tol), spent = hi - lo <= tol || tries >= 60;
+        sm.tsc[TS_LO * g.T + t] = lo;
+        sm.tsc[TS_HI * g.T + t] = hi;
+        sm.tsc[TS_PS * g.T + t] = s0;
+        sm.tsc[TS_PP * g.T + t] = p;
+        sm.tsc[TS_S * g.T + t] = in ? next : (spent ? hi : mid);
+        sm.tin[TI_BUSY * g.T + t] = !small && !spent;
+        sm.tin[TI_CH * g.T + t] = spent ? 60 : tries;    // 60: nothing left to try
+      };
       int phase = (j >= 1) ? PH_MAIN : PH_DONE;
       if (phase == PH_DONE) {
     #pragma unroll
@@ -1845,7 +1868,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
               const bool act = sm.tin[TI_ACT * g.T + t] != 0;
               double len = 0.0;
               if (phase == PH_ROOT) len = act && sm.tin[TI_BUSY * g.T + t] ? sm.tsc[TS_S * g.T + t] : 0.0;
-              else if (phase == PH_SSTAR) len = act ? sm.tsc[TS_HI * g.T + t] : 0.0;
+              else if (phase == PH_SSTAR) len = act ? sm.tsc[TS_S * g.T + t] : 0.0;
               else len = act ? g.dt - sm.tsc[TS_S0 * g.T + t] : 0.0;
               sm.tsc[TS_X * g.T + t] = len;
             }
@@ -2009,29 +2032,8 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
           reduce_tau<2>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
           if (threadIdx.x < g.T) {
             const int t = threadIdx.x;
-            if (sm.tin[TI_ACT * g.T + t] && sm.tin[TI_BUSY * g.T + t]) {
-              const double s0 = sm.tsc[TS_S * g.T + t], ps = sm.tsc[TS_PS * g.T + t], pp = sm.tsc[TS_PP * g.T + t];
-              const double f = sm.tsc[TS_V0 * g.T + 2 * t] - sm.tsc[TS_R * g.T + t], p = sm.tsc[TS_V0 * g.T + 2 * t + 1];
-              double lo = sm.tsc[TS_LO * g.T + t], hi = sm.tsc[TS_HI * g.T + t];
-              if (f <= 0.0) hi = s0;
-              else lo = s0;
-              const double step = f / p, next = s0 + step, mid = 0.5 * (lo + hi);
-              const int tries = sm.tin[TI_CH * g.T + t] + 1;
-              const bool in = p > 0.0 && next >= lo && next <= hi;
-              // what Newton's step leaves: |n'' / (2 n')| step^2, n'' from the two latest slopes
-              const double left = fabs((p - pp) / (s0 - ps)) * step * step / p;
-              sm.tin[TI_CH * g.T + t] = tries;
-              if ((in && (left <= tol || fabs(step) <= tol)) || hi - lo <= tol || tries >= 60) {
-                sm.tsc[TS_HI * g.T + t] = in ? next : hi;
-                sm.tin[TI_BUSY * g.T + t] = 0;
-              } else {
-                sm.tsc[TS_LO * g.T + t] = lo;
-                sm.tsc[TS_HI * g.T + t] = hi;
-                sm.tsc[TS_PS * g.T + t] = s0;
-                sm.tsc[TS_PP * g.T + t] = p;
-                sm.tsc[TS_S * g.T + t] = in ? next : mid;
-              }
-            }
+            if (sm.tin[TI_ACT * g.T + t] && sm.tin[TI_BUSY * g.T + t])
+              newton(t, sm.tsc[TS_V0 * g.T + 2 * t] - sm.tsc[TS_R * g.T + t], sm.tsc[TS_V0 * g.T + 2 * t + 1]);
           }
           __syncthreads();
           continue;
@@ -2039,11 +2041,33 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
     #pragma unroll
           for (int q = 0; q < EPT; ++q)
             if (it.ok(q)) A[it.item(q)] = acc[q];
+          if (threadIdx.x == 0) sm.flag[1] = 0;
+          __syncthreads();
+          double nv[1] = {norm_part<R, EPT, NL>(it, acc)};
+          reduce_tau<1>(nv, g, sm.red, sm.tsc + TS_V0 * g.T);
+          const double nstar = threadIdx.x < g.T ? sm.tsc[TS_V0 * g.T + threadIdx.x] : 0.0;
           __syncthreads();
           // channel probabilities p_l = ||L_l phi||^2
           double v[KT_MAX_LIND];
           for (int l = 0; l < KT_MAX_LIND; ++l) v[l] = l < g.n_lind ? channel(l, A) : 0.0;
           reduce_tau<KT_MAX_LIND>(v, g, sm.red, sm.tsc + TS_V0 * g.T);
+          // the norm there is r to its own rounding (one of its type per term), or this was a trial like the others: the
+          // estimate of what a step leaves can be wrong, two slopes may agree by chance
+          if (threadIdx.x < g.T && sm.tin[TI_ACT * g.T + threadIdx.x] && !g.first_order) {
+            const int t = threadIdx.x;
+            const double f = nstar - sm.tsc[TS_R * g.T + t];
+            if (fabs(f) > (sizeof(R) == 8 ? 0x1p-52 : 0x1p-23) * g.K && sm.tin[TI_CH * g.T + t] < 60) {
+              double p = 0.0;
+              for (int l = 0; l < g.n_lind; ++l) p += sm.tsc[TS_V0 * g.T + t * KT_MAX_LIND + l];
+              newton(t, f, p);
+              sm.flag[1] = 1;
+            }
+          }
+          __syncthreads();
+          if (sm.flag[1]) {
+            phase = PH_ROOT;
+            continue;
+          }
           if (threadIdx.x < g.T) {
             const int t = threadIdx.x, k = tile * g.T + t;
             int ch = -1;
@@ -2073,7 +2097,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
                   ch = -1;
                 } else {
                   const double cnorm = 1.0 / sqrt(p[ch]);
-                  const double sstar = sm.tsc[TS_S0 * g.T + t] + sm.tsc[TS_HI * g.T + t];
+                  const double sstar = sm.tsc[TS_S0 * g.T + t] + sm.tsc[TS_S * g.T + t];
                   const size_t ri = (size_t)k * g.max_jumps + (m - 1);
                   a.rec_step[ri] = j;
                   a.rec_ch[ri] = ch;
@@ -2167,7 +2191,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
             const double *o = sm.tsc + TS_V0 * g.T + 4 * t;
             sm.tsc[TS_LO * g.T + t] = 0.0;
             sm.tsc[TS_HI * g.T + t] = len;
-            sm.tsc[TS_S * g.T + t] = hermite_root(o[1], n1, o[2], o[0], len, sm.tsc[TS_R * g.T + t]);
+            sm.tsc[TS_S * g.T + t] = g.first_order ? len : hermite_root(o[1], n1, o[2], o[0], len, sm.tsc[TS_R * g.T + t]);
             sm.tsc[TS_PS * g.T + t] = len;
             sm.tsc[TS_PP * g.T + t] = o[0];
             sm.tin[TI_CH * g.T + t] = 0;                     // trials of the root search
