@@ -1,6 +1,7 @@
 // Internal definitions shared by the host runtime and the CUDA kernels.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 
 #ifdef __CUDACC__
@@ -47,35 +48,74 @@
 // started far above the wanted orders from (0, tiny) and normalised with the Neumann
 // identity J_0 + 2 sum_{m >= 1} J_{2m} = 1 (J.C.P. Miller, 1952; Numerical Recipes' bessj).
 // Values are rescaled whenever they grow past 1e150 so that tiny alpha cannot overflow.
-KT_HD int kt_bessel_miller(double alpha, int n, double *out) {
-  if (n < 1 || n > 256 || !(alpha >= 0.0)) return -1;
-  if (alpha < 1e-290) {
-    out[0] = 1.0;
-    for (int k = 1; k < n; ++k) out[k] = 0.0;
+template <typename F>
+inline int kt_bessel_miller(F alpha, int n, F *out) {
+  if (n < 1 || n > 256 || !(alpha >= 0)) return -1;
+  if (alpha < (F)1e-290) {
+    out[0] = 1;
+    for (int k = 1; k < n; ++k) out[k] = 0;
     return 0;
   }
   int start = n + 20 + (int)(alpha);
   start += (start & 1);                 // even start keeps the Neumann sum bookkeeping simple
-  for (int k = 0; k < n; ++k) out[k] = 0.0;
-  double jp1 = 0.0, jk = 1e-200, norm = 0.0;
-  const double inv = 2.0 / alpha;
-  const bool small = alpha < 1.0 || start > 140;   // else J_start / J_0 > 1e-290 and nothing overflows
+  for (int k = 0; k < n; ++k) out[k] = 0;
+  F jp1 = 0, jk = (F)1e-200, norm = 0;
+  const F inv = 2 / alpha;
   for (int k = start; k >= 1; --k) {
-    double jm1 = (double)k * inv * jk - jp1;
+    F jm1 = (F)k * inv * jk - jp1;
     jp1 = jk;
     jk = jm1;                            // jk now holds J_{k-1}
     int km1 = k - 1;
     if (km1 < n) out[km1] = jk;
-    if (km1 > 0 && (km1 & 1) == 0) norm += 2.0 * jk;
-    if (small && (jk > 1e150 || jk < -1e150)) {
-      jk *= 1e-150; jp1 *= 1e-150; norm *= 1e-150;
-      for (int q = km1; q < n; ++q) out[q] *= 1e-150;
+    if (km1 > 0 && (km1 & 1) == 0) norm += 2 * jk;
+    if (jk > (F)1e150 || jk < (F)-1e150) {
+      jk *= (F)1e-150; jp1 *= (F)1e-150; norm *= (F)1e-150;
+      for (int q = km1; q < n; ++q) out[q] *= (F)1e-150;
     }
   }
   norm += jk;                            // + J_0
-  const double s = 1.0 / norm;
+  const F s = 1 / norm;
   for (int k = 0; k < n; ++k) out[k] *= s;
   return 0;
+}
+
+// Coefficients m_k = (2 - delta_k0) J_k(r s) of a piece of an interval: Taylor series about the middle of the unit segment
+// of r s, |x| <= 1/2, cut at KT_PIECE_DEG (what is left is below 2 (1/2)^16 / 16! = 1.5e-18).  The segment's middle is
+// exact, so x = r s - middle is rounded at its own size and the value is as good as the table's: Miller's recurrence at
+// the middle, in long double because its error grows with the argument (5e-15 at r s = 60 in double).  (Chebyshev series over the whole interval, summed by Clenshaw's recurrence, were off by
+// 1.5e-15 ... 3e-15 up to K = 36 and 1.3e-14 at r dt = 60.)
+#define KT_PIECE_DEG 15
+inline int kt_piece_segments(double alpha_max) { return alpha_max > 1.0 ? (int)std::ceil(alpha_max) : 1; }
+// out[segment][n][k], n <= KT_PIECE_DEG, k < K <= KT_MAX_K: with J_k' = (J_{k-1} - J_{k+1}) / 2,
+// J_k^(n) = 2^-n sum_i (-1)^i C(n, i) J_{k-n+2i}, J_{-m} = (-1)^m J_m.
+inline void kt_piece_table(int segs, int K, double *out) {
+  long double L[KT_MAX_K + KT_PIECE_DEG + 1];
+  double J[KT_MAX_K + KT_PIECE_DEG + 1];
+  for (int q = 0; q < segs; ++q) {
+    kt_bessel_miller<long double>(q + 0.5, K + KT_PIECE_DEG + 1, L);
+    for (int k = 0; k <= K + KT_PIECE_DEG; ++k) J[k] = (double)L[k];
+    for (int k = 0; k < K; ++k) {
+      double scale = k == 0 ? 1 : 2;                    // over 2^n n!
+      for (int n = 0; n <= KT_PIECE_DEG; ++n) {
+        double c = 1, v = 0;                            // (-1)^i C(n, i)
+        for (int i = 0; i <= n; ++i) {
+          const int m = k - n + 2 * i;
+          v += c * (m >= 0 ? J[m] : (m & 1 ? -J[-m] : J[-m]));
+          c = -c * (n - i) / (i + 1);
+        }
+        out[((size_t)q * (KT_PIECE_DEG + 1) + n) * K + k] = scale * v;
+        scale /= 2 * (n + 1);
+      }
+    }
+  }
+}
+KT_HD double kt_piece_coef(const double *table, int segs, int K, int k, double r, double s) {
+  const int q0 = (int)(r * s), q = q0 < segs ? q0 : segs - 1;
+  const double x = fma(r, s, -(q + 0.5));
+  const double *t = table + (size_t)q * (KT_PIECE_DEG + 1) * K + k;
+  double v = t[KT_PIECE_DEG * K];
+  for (int n = KT_PIECE_DEG - 1; n >= 0; --n) v = fma(v, x, t[n * K]);
+  return v;
 }
 
 struct KtCplx { double re, im; };
@@ -118,8 +158,8 @@ struct KtGenImage {
   const KtCplx *pair_val;     // [P][n_loc*n_loc]
   const double *cheb_full;    // [sets][K] full-step coefficients lambda_s (2 - delta_k0) J_k(r dt)
   const KtCplx *phase_full;   // [sets] exp(-i c dt) / lambda_s
-  const double *piece;        // [n_piece][K] Chebyshev coefficients in u = s / dt of m_k(s), 0 <= s <= dt (pieces of an interval)
-  int n_piece;
+  const double *piece;        // [piece_segs][KT_PIECE_DEG + 1][K] coefficients of a piece of an interval (kt_piece_coef)
+  int piece_segs;
   int sets;                   // interval j takes set j % sets (a power of two)
   int quick_pulse;            // each node carries at most one control term and no control touches a diagonal
   const KtCplx *pair_coef;    // [P] coefficient of pair term p (value = coef * a^dag a entries)

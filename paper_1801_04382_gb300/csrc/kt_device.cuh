@@ -774,23 +774,16 @@ template <typename R> __device__ __forceinline__ typename C2<R>::T t_coef(int k,
 }
 
 // Coefficients of exp(-i G s) for every trajectory, s in sm.tsc[TS_X] (synchronised): m_k = (2 - delta_k0) J_k(r s) and the
-// phase exp(-i c s).  Called by the whole block, one thread per coefficient: its Chebyshev series in s / dt by Clenshaw's
-// recurrence.  (One thread running Miller's recurrence for all orders took longer than a series of a small problem in
-// FP64, where an instruction costs a warp 64 cycles however few of its lanes work: passes with several jumps per
-// trajectory at d = 81 28.5 -> 25.3 ms, d = 216 FP32 9.9 -> 8.3 ms, d = 729 FP32 26.9 -> 25.4 ms.)
+// phase exp(-i c s).  Called by the whole block, one thread per coefficient: a Taylor series of 16 terms.  (One thread
+// running Miller's recurrence for all orders took longer than a series of a small problem in FP64, where an
+// instruction costs a warp 64 cycles however few of its lanes work: passes with several jumps per trajectory at d = 81
+// 28.5 -> 25.3 ms, d = 216 FP32 9.9 -> 8.3 ms, d = 729 FP32 26.9 -> 25.4 ms.)
 template <typename R, bool TF>
 __device__ void piece_coefs(const KtGeom &g, const KtGenImage &im, const Smem &sm, double c_gen) {
   Coef<R, TF> *cf = (Coef<R, TF> *)sm.coef;
   for (int e = threadIdx.x; e < g.K * g.T; e += blockDim.x) {
     const int k = e / g.T;
-    const double y = 2.0 * (sm.tsc[TS_X * g.T + e % g.T] / g.dt) - 1.0, y2 = 2.0 * y;
-    double b1 = 0.0, b2 = 0.0;
-    for (int j = im.n_piece - 1; j >= 1; --j) {
-      const double b = fma(y2, b1, im.piece[j * g.K + k] - b2);
-      b2 = b1;
-      b1 = b;
-    }
-    const double m = fma(y, b1, im.piece[k] - b2);
+    const double m = kt_piece_coef(im.piece, im.piece_segs, g.K, k, g.r, sm.tsc[TS_X * g.T + e % g.T]);
     if constexpr (TF) {
       double sn, cs;
       sincos(-c_gen * sm.tsc[TS_X * g.T + e % g.T], &sn, &cs);

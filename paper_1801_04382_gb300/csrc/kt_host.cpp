@@ -1090,7 +1090,7 @@ struct HostImage {
   std::vector<int> dl, poff;
   std::vector<KtCplx> base, cslot, dg, cdg, pval, pc;
   std::vector<double> cf, piece;
-  int n_piece = 0;
+  int piece_segs = 0;
   std::vector<KtCplx> phase;
   int quick_pulse = 0;
   int pdst[KT_MAX_PAIRS], psrc[KT_MAX_PAIRS];
@@ -1659,30 +1659,9 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
 
   // ---- generator tables for both directions: B = -2i (G - c) / r
   const cd scale = cd(0.0, -2.0) / r;
-  // coefficients of a piece of an interval as Chebyshev series in u = s / dt: m_k(s) = (2 - delta_k0) J_k(r dt u) is entire, and
-  // its series ends about 25 terms after r dt / 2 (cut at 1e-18 of the largest value, 1)
-  const int n_node = std::min(256, 48 + (int)(r * dt));
-  std::vector<double> piece((size_t)n_node * K, 0.0);
-  {
-    std::vector<double> Ju(K), f((size_t)n_node * K);
-    for (int q = 0; q < n_node; ++q) {
-      const double th = M_PI * (q + 0.5) / n_node;
-      kt_bessel_miller(r * dt * 0.5 * (1.0 + std::cos(th)), K, Ju.data());
-      for (int k = 0; k < K; ++k) f[(size_t)q * K + k] = (k == 0 ? 1.0 : 2.0) * Ju[k];
-    }
-    for (int j = 0; j < n_node; ++j)
-      for (int q = 0; q < n_node; ++q) {
-        // cos(pi j (2 q + 1) / (2 n)), the angle reduced in whole numbers
-        const double w = std::cos(M_PI * ((long long)j * (2 * q + 1) % (4 * n_node)) / (2.0 * n_node)) * (j == 0 ? 1.0 : 2.0) / n_node;
-        for (int k = 0; k < K; ++k) piece[(size_t)j * K + k] += w * f[(size_t)q * K + k];
-      }
-  }
-  int n_piece = 2;
-  for (int j = 2; j < n_node; ++j)
-    for (int k = 0; k < K; ++k)
-      if (std::fabs(piece[(size_t)j * K + k]) > 1e-17) n_piece = j + 1;
-  n_piece = std::min(n_piece, 32 + (int)(0.75 * r * dt));   // what is left there is the transform's rounding
-  piece.resize((size_t)n_piece * K);
+  const int segs = kt_piece_segments(r * dt);
+  std::vector<double> piece((size_t)segs * (KT_PIECE_DEG + 1) * K);
+  kt_piece_table(segs, K, piece.data());
   auto build_image = [&](const Gen &gen, double cgen, HostImage &im) {
     const int nls = nl * g.S;
     im.dl.assign((size_t)N * nls, 0);
@@ -1774,7 +1753,7 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
       }
     }
     im.piece = piece;
-    im.n_piece = n_piece;
+    im.piece_segs = segs;
     const int sets = P.fp64 ? 1 : KT_COEF_SETS;
     im.cf.resize((size_t)sets * K);
     im.phase.resize(sets);
@@ -1866,7 +1845,7 @@ kt_status upload_image(kt_problem *p, const HostImage &h, KtGenImage &im, cudaSt
   im.sets = (int)h.phase.size();
   im.quick_pulse = h.quick_pulse;
   if ((t = upload(p, (double **)&im.piece, h.piece.data(), h.piece.size(), st)) != KT_OK) return t;
-  im.n_piece = h.n_piece;
+  im.piece_segs = h.piece_segs;
   for (int q = 0; q < 2 * KT_MAX_NL; ++q) im.kd64[q] = h.kd[q];
   for (int q = 0; q < KT_MAX_NL; ++q) {
     im.kd32[3 * q] = (float)h.kd[2 * q];
