@@ -1,67 +1,8 @@
 """Device memory of the gradient's set-up, on the host: the library runs in a child process against a stand-in for the
 CUDA runtime (host memory, kernels that do nothing) whose n-th allocation fails, or whose memory is small."""
-import os
-import shutil
-import subprocess
-import sys
-
 import pytest
 
-from paper_1801_04382_gb300 import build as pkg_build
-
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-
-FAKE = r"""
-#include <stdlib.h>
-#include <string.h>
-typedef int E; typedef void *P; typedef size_t Z;
-static int left = -1, made = 0, launches = 0;
-static Z total = (Z)8 << 30, used = 0;
-void fake_set_total(Z n) { total = n; }
-void fake_fail_in(int n) { left = n; }
-int fake_mallocs(void) { return made; }
-int fake_launches(void) { return launches; }
-E cudaMalloc(P *p, Z n)
-{
-  *p = 0;
-  if ((left > 0 && --left == 0) || used + n > total) return 2;
-  Z *h = calloc(1, n + 256);
-  if (!h) return 2;
-  ++made;
-  used += *h = n;
-  *p = (char *)h + 256;
-  return 0;
-}
-E cudaFree(P p) { if (p) { Z *h = (Z *)((char *)p - 256); used -= *h; free(h); } return 0; }
-E cudaMemcpy(P d, const void *s, Z n, int k) { (void)k; if (n && (!d || !s)) return 1; memcpy(d, s, n); return 0; }
-E cudaMemcpyAsync(P d, const void *s, Z n, int k, P st) { (void)st; return cudaMemcpy(d, s, n, k); }
-E cudaMemsetAsync(P d, int v, Z n, P st) { (void)st; if (n && !d) return 1; memset(d, v, n); return 0; }
-E cudaMemGetInfo(Z *f, Z *t) { *t = total; *f = total - used; return 0; }
-E cudaGetDevice(int *d) { *d = 0; return 0; }
-E cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
-E cudaGetLastError(void) { return 0; }
-const char *cudaGetErrorString(E e) { (void)e; return "stand-in"; }
-E cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
-E cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int b, Z s, unsigned g)
-{ (void)f; (void)b; (void)s; (void)g; *n = 1; return 0; }
-E cudaGetSymbolAddress(P *p, const void *s) { (void)s; static char mem[1 << 20]; *p = mem; return 0; }
-E cudaStreamSynchronize(P s) { (void)s; return 0; }
-E cudaStreamCreateWithFlags(P *s, unsigned f) { (void)f; *s = malloc(1); return 0; }
-E cudaStreamDestroy(P s) { free(s); return 0; }
-E cudaEventCreate(P *s) { *s = malloc(1); return 0; }
-E cudaEventCreateWithFlags(P *s, unsigned f) { (void)f; *s = malloc(1); return 0; }
-E cudaEventDestroy(P s) { free(s); return 0; }
-E cudaLaunchKernelExC(const void *c, const void *f, P *a) { (void)c; (void)f; (void)a; ++launches; return 0; }
-E __cudaLaunchKernel(void) { ++launches; return 0; }
-E __cudaGetKernel(P *k, const void *f) { *k = (P)f; return 0; }
-E __cudaPopCallConfiguration(void) { return 0; }
-E __cudaPushCallConfiguration(void) { return 0; }
-P *__cudaRegisterFatBinary(P f) { (void)f; static P h; return &h; }
-void __cudaRegisterFatBinaryEnd(P *h) { (void)h; }
-void __cudaRegisterFunction(void) {}
-void __cudaRegisterVar(void) {}
-void __cudaUnregisterFatBinary(P *h) { (void)h; }
-"""
+from fake_cudart import run_child
 
 CHILD = r"""
 import ctypes as ct, sys
@@ -142,20 +83,6 @@ states = (200 // 14 + 1 + 14 + 2) * M * 729 * 8      # kept every 14 intervals, 
 assert p.get_info().device_bytes - before >= states + terms, (p.get_info().device_bytes - before, states, terms)
 print("ok")
 """
-
-
-def run_child(tmp_path, code, *args):
-    if not shutil.which("gcc"):
-        pytest.skip("no C compiler")
-    if not os.path.exists(pkg_build.lib_path()):
-        pkg_build.build()
-    src, so = tmp_path / "fake_cudart.c", tmp_path / "libfake_cudart.so"
-    src.write_text(FAKE)
-    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-w", str(src), "-o", str(so)], check=True)
-    env = dict(os.environ, LD_PRELOAD=str(so), PYTHONPATH=ROOT)
-    res = subprocess.run([sys.executable, "-c", code, str(so), *[str(a) for a in args]], env=env,
-                         capture_output=True, text=True, timeout=300)
-    assert res.returncode == 0 and res.stdout.strip() == "ok", res.stdout + res.stderr
 
 
 @pytest.mark.parametrize("N,nc,precision,fallback", [(4, 2, "fp64", "refused"), (3, 2, "fp32", "strided")])
