@@ -169,8 +169,8 @@ typedef struct {
   int per_interval_launches; /* 0 = automatic: when the problem runs on the strided mapping or one element per thread, every tile
                                is resident on the GPU at once and every co-state is kept (small
                                problems), each sweep is one
-                               launch -- the backward sweep a plain one, the forward sweep a cooperative
-                               one whose CTAs exchange their partial sums after each interval to form the
+                               launch -- the backward and the guess sweep a plain one, the updating sweep a
+                               cooperative one whose CTAs exchange their partial sums after each interval to form the
                                update (Sec. 2.2: the update of interval j+1 needs every trajectory's
                                state at t_j); bit-identical to the per-interval launches.  Not used for
                                shards, the sweeps that keep states for the gradient, or the updating

@@ -3,7 +3,7 @@
 #include "kt_device.cuh"
 
 namespace kt {
-// a whole sweep (strided mapping only, the mapping of the small problems) runs one tile per CTA
+// a whole sweep (strided and row mapping, those of the small problems) runs one tile per CTA
 template <typename R, int EPT, int NL, int ACS, int MAXT>
 static cudaError_t launch_bwd_t(const KtGeom &g, const KtGenImage &im, const KtOps &ops, const BwdArgs &a, size_t smem,
                                 cudaStream_t st) {

@@ -1673,7 +1673,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
   // with g.fwd_grid > 0 the CTAs loop over tiles blockIdx.x, blockIdx.x + gridDim.x, ...: the tables and
   // the item mapping are built once, and the next tile's psi (fourth buffer, barriers [0] / [3] in turn)
   // and chi (third buffer) arrive by bulk copy while the current tile is propagated.
-  // SWEEP (a.sweep): one cooperative launch runs intervals a.j .. nt of one tile per CTA (see FwdArgs);
+  // SWEEP (a.sweep): one launch runs intervals a.j .. nt of one tile per CTA (see FwdArgs);
   // a compile-time switch, so that the per-interval kernels carry none of the sweep's state.
   constexpr bool sweep = SWEEP;
   const bool persist = !sweep && g.fwd_grid > 0;

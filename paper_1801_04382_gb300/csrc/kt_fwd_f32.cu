@@ -4,8 +4,8 @@
 
 namespace kt {
 // occ != nullptr: no launch, the kernel's resident CTAs per SM for this block and shared size.
-// a.sweep: a cooperative launch, one tile per CTA (all CTAs resident, as the exchange of the partials needs).
-// Whole-sweep kernels exist for the strided mapping only (the mapping of the small problems).
+// a.sweep: one tile per CTA; with the update a cooperative launch (all CTAs resident, as the exchange of the partials
+// needs).  Whole-sweep kernels exist for the strided and the row mapping (those of the small problems).
 template <typename R, int EPT, int NL, int ACS, int MAXT>
 static cudaError_t launch_fwd_t(const KtGeom &g, const KtGenImage &im, const KtOps &ops, const FwdArgs &a, size_t smem,
                                 cudaStream_t st, int *occ) {
@@ -26,7 +26,7 @@ static cudaError_t launch_fwd_t(const KtGeom &g, const KtGenImage &im, const KtO
       at[0].id = cudaLaunchAttributeCooperative;
       at[0].val.cooperative = 1;
       cfg.attrs = at;
-      cfg.numAttrs = 1;
+      cfg.numAttrs = a.overlap ? 1 : 0;
       return cudaLaunchKernelEx(&cfg, fwd_kernel<R, EPT, 0, ACS, true, MAXT>, g, im, ops, a);
     } else {
       if (occ) *occ = 0;

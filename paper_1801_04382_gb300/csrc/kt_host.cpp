@@ -670,7 +670,7 @@ kt_status enqueue_forward(kt_problem *p, int update, cudaStream_t st, bool save_
     return fail(KT_ERR_STATE, "a trajectory shard runs through its group (krotov_group_update) or over NCCL "
                               "(krotov_shard_nccl)");
   if ((update ? p->whole_sweep != 0 : p->whole_plain) && !save_psi) {
-    // the whole sweep as one cooperative launch: interval 0 (the update overlap at t_0) when
+    // the whole sweep as one launch (cooperative when updating): interval 0 (the update overlap at t_0) when
     // updating, then 1 .. nt, psi(t_j) in psi[j & 1] as on the per-interval path
     KT_CUDA(kt_launch_init_pass(p->g, p->U, p->pass, p->rstate, p->jcount[p->cur], st));
     FwdArgs a = fwd_args(p, update);

@@ -51,7 +51,7 @@ struct FwdArgs {
   KtCplx *tau;           // [M_pad] (j == nt)
   double *norm2;         // [M_pad] (j == nt)
   int *status;
-  // whole forward sweep in one cooperative launch (one tile per CTA, every CTA resident): intervals
+  // whole forward sweep in one launch (one tile per CTA; with the update cooperative, every CTA resident): intervals
   // j .. nt, the state kept in shared memory between them; psi(t_i) goes to psi_ring[i & 1] (the
   // input of interval 1 is psi_in), chi(t_i) is read from chi_slots + i * slot_bytes.  With the
   // update every CTA puts its partials of interval i into partials [nt][n_tiles][n_ctrl] (every bit set
