@@ -1541,9 +1541,10 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
   const bool row = N <= 3 && npair <= 3 && S <= 2 && (long long)d * std::max(1, cfg->tile_traj) <= row_max && (N <= 2 || d <= 256 || cfg->prec == KT_FP64) &&
                    (autom || cfg->items_per_thread == 1) &&
                    (ri || ri_classes(gf, gb, lo_val, ra_val, cols, false));
-  // density matrix of two nodes: the cluster kernel (real / imaginary classes, two slots per node row, at most six pair terms,
-  // one element per thread of at most eight CTAs)
-  const bool cluster = density && N == 4 && npair <= 6 && S <= 2 && d > 736 && d <= 8 * 832 && !cfg->inject_copy_timeout &&
+  // density matrix of two nodes, mapping automatic: the cluster kernel (real / imaginary classes, two slots per node row, at
+  // most six pair terms, one element per thread of at most eight CTAs)
+  const bool cluster = density && cfg->items_per_thread == 0 && N == 4 && npair <= 6 && S <= 2 && d > 736 && d <= 8 * 832 &&
+                       !cfg->inject_copy_timeout &&
                        (ri || ri_classes(gf, gb, lo_val, ra_val, cols, false));
   if (ri || row || cluster) S = 2;
   const bool small = few && autom;

@@ -40,7 +40,30 @@ assert rows and all(r[4] == 0 for r in rows), rows
 print("ok")
 """
 
+DENSITY = HEAD + r"""
+def density(items):
+    s = spec(2, 1, 4, 1, uniforms=np.full((1, 1, 1), -1.0))
+    keep, md, cfg = _descriptors(s["net"], s["T"], s["nt"], 1, s["eps_guess"], s["shape"], s["lam"], s["uniforms"],
+                                 items_per_thread=items)
+    lib, h = _capi.load(), ct.c_void_p()
+    assert lib.krotov_init_density(ct.byref(md), ct.byref(cfg), None, ct.byref(h)) == 0
+    info = _capi.Info()
+    assert lib.krotov_get_info(h, ct.byref(info)) == 0
+    rows = launched(lambda: lib.propagate_forward(h, 0, None, None))
+    lib.krotov_free(h)
+    return info, rows
 
-@pytest.mark.parametrize("code", [COOPERATIVE], ids=["cooperative"])
+
+info, rows = density(0)
+assert rows and all("density_kernel" in r[0] and r[5] == 4 for r in rows), rows
+for items in (4, 8):
+    info, rows = density(items)
+    assert info.items_per_thread == items
+    assert rows and all("fwd_kernelIdLi%dELi0" % items in r[0] for r in rows), rows
+print("ok")
+"""
+
+
+@pytest.mark.parametrize("code", [COOPERATIVE, DENSITY], ids=["cooperative", "density_items"])
 def test_routes(tmp_path, code):
     run_child(tmp_path, code)
