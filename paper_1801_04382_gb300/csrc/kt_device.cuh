@@ -873,8 +873,8 @@ __device__ __forceinline__ void sweep_tables(const KtGeom &g, const KtGenImage &
   }
 }
 
-// Full-step coefficients and phase of interval j: the kept set (in run, the copy of sm that the series takes: sm's own
-// places stay known to the jump phases), or loaded.
+// Full-step coefficients and phase of interval j: the kept set (in run, the copy of sm that the series takes: the jump
+// phases write their coefficients through sm, and must not write over the sets), or loaded.
 template <typename R>
 __device__ __forceinline__ void sweep_coefs(const KtGeom &g, const KtGenImage &im, const Smem &sm, Smem &run,
                                             const SweepKeep &kp, char *extra, int j) {
@@ -981,7 +981,7 @@ __device__ __forceinline__ R sqrt_n(int n) {
 // two FMAs each; the pulse-independent coefficients (last node's diagonal and cavity couplings,
 // pair coefficients, ladder values) are kernel-parameter or compile-time constants, so only the
 // drive couplings, the other nodes' pair tables and the states are read from shared memory.
-// CACHE: the other nodes' rows come from rc (registers) instead of the shared tables.
+// CACHE: the other nodes' rows come from rc (registers, the reverse gradient) instead of the shared tables.
 template <typename R, int NC, int TT, bool RI, bool CACHE, bool PREV, bool TF>
 __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im, const Smem &sm,
                                           const typename C2<R>::T *__restrict__ v,
@@ -1134,7 +1134,7 @@ __device__ __forceinline__ void apply_acs(const KtGeom &g, const KtGenImage &im,
   for (int q = 0; q < NL; ++q) out[q] = diag_done<TF>(diag(q), vk[q], PREV ? prev[base + q * T] : zero, out[q]);
 }
 
-template <typename R, int NC, int TT, bool RI, bool CACHE, bool TF, class IT>
+template <typename R, int NC, int TT, bool RI, bool TF, class IT>
 __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &sm, const IT &it,
                              int K, typename C2<R>::T (&acc)[3 * (NC + 1)]) {
   typedef typename C2<R>::T C;
@@ -1150,10 +1150,7 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
   const int last = g.n_nodes - 1;
   Diag<R> Df{(R)0, (R)0, (R)0};
   for (int i = 0; i < last; ++i) Df = add_diag(Df, load_diag<R, TF>(sm, i * NL + ((fdig >> (4 * i)) & 15)));
-  RowCache<R> rc;
-  if constexpr (RI && CACHE) {
-    if (ok) load_rows<R, NL>(g, sm, fdig, rc);
-  }
+  const RowCache<R> rc{};   // not read: the other nodes' rows come from the tables
   C vk[NL];
   const Coef<R, TF> c0 = cf[tau];
 #pragma unroll
@@ -1164,7 +1161,7 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
   if (K > 1) {
     C t[NL];
     if (ok) {
-      apply_acs<R, NC, TT, RI, CACHE, false, TF>(g, im, sm, A, A, base, fdig, Df, vk, t, rc);
+      apply_acs<R, NC, TT, RI, false, false, TF>(g, im, sm, A, A, base, fdig, Df, vk, t, rc);
       const Coef<R, TF> c1 = cf[T + tau];
 #pragma unroll
       for (int q = 0; q < NL; ++q) {
@@ -1180,7 +1177,7 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
       if (ok) {
         const Coef<R, TF> a = cf[k * T + tau];
         if constexpr (RI) keep_in_loop(Df);
-        apply_acs<R, NC, TT, RI, CACHE, true, TF>(g, im, sm, Q, P, base, fdig, Df, vk, t, rc);
+        apply_acs<R, NC, TT, RI, false, true, TF>(g, im, sm, Q, P, base, fdig, Df, vk, t, rc);
 #pragma unroll
         for (int q = 0; q < NL; ++q) {
           P[base + q * T] = t[q];
@@ -1574,7 +1571,7 @@ __device__ void cheb_run_row(const KtGeom &g, const KtGenImage &im, const Smem &
   apply_phase<R, 1>(g, sm, tau, acc, [&](int) { return D.lo; });
 }
 
-template <typename R, int EPT, int NL, int ACS, bool CACHE, class IT>
+template <typename R, int EPT, int NL, int ACS, class IT>
 __device__ __forceinline__ void cheb_dispatch(const KtGeom &g, const KtGenImage &im, const Smem &sm,
                                               const IT &it, int K, typename C2<R>::T (&acc)[EPT]) {
   // ACS: 1 cavity structure, 2 the same with T = 1, 3 with real / imaginary couplings, 4 both
@@ -1584,7 +1581,7 @@ __device__ __forceinline__ void cheb_dispatch(const KtGeom &g, const KtGenImage 
   if constexpr (A == 6) cheb_run_row<R, 2, 1>(g, im, sm, it, K, acc);
   else if constexpr (A == 7) cheb_run_row<R, 3, 3>(g, im, sm, it, K, acc);
   else if constexpr (A == 5) cheb_run_blk<R, NL / 3 - 1, TF>(g, im, sm, it, K, acc);
-  else if constexpr (A) cheb_run_acs<R, NL / 3 - 1, (A == 2 || A == 4) ? 1 : 0, (A >= 3), CACHE, TF>(g, im, sm, it, K, acc);
+  else if constexpr (A) cheb_run_acs<R, NL / 3 - 1, (A == 2 || A == 4) ? 1 : 0, (A >= 3), TF>(g, im, sm, it, K, acc);
   else if constexpr (NL > 0) cheb_run_fiber<R, NL, TF>(g, im, sm, it, K, acc);
   else cheb_run<R, EPT>(g, im, sm, it, K, acc);
 }
@@ -1737,7 +1734,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
     }
     if (j != a.j) {
       // sweep: the next interval.  Its pulse is in sm.eps (guess sweep: eps_old; updating: the value
-      // the barrier's finisher formed), its chi goes to the third buffer once every thread is done
+      // the exchange's finisher formed), its chi goes to the third buffer once every thread is done
       // with the previous one, and the tables are rebuilt for the new pulse.
       if (!a.update && threadIdx.x < g.n_ctrl) sm.eps[threadIdx.x] = eps_next;
       fence_proxy_async_smem();
@@ -1870,7 +1867,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) f
             piece_coefs<R, t_form<R, NL, ACS>()>(g, im, sm, g.c_fwd);
           }
           __syncthreads();
-          cheb_dispatch<R, EPT, NL, ACS, false>(g, im, run, it, g.K, acc);
+          cheb_dispatch<R, EPT, NL, ACS>(g, im, run, it, g.K, acc);
         }
         if (phase == PH_MAIN || phase == PH_DONE) {
           // ---- norm of the result and update overlap at t_j, g_c = sum_k Im <chi_k|hc_c|psi_k>, in one reduction.
@@ -2478,7 +2475,7 @@ __global__ void __launch_bounds__(MAXT, kt_min_ctas(sizeof(R), EPT, NL, MAXT)) b
             if (it.ok(q)) A[it.item(q)] = B[it.item(q)];
         }
         __syncthreads();
-        cheb_dispatch<R, EPT, NL, ACS, false>(g, im, run, it, g.K, acc);
+        cheb_dispatch<R, EPT, NL, ACS>(g, im, run, it, g.K, acc);
         if (rnd == rounds) break;
   #pragma unroll
         for (int q = 0; q < EPT; ++q)

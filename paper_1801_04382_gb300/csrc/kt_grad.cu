@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
       __syncthreads();
       piece_coefs<R, false>(g, imf, sm, g.c_fwd);
       __syncthreads();
-      cheb_run_acs<R, NC, 1, true, false, false>(g, imf, sm, it, g.K, acc);
+      cheb_run_acs<R, NC, 1, true, false>(g, imf, sm, it, g.K, acc);
       if (ok) {
 #pragma unroll
         for (int e = 0; e < NL; ++e) A[base + e] = acc[e];

@@ -1232,9 +1232,8 @@ bool ri_classes(const Gen &gf, const Gen &gb, const std::vector<cd> &lo_val, con
 
 // The block mapping (kt_device.cuh, apply_blk) on top of the real / imaginary classes: the middle node (the one
 // before the last) couples like the last one -- slot 0 (r, n-1) <-> (g, n), slot 1 (r, n) <-> (e, n), the drive at
-// every photon number or at none -- and one or two nodes lie outside.
+// every photon number or at none.
 bool block_structure(int N, int nl, const std::vector<std::vector<int>> &cols) {
-  if (N < 3 || N > 4) return false;
   const int NP = nl / 3, NC = NP - 1, m = N - 2;
   for (int x = 0; x < nl; ++x) {
     const int a = x / NP, n = x % NP, yr = cols[(size_t)m * nl + x][0], yi = cols[(size_t)m * nl + x][1];
@@ -2026,8 +2025,8 @@ kt_status create_problem(const kt_model_desc *md, const kt_config *cfg, const Ho
     p->n_chi_slots = n_ckpt_slots(nt, p->ckpt_dense, p->ckpt);
     TRY(dev_alloc(p, &p->chi, p->state_bytes * p->n_chi_slots));
     if (p->ckpt > 0) TRY(dev_alloc(p, &p->seg, p->state_bytes * (p->ckpt + 1)));
-    // whole-sweep launches: the strided mapping (the small problems' mapping; the sweep kernels are
-    // compiled for it only), every tile resident at once (the forward sweep's exchange of partials), every
+    // whole-sweep launches: the strided and the row mapping (those of the small problems; the sweep kernels are
+    // compiled for them only) or the cluster kernel, every tile resident at once (the forward sweep's exchange of partials), every
     // co-state kept (each interval's co-state has its slot), no exchange with other shards; the
     // cross-trajectory rule's updating sweep keeps one launch per interval, for the pair sums in between
     int dev = 0, sms = 0, per = 0;
