@@ -151,6 +151,25 @@ __device__ __forceinline__ void grad_finish(const KtGeom &g, const Smem &sm, con
   if (threadIdx.x == 0) *a.counter = 0u;
 }
 
+// A sum over the terms and pieces of an interval.  FP32: in two floats (Knuth's two-sum), the rounding errors of the first
+// collected in the second -- seven FP32 additions where one to FP64 would take a warp 128 cycles; what is added at a
+// time is a sum over at most nine elements.
+template <typename R> struct Wide;
+template <> struct Wide<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double x) { s += x; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct Wide<float> {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = s + x, z = t - s;
+    e += (s - (t - z)) + (x - z);
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
 // One step of the reverse series on the thread's fiber (tile width 1): out[q] = h (B^dag b)[q] + add[q], b's own values
 // in bk, add[q] = m W[q] + prev[base + q]; and dot[i] += h sum_q Re(conj(b at the drive neighbour of node i) y[q]) for the
 // outer nodes, dl[.] the same for the last node, one slot per e_n and r_n row.
@@ -159,8 +178,8 @@ __device__ __forceinline__ void adj_step(const KtGeom &g, const KtGenImage &im, 
                                          const typename C2<R>::T *__restrict__ v, const typename C2<R>::T *prev, int base,
                                          uint32_t fdig, Diag<R> Df, const RowCache<R> &rc, R h, R m,
                                          const typename C2<R>::T (&w)[3 * (NC + 1)], typename C2<R>::T (&bk)[3 * (NC + 1)],
-                                         const typename C2<R>::T *__restrict__ ysrc, int ystride, R (&dot)[3],
-                                         R (&dl)[2 * (NC + 1)]) {
+                                         const typename C2<R>::T *__restrict__ ysrc, int ystride, Wide<R> (&dot)[3],
+                                         Wide<R> (&dl)[2 * (NC + 1)]) {
   typedef typename C2<R>::T C;
   constexpr int NP = NC + 1, NL = 3 * NP;
   const C *pv = (const C *)sm.pair_val;
@@ -185,8 +204,8 @@ __device__ __forceinline__ void adj_step(const KtGeom &g, const KtGenImage &im, 
     const int qr = 2 * NP + n, qe = NP + n;
     out[qr] = rfma(ld[qr * NL + qe].x, bk[qe], out[qr]);
     out[qe] = rfma(ld[qe * NL + qr].x, bk[qr], out[qe]);
-    dl[n] = fma(h, bk[qr].x * y[qe].x + bk[qr].y * y[qe].y, dl[n]);               // row e_n, neighbour r_n
-    dl[NP + n] = fma(h, bk[qe].x * y[qr].x + bk[qe].y * y[qr].y, dl[NP + n]);     // row r_n, neighbour e_n
+    dl[n].add(h * fma(bk[qr].y, y[qe].y, bk[qr].x * y[qe].x));             // row e_n, neighbour r_n
+    dl[NP + n].add(h * fma(bk[qe].y, y[qr].y, bk[qe].x * y[qr].x));        // row r_n, neighbour e_n
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -203,7 +222,7 @@ __device__ __forceinline__ void adj_step(const KtGeom &g, const KtGenImage &im, 
         s = fma(x.x, y[q].x, s);
         s = fma(x.y, y[q].y, s);
       }
-      dot[i] = fma(h, s, dot[i]);
+      dot[i].add(h * s);
     }
   }
   for (int p = 0; p < g.n_pairs; ++p) {
@@ -286,9 +305,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
   const int ys = blockDim.x;
   auto sb = [&](int p) -> double { return p == 0 ? 0.0 : (p > m ? g.dt : a.rec_s[rb + sm.tin[TI_J0 + p - 1]]); };
   const R *cf = (const R *)sm.coef;
-  R dot[3] = {(R)0, (R)0, (R)0}, dl[2 * NP];
-#pragma unroll
-  for (int q = 0; q < 2 * NP; ++q) dl[q] = (R)0;
+  Wide<R> dot[3], dl[2 * NP];
   C w[NL];   // the co-state at the end of the current piece
 #pragma unroll
   for (int q = 0; q < NL; ++q) w[q] = ok ? chi[(size_t)(base + q) * T_layout] : mkc((R)0, (R)0);
@@ -446,12 +463,12 @@ __global__ void __launch_bounds__(MAXT, MAXT == 96 && sizeof(R) == 4 ? 5 : 1)
     const KtCplx *slot = imb.ctrl_slot + (size_t)c * nls;
     if (node == last) {
 #pragma unroll
-      for (int e = 0; e < 2 * NP; ++e) part[c] += (double)(R)slot[(NP + e) * g.S + 1].re * (double)dl[e];
+      for (int e = 0; e < 2 * NP; ++e) part[c] += (double)(R)slot[(NP + e) * g.S + 1].re * dl[e].value();
     } else {
-      R d = dot[0];
-      if (node == 1) d = dot[1];
-      if (node == 2) d = dot[2];
-      part[c] = (double)(R)slot[((fdig >> (4 * node)) & 15) * g.S + 1].re * (double)d;
+      double d = dot[0].value();
+      if (node == 1) d = dot[1].value();
+      if (node == 2) d = dot[2].value();
+      part[c] = (double)(R)slot[((fdig >> (4 * node)) & 15) * g.S + 1].re * d;
     }
   }
   grad_finish(g, sm, a, part);
