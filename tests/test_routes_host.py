@@ -17,7 +17,7 @@ def launched(fn):
     fake.fake_log_clear()
     fn()
     rows = [ln.split() for ln in fake.fake_log().decode().splitlines()]
-    return [(r[0], *map(int, r[1:])) for r in rows if any(k in r[0] for k in ("fwd_kernel", "bwd_kernel", "density_kernel", "grad_"))]
+    return [(r[0], *map(int, r[1:])) for r in rows if any(k in r[0] for k in ("fwd_kernel", "bwd_kernel", "density_kernel", "grad_kernel", "grad_adj_kernel"))]
 
 
 def spec(n, nc, nt, M, **more):
@@ -64,6 +64,63 @@ print("ok")
 """
 
 
-@pytest.mark.parametrize("code", [COOPERATIVE, DENSITY], ids=["cooperative", "density_items"])
+KERNELS = HEAD + r"""
+import cmath
+
+
+def kernel(net, nt, M, how="forward", **more):
+    s = spec(net.n_nodes, 1, nt, M, net=net, **more)
+    with Problem(**s) as p:
+        if how == "forward":
+            rows = launched(lambda: p.forward())
+        elif how == "kept":
+            rows = launched(lambda: p.forward(keep_for_gradient=True))
+        else:
+            p.forward(keep_for_gradient=True)
+            out = np.zeros((net.n_nodes, nt))
+            rows = launched(lambda: p._lib.krotov_gradient(p._h, None, out.ctypes.data_as(ct.c_void_p), None))
+    assert rows, how
+    names = {r[0].split("EEEv")[0].replace("_ZN2kt", "").lstrip("0123456789") for r in rows}
+    assert len(names) == 1 or how == "gradient", names
+    return names if how == "gradient" else names.pop()
+
+
+def plain(N, nc):
+    net = cascaded_chain(N, nc)
+    x = np.zeros((net.n_loc, net.n_loc), dtype=complex)
+    x[0, nc + 1] = x[nc + 1, 0] = 0.4
+    net.h0_local = net.h0_local + x
+    return net
+
+
+def phase(N, nc):
+    return cascaded_chain(N, nc, g=cmath.exp(0.2j * cmath.pi))
+
+
+T = {"fp32": "f", "fp64": "d"}
+for prec in ("fp32", "fp64"):
+    t = T[prec]
+    # fibers: plain, complex cavity structure (tile width 1 compiled in for n_loc = 9), real / imaginary
+    assert kernel(plain(2, 1), 4, 5, tile_traj=2, precision=prec).startswith(f"fwd_kernelI{t}Li6ELi6ELi0ELb0")
+    assert kernel(plain(2, 2), 4, 5, tile_traj=1, precision=prec).startswith(f"fwd_kernelI{t}Li9ELi9ELi0ELb0")
+    assert kernel(phase(2, 1), 4, 5, tile_traj=1, precision=prec).startswith(f"fwd_kernelI{t}Li6ELi6ELi1ELb0")
+    assert kernel(phase(2, 2), 4, 5, tile_traj=2, precision=prec).startswith(f"fwd_kernelI{t}Li9ELi9ELi1ELb0")
+    assert kernel(phase(2, 2), 4, 5, tile_traj=1, precision=prec).startswith(f"fwd_kernelI{t}Li9ELi9ELi2ELb0")
+    assert kernel(cascaded_chain(3, 1), 4, 5, tile_traj=2, precision=prec).startswith(f"fwd_kernelI{t}Li6ELi6ELi3ELb0")
+    # gradient: strided where the couplings are complex, reverse where they are not
+    assert any(k.startswith(f"grad_kernelI{t}Li4") for k in kernel(phase(2, 1), 4, 3, "gradient", precision=prec))
+    assert all(k.startswith(f"grad_adj_kernelI{t}Li2") for k in kernel(cascaded_chain(3, 2), 4, 3, "gradient", precision=prec))
+# FP32 fibers and blocks: the T form; sweeps that keep states for the gradient: the y form (codes 8 higher)
+assert kernel(cascaded_chain(3, 2), 4, 5, precision="fp32").startswith("fwd_kernelIfLi9ELi9ELi4ELb0")
+assert kernel(cascaded_chain(3, 2), 4, 5, "kept", precision="fp32").startswith("fwd_kernelIfLi9ELi9ELi12ELb0")
+assert kernel(cascaded_chain(4, 1), 4, 5, precision="fp32").startswith("fwd_kernelIfLi12ELi6ELi5ELb0")
+assert kernel(cascaded_chain(4, 1), 4, 5, "kept", precision="fp32").startswith("fwd_kernelIfLi12ELi6ELi13ELb0")
+assert kernel(cascaded_chain(3, 2), 4, 5, precision="fp64").startswith("fwd_kernelIdLi1ELi0ELi7ELb0")
+assert all(k.startswith("grad_adj_kernelIdLi2ELi736") for k in kernel(cascaded_chain(4, 2), 3, 2, "gradient", precision="fp64"))
+print("ok")
+"""
+
+
+@pytest.mark.parametrize("code", [COOPERATIVE, DENSITY, KERNELS], ids=["cooperative", "density_items", "kernels"])
 def test_routes(tmp_path, code):
     run_child(tmp_path, code)
