@@ -71,7 +71,7 @@ PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # this workload's launch size (1024 trajectories, d = 6561, FP32-mixed), from one ncu capture of the
 # current kernels (`bench.py --workload profile`, full section set: an updating forward launch and a
 # backward launch); None where no capture of the current kernel exists.
-NCU_TRAFFIC_PER_LAUNCH = {"bwd": 53903872 + 4008704, "fwd": 107751680 + 16918016}
+NCU_TRAFFIC_PER_LAUNCH = {"bwd": 53896448 + 4053760, "fwd": 107888384 + 19765248}
 FP32_LANES = 128              # FP32 FMA lanes per SM (Blackwell)
 
 
@@ -85,12 +85,13 @@ def fp32_peak_tflops(clk_mhz: float) -> float:
     return sm_count() * FP32_LANES * 2 * clk_mhz * 1e6 / 1e12
 
 
-def executed_flops_per_elem_term(nnz: float, ri: bool) -> float:
+def executed_flops_per_elem_term(nnz: float, ri: bool, t_form: bool = False) -> float:
     """FP32 flops one element of one Chebyshev term executes: every off-diagonal coupling of the
     cavity network is purely real or purely imaginary, so the kernels apply it with two FMAs
     (4 flops) instead of a complex multiply-add (8); the diagonal takes 8 (the sum of its node parts 2, real
-    part 2, imaginary part 4), the term before last 2 and the running sum with real coefficients 4."""
-    return (4.0 if ri else 8.0) * (nnz - 1.0) + 8.0 + 2.0 + 4.0
+    part 2, imaginary part 4), the term before last 2 and the running sum with real coefficients 4, with complex ones
+    (``t_form``: FP32 fibers and blocks) 8."""
+    return (4.0 if ri else 8.0) * (nnz - 1.0) + 8.0 + 2.0 + (8.0 if t_form else 4.0)
 
 
 def measured_peaks():
@@ -735,7 +736,8 @@ def run_ours(args, rank, world):
     nnz = avg_row_nonzeros(net)
     K = info.cheb_terms
     ri = info.threads > 0 and wl.n_cav == 2      # cavity network with real / imaginary coupling classes
-    exec_per_elem_term = executed_flops_per_elem_term(nnz, ri)
+    t_form = wl.precision == "fp32" and wl.d > 256 and info.items_per_thread == 0
+    exec_per_elem_term = executed_flops_per_elem_term(nnz, ri, t_form)
     survey_per_elem_term = 8.0 * nnz + 12.0      # every coupling counted as a complex multiply-add
     flops_per_launch = exec_per_elem_term * K * wl.d * M_rank
     clk_max = (clocks or {}).get("sm_max_mhz") or peaks.get("sm_max_mhz", 2070.0)

@@ -1205,7 +1205,7 @@ __device__ void cheb_run_acs(const KtGeom &g, const KtGenImage &im, const Smem &
 // and branches per fiber, with 23 warps of 80 registers to hide them.  Here a neighbour's block serves the
 // hops onto the middle and onto the last node at once, a hop between those two stays in registers, and every
 // offset and coefficient is shared by 27 elements, with 8 warps of 255 registers whose 27 independent
-// rows cover the latency.  1024 trajectories of d = 6561, per interval: forward with update 381 -> 352 us, backward 313 -> 286 us.
+// rows cover the latency.  1024 trajectories of d = 6561, per interval: forward with update 370 -> 345 us, backward 313 -> 294 us.
 template <typename R, int NP>
 struct BlkCache {
   int off0[2], off1[2];   // outer nodes: element offsets of the two slots (0 = none)

@@ -24,8 +24,8 @@
 // backward interval kernel is not launched.  B_i has the drive's entries only: its bilinear forms take the neighbour
 // values that B^dag loads anyway.  The z_k of a thread's own fiber wait in global memory (K states; written and
 // read back once, coalesced, mostly in L2).  Per interval, gradient, backward and replay launches of before together against
-// this one: d = 729, 1024 trajectories, three controls, FP32 572 -> 175 us; d = 6561, 64 trajectories 2084 -> 159 us; d = 216,
-// 200 trajectories 362 -> 50 us; d = 81, 100 trajectories, FP64 693 -> 380 us.
+// this one: d = 729, 1024 trajectories, three controls, FP32 572 -> 189 us; d = 6561, 64 trajectories 2084 -> 182 us; d = 216,
+// 200 trajectories 362 -> 50 us; d = 81, 100 trajectories, FP64 693 -> 382 us.
 //
 // One CTA per trajectory, gathered from the problem's interleaved tile layout.
 #include "kt_device.cuh"
@@ -153,7 +153,8 @@ __device__ __forceinline__ void grad_finish(const KtGeom &g, const Smem &sm, con
 
 // A sum over the terms and pieces of an interval.  FP32: in two floats (Knuth's two-sum), the rounding errors of the first
 // collected in the second -- seven FP32 additions where one to FP64 would take a warp 128 cycles; what is added at a
-// time is a sum over at most nine elements.
+// time is a sum over at most nine elements.  Against sums in single floats: d = 729, 1024 trajectories 183 -> 189 us, d = 6561, 64
+// trajectories 160 -> 182 us (80 registers).
 template <typename R> struct Wide;
 template <> struct Wide<double> {
   double s = 0.0;
