@@ -1646,7 +1646,9 @@ kt_status plan(const kt_model_desc *md, const kt_config *cfg, HostPlan &P, bool 
     if (g.prefetch_chi && cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
       const int slots = std::max(1, std::min(2048 / g.nthreads, 65536 / (regs * g.nthreads)));
-      const int per_sm = std::max(1, std::min((int)((227 * 1024) / smem3), slots));
+      // the backward kernel of n_loc = 6 fibers takes 72 registers in CTAs of more than 256 threads: two of 448 fit an SM
+      const int slots_b = P.ept == -306 && !P.fp64 && g.nthreads > 256 ? std::max(1, 65536 / (72 * g.nthreads)) : slots;
+      const int per_sm = std::max(1, std::min((int)((227 * 1024) / smem3), slots_b));
       if (g.n_tiles > sms * per_sm) g.bwd_grid = sms * per_sm;
       // forward kernel: the same tile loop when a fourth buffer (the next tile's psi) fits as well
       const size_t smem4 = kt_smem_bytes(g, esz, true, true);

@@ -110,6 +110,10 @@ for prec in ("fp32", "fp64"):
     # gradient: strided where the couplings are complex, reverse where they are not
     assert any(k.startswith(f"grad_kernelI{t}Li4") for k in kernel(phase(2, 1), 4, 3, "gradient", precision=prec))
     assert all(k.startswith(f"grad_adj_kernelI{t}Li2") for k in kernel(cascaded_chain(3, 2), 4, 3, "gradient", precision=prec))
+# tile loops: two CTAs of 448 threads per SM where the kernel's 72 registers leave room for them
+with Problem(**spec(4, 1, 3, 1024, precision="fp32")) as p:
+    p.forward()
+    assert all(r[1:3] == (304, 448) for r in launched(lambda: p.backward()))
 # FP32 fibers and blocks: the T form; sweeps that keep states for the gradient: the y form (codes 8 higher)
 assert kernel(cascaded_chain(3, 2), 4, 5, precision="fp32").startswith("fwd_kernelIfLi9ELi9ELi4ELb0")
 assert kernel(cascaded_chain(3, 2), 4, 5, "kept", precision="fp32").startswith("fwd_kernelIfLi9ELi9ELi12ELb0")
